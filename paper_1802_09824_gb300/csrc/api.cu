@@ -59,6 +59,7 @@ void pm_free(ph_pm *h);
 int pm_status(const ph_pm *h);
 void sim_free(ph_sim *h);
 void fit_factor_poly(double U, int deg, float *coef);
+void fit_inverse_form(BoxDev &bx, double G, double rcut, double rs);
 
 static thread_local char g_err[512] = "";
 static std::atomic<long long> g_launches{0};
@@ -185,6 +186,27 @@ int poly_degree_for(double U)
     return -1;
 }
 
+// The inverse-distance form holds for U = rcut / 2R_s up to 2.3 and a softening
+// up to 2R_s / 64 (fit_inverse_form: its error there is at most 1.2e-7 of the
+// Newtonian term, below that of the general form, 3.5e-7).  A larger U would
+// subtract nearly equal terms at large r, a larger softening needs more terms
+// of its expansion: those boxes take the general form.
+bool inverse_form_ok(const ph_params &p)
+{
+    return p.rcut <= 2.0 * p.rs * 2.3 && p.eps <= 2.0 * p.rs / 64.0;
+}
+
+int exact_degree_for(const ph_params *p, int n_boxes)
+{
+    bool inv = true;
+    int deg = 10;
+    for (int b = 0; b < n_boxes; b++) {
+        inv = inv && inverse_form_ok(p[b]);
+        deg = std::max(deg, poly_degree_for(p[b].rcut / (2.0 * p[b].rs)));
+    }
+    return inv ? kInvDeg : deg;
+}
+
 static int check_params(const ph_params &p, int b)
 {
     if (!(std::isfinite(p.L) && p.L > 0)) return fail(PH_ERR_ARG, "box %d: L must be finite and > 0", b);
@@ -233,7 +255,11 @@ void fill_box(BoxDev &bx, const ph_params &p, int key_bits, int poly_degree, int
     bx.first = first;
     bx.n = (int32_t)n_box;
     bx.group_size = group_size;
-    fit_factor_poly(p.rcut / (2.0 * p.rs), poly_degree, bx.poly);
+    bx.sc = 1.f;   // the general form keeps the box's own lengths
+    if (poly_degree == kInvDeg)
+        fit_inverse_form(bx, p.G, p.rcut, p.rs);
+    else
+        fit_factor_poly(p.rcut / (2.0 * p.rs), poly_degree, bx.poly);
 }
 
 int check_built(const ph_leaves *lv, const ph_pairs *pr)
@@ -351,11 +377,7 @@ static int leaves_common(const void *pos, int pos_type, const float *mass, const
     h->pp_variant = params[0].pp_variant;
     h->queue_order = params[0].queue_order;
     h->boxes_host.resize(nb);
-    int deg = 10;
-    for (int b = 0; b < nb; b++) {
-        int d = poly_degree_for(params[b].rcut / (2.0 * params[b].rs));
-        if (d > deg) deg = d;
-    }
+    const int deg = exact_degree_for(params, nb);
     h->poly_degree = deg;
     int cells = 0;
     std::vector<int32_t> bf(nb + 1);

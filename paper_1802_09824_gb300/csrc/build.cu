@@ -518,6 +518,80 @@ void fit_factor_poly(double U, int deg, float *coef)
     for (int k = 0; k <= kMaxPoly; k++) coef[k] = k < n ? (float)m[k] : 0.f;
 }
 
+// (1 - f)/u^3 as a function of v = u^2, u = r / 2R_s: entire, since
+// 1 - f = erf(u) - (2u/sqrt(pi)) exp(-u^2) = (4/sqrt(pi)) sum (-1)^n u^(2n+3) / (n! (2n+3)).
+static double one_minus_f_over_u3(double v)
+{
+    if (v < 1.0) {
+        double term = 1.0, s = 0.0;
+        for (int n = 0; n < 24; n++) {
+            s += term / (2 * n + 3);
+            term *= -v / (n + 1);
+        }
+        return 4.0 / std::sqrt(M_PI) * s;
+    }
+    const double u = std::sqrt(v);
+    return (std::erf(u) - 2.0 * u / std::sqrt(M_PI) * std::exp(-v)) / (u * v);
+}
+
+// The exact kernel's inverse-distance form of the softened short-range weight
+// W = f(r) (r^2 + eps^2)^(-3/2).  In units of 2R_s, with v = r^2, e = eps^2,
+// x = v + e: W = x^(-3/2) - (1 - e/x)^(3/2) E(v), E(v) = (1 - f)/v^(3/2)
+// entire.  (1 - e/x)^(3/2) = 1 - 1.5 e/x + kappa (e/x)^2 up to its third
+// order, so the second term is b1/x + b2/x^2 (the singular parts of E times
+// that expansion) plus a function smooth in x, interpolated by a degree-9
+// polynomial P in x at the zeros of the weighted minimax error curve for
+// U = 2.25 (weight x^(3/2): the error in units of the Newtonian term), scaled
+// to [0, U^2].  kappa = 0.46 instead of the Taylor 0.375 evens the rest out
+// over r ~ eps.  Error in those units: 8e-8 at U = 2.25, 1.2e-7 at U = 2.3,
+// and 1.1e-7 at r < eps for eps = 2R_s / 64 (the form it replaced: 3.5e-7
+// from its degree-10 polynomial and ex2).
+// The kernel evaluates (1 - k) W = Y (y (x Y - k) + b1' + b2' Y) + P', with
+// y = rsqrt(x), Y = y^2 and k = 5/3: (x Y - k) / (1 - k) = 1 + 1.5 (1 - x Y)
+// corrects the three-fold error of an SFU rsqrt in y^3 to second order.  k is
+// the FP32 number nearest 5/3 and 1 - k is taken of that number, so its
+// rounding leaves no bias in the Newtonian term (6e-8 with an exact -2/3).
+void fit_inverse_form(BoxDev &bx, double G, double rcut, double rs)
+{
+    constexpr int n = kInvDeg + 1;
+    static const double node[n] = {0.05768249, 0.14244654, 0.25282438, 0.38132087, 0.51875132,
+                                   0.65494475, 0.77953489, 0.88282818, 0.95665679, 0.99511833};
+    const double kappa = 0.46;
+    const double s2 = bx.s2, unit = 4.0 * rs * rs * s2;   // scaled x = unit * (x in units of 2R_s)
+    const double e = (double)bx.eps2s / unit;
+    const double V = rcut * rcut / (4.0 * rs * rs);
+    const double E0 = 4.0 / (3.0 * std::sqrt(M_PI)), E1 = -0.6 * E0, E2 = 3.0 / 14.0 * E0;
+    const double a0 = E0 - E1 * e + E2 * e * e, a1 = E1 - 2.0 * E2 * e;   // E(x - e) = a0 + a1 x + ...
+    const double b1 = -1.5 * e * a0 + kappa * e * e * a1, b2 = kappa * e * e * a0;
+    // Newton's divided differences in t = (x - zc) / (V / 2), zc = e + V / 2,
+    // expanded to monomials
+    double t[n], d[n], m[n] = {0};
+    for (int k = 0; k < n; k++) {
+        const double v = node[k] * V, x = v + e;
+        t[k] = 2.0 * node[k] - 1.0;
+        d[k] = std::pow(1.0 - e / x, 1.5) * one_minus_f_over_u3(v) - b1 / x - b2 / (x * x);
+    }
+    for (int j = 1; j < n; j++)
+        for (int k = n - 1; k >= j; k--) d[k] = (d[k] - d[k - 1]) / (t[k] - t[k - j]);
+    for (int k = n - 1; k >= 0; k--) {
+        for (int j = n - 1; j > 0; j--) m[j] = m[j - 1] - t[k] * m[j];
+        m[0] = d[k] - t[k] * m[0];
+    }
+    const double su = std::sqrt(unit);
+    const double mk = (double)kInvK - 1.0;
+    double scale = mk / (unit * su);
+    for (int k = 0; k < n; k++) {
+        bx.inv_poly[k] = (float)(m[k] * scale);
+        scale *= 2.0 / (V * unit);
+    }
+    bx.inv_b1 = (float)(b1 * mk / su);
+    bx.inv_b2 = (float)(b2 * mk * su);
+    bx.inv_zc = (float)(-(e + 0.5 * V) * unit);
+    bx.inv_cut = (float)(rcut * rcut * s2 + (double)bx.eps2s);
+    bx.sc = (float)std::sqrt(s2);
+    bx.inv_g = (float)(-G * s2 / mk);
+}
+
 // Enqueue the whole leaf/group build for the particles already in device
 // memory (pos, mass).  The handle's box table and buffers are set up.
 int build_leaves_device(ph_leaves *h, const void *pos, int pos_type, const float *mass, cudaStream_t s)

@@ -14,9 +14,11 @@
 //
 // Per pair (Eq. (split), Plummer factor, hard cutoff):
 //   r2 = |d|^2,  w = m_j f(r) / (r2 + eps^2)^{3/2}  if r2 < rcut^2 else 0
-//   f(r) = 2^(r2 c_e) h(t),  t = r / (R_s U) - 1,  h a degree-NPOLY polynomial
-// with rsqrt (plus one Newton correction), sqrt and ex2 on the SFU.  Partial
-// sums over runs of 16 sources are added to the total with Kahan compensation.
+// in one of two forms: the inverse-distance form, the Newtonian term minus a
+// polynomial in r2 + eps^2 (one SFU rsqrt; see interact2), or, for boxes
+// outside its range, f(r) = 2^(r2 c_e) h(t), t = 2r / rcut - 1, h a
+// degree-NPOLY polynomial, with rsqrt, sqrt and ex2 on the SFU.  Partial sums
+// over runs of 16 sources are added to the total with Kahan compensation.
 #include <cstring>
 
 #include "factor.cuh"
@@ -48,7 +50,9 @@ constexpr int kJBuf = 256;      // staged sources per warp (even)
 struct PairConsts {
     f2_t poly[kMaxPoly + 1];
     f2_t s2, eps2s, c_t, c_e, m1;
-    float rcut2, rfilt2;
+    float rcut2, rfilt2;   // scaled by sc^2 in the inverse-distance form
+    f2_t zc, b1, b2, m53;  // inverse-distance form (poly holds its polynomial)
+    float sc;              // length scale of the staged sources (1 in the general form)
 };
 
 struct PPArgs {
@@ -84,8 +88,34 @@ struct PPArgs {
     const float2 *table;
     float tab_scale2;                // (kTabN / rcut)^2
     int64_t n_pos;                   // rows of pos_leaf (bounds checks)
+    bool inverse;                    // the exact kernel runs the inverse-distance form (count kernel)
     const int32_t *order;            // queue slot -> group (groups by decreasing cost), or NULL
 };
+
+// The constants of a group's box (boxes with different constants).
+template <int NPOLY>
+__device__ __forceinline__ void box_consts(const BoxDev &bx, PairConsts &c)
+{
+    constexpr bool inv = NPOLY == kInvDeg;
+    const float *p = inv ? bx.inv_poly : bx.poly;
+#pragma unroll
+    for (int q = 0; q <= NPOLY; q++) c.poly[q] = pk(p[q], p[q]);
+    c.eps2s = pk(bx.eps2s, bx.eps2s);
+    c.rcut2 = inv ? bx.inv_cut : bx.rcut2;
+    c.rfilt2 = inv ? bx.rfilt2 * bx.s2 : bx.rfilt2;
+    c.sc = inv ? bx.sc : 1.f;
+    if (inv) {
+        c.zc = pk(bx.inv_zc, bx.inv_zc);
+        c.b1 = pk(bx.inv_b1, bx.inv_b1);
+        c.b2 = pk(bx.inv_b2, bx.inv_b2);
+        c.m53 = pk(-kInvK, -kInvK);
+    } else {
+        c.s2 = pk(bx.s2, bx.s2);
+        c.c_t = pk(bx.c_t, bx.c_t);
+        c.c_e = pk(bx.c_e, bx.c_e);
+        c.m1 = pk(-1.f, -1.f);
+    }
+}
 
 struct Kahan3 {
     float sx = 0.f, sy = 0.f, sz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
@@ -100,11 +130,39 @@ struct Kahan3 {
 
 // Two sources (A = x0 x1 y0 y1, B = z0 z1 m0 m1) against one target: add
 // m_j f(r) d / (r^2 + eps^2)^{3/2} into the pair accumulators.
+//
+// NPOLY = kInvDeg is the inverse-distance form (fit_inverse_form; lengths
+// scaled by sc): 25 packed FP32 instructions and one SFU operation per pair,
+// where the general form (NPOLY = 10 and up) takes 27 and three.  Bound by
+// the FMA pipe (ncu: 80 % busy): a loop over staged pairs alone took 66.2
+// cycles per two pairs and warp, 69.3 with the general form.  2-norm of the
+// force error against FP64 sums: 1.1e-7 of the forces' on uniform boxes
+// (general form 1.6e-7), 4.3e-8 on halo mixtures (9.0e-8).
 template <int NPOLY>
 __device__ __forceinline__ void interact2(const float4 a, const float4 b, const f2_t xi, const f2_t yi, const f2_t zi,
                                           const PairConsts &c, f2_t &px, f2_t &py, f2_t &pz)
 {
     const f2_t dx = sub2(pk(a.x, a.y), xi), dy = sub2(pk(a.z, a.w), yi), dz = sub2(pk(b.x, b.y), zi);
+    if (NPOLY == kInvDeg) {
+        f2_t x = fma2(dx, dx, c.eps2s);
+        x = fma2(dy, dy, x);
+        x = fma2(dz, dz, x);
+        const f2_t y = pk(rsqrt_sfu(lo_of(x)), rsqrt_sfu(hi_of(x)));
+        const f2_t Y = mul2(y, y);
+        const f2_t z = add2(x, c.zc);
+        f2_t h = c.poly[kInvDeg];
+#pragma unroll
+        for (int q = kInvDeg - 1; q >= 0; q--) h = fma2(h, z, c.poly[q]);
+        const f2_t q = fma2(fma2(x, Y, c.m53), y, fma2(c.b2, Y, c.b1));
+        const f2_t w = mul2(pk(b.z, b.w), fma2(q, Y, h));
+        const float w0 = lo_of(x) < c.rcut2 ? lo_of(w) : 0.f;
+        const float w1 = hi_of(x) < c.rcut2 ? hi_of(w) : 0.f;
+        const f2_t wm = pk(w0, w1);
+        px = fma2(wm, dx, px);
+        py = fma2(wm, dy, py);
+        pz = fma2(wm, dz, pz);
+        return;
+    }
     f2_t r2 = mul2(dx, dx);
     r2 = fma2(dy, dy, r2);
     r2 = fma2(dz, dz, r2);
@@ -478,23 +536,19 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
         const int i0 = a.group_first[g], ni = a.group_first[g + 1] - i0;
         const BoxDev &bx = a.boxes[a.group_box[g]];
         PairConsts cl;
-        if (!kUniform) {
-#pragma unroll
-            for (int q = 0; q <= NPOLY; q++) cl.poly[q] = pk(bx.poly[q], bx.poly[q]);
-            cl.s2 = pk(bx.s2, bx.s2);
-            cl.eps2s = pk(bx.eps2s, bx.eps2s);
-            cl.c_t = pk(bx.c_t, bx.c_t);
-            cl.c_e = pk(bx.c_e, bx.c_e);
-            cl.m1 = pk(-1.f, -1.f);
-            cl.rcut2 = bx.rcut2;
-            cl.rfilt2 = bx.rfilt2;
-        }
+        if (!kUniform) box_consts<NPOLY>(bx, cl);
         const PairConsts &c = kUniform ? a.uc : cl;
         const float rf2 = c.rfilt2;
-        const float4 gh = a.group_h4[g];
+        float4 gh = a.group_h4[g];
         constexpr int G = 32 / kSplit;
         const int ti = lane & (G - 1), hs = lane / G;   // target slot, source slot
-        const float4 xi4 = ti < ni ? a.pos_group[i0 + ti] : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 xi4 = ti < ni ? a.pos_group[i0 + ti] : make_float4(0.f, 0.f, 0.f, 0.f);
+        // the inverse-distance form works in lengths scaled by a power of two
+        const float sc = NPOLY == kInvDeg ? c.sc : 1.f;
+        if (NPOLY == kInvDeg) {
+            gh.x *= sc; gh.y *= sc; gh.z *= sc;
+            xi4.x *= sc; xi4.y *= sc; xi4.z *= sc;
+        }
         const f2_t xi = pk(xi4.x, xi4.x), yi = pk(xi4.y, xi4.y), zi = pk(xi4.z, xi4.z);
         Kahan3 k;
         int nbuf = 0;
@@ -517,9 +571,10 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
                 float4 p = cur.p;
                 bool keep = false;
                 if (cur.valid) {
-                    p.x = __fadd_rn(p.x, cur.ox);
-                    p.y = __fadd_rn(p.y, cur.oy);
-                    p.z = __fadd_rn(p.z, cur.oz);
+                    // sc (p + o), rounded once: sc is a power of two
+                    p.x = __fmaf_rn(p.x, sc, cur.ox * sc);
+                    p.y = __fmaf_rn(p.y, sc, cur.oy * sc);
+                    p.z = __fmaf_rn(p.z, sc, cur.oz * sc);
                     const float qx = fmaxf(fabsf(p.x) - gh.x, 0.f);
                     const float qy = fmaxf(fabsf(p.y) - gh.y, 0.f);
                     const float qz = fmaxf(fabsf(p.z) - gh.z, 0.f);
@@ -580,7 +635,7 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
         }
         if (hs == 0 && ti < ni) {
             const int64_t o = a.perm[i0 + ti];
-            const float Gc = kLearned ? bx.G : bx.c_g;
+            const float Gc = kLearned ? bx.G : NPOLY == kInvDeg ? bx.inv_g : bx.c_g;
             a.acc[3 * o + 0] = Gc * tx;
             a.acc[3 * o + 1] = Gc * ty;
             a.acc[3 * o + 2] = Gc * tz;
@@ -624,23 +679,20 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
         const int i0 = a.group_first[g], ni = a.group_first[g + 1] - i0;
         const BoxDev &bx = a.boxes[a.group_box[g]];
         PairConsts cl;
-        if (!kUniform) {
-#pragma unroll
-            for (int q = 0; q <= NPOLY; q++) cl.poly[q] = pk(bx.poly[q], bx.poly[q]);
-            cl.s2 = pk(bx.s2, bx.s2);
-            cl.eps2s = pk(bx.eps2s, bx.eps2s);
-            cl.c_t = pk(bx.c_t, bx.c_t);
-            cl.c_e = pk(bx.c_e, bx.c_e);
-            cl.m1 = pk(-1.f, -1.f);
-            cl.rcut2 = bx.rcut2;
-            cl.rfilt2 = bx.rfilt2;
-        }
+        if (!kUniform) box_consts<NPOLY>(bx, cl);
         const PairConsts &c = kUniform ? a.uc : cl;
-        const float rf2 = c.rfilt2;
-        const float4 gh = a.group_h4[g];
+        const float rf2 = c.rfilt2;   // of the staged (scaled) sources
+        const float4 gh0 = a.group_h4[g];
+        float4 gh = gh0;
         constexpr int G = 32 / kSplit;
         const int ti = lane & (G - 1), hs = lane / G;   // target slot, source slot
-        const float4 xi4 = ti < ni ? a.pos_group[i0 + ti] : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 xi4 = ti < ni ? a.pos_group[i0 + ti] : make_float4(0.f, 0.f, 0.f, 0.f);
+        // the inverse-distance form works in lengths scaled by a power of two
+        const float sc = NPOLY == kInvDeg ? c.sc : 1.f;
+        if (NPOLY == kInvDeg) {
+            gh.x *= sc; gh.y *= sc; gh.z *= sc;
+            xi4.x *= sc; xi4.y *= sc; xi4.z *= sc;
+        }
         const f2_t xi = pk(xi4.x, xi4.x), yi = pk(xi4.y, xi4.y), zi = pk(xi4.z, xi4.z);
         Kahan3 k;
         int nbuf = 0;
@@ -654,9 +706,10 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
                 float4 p = cur.p;
                 bool keep = false;
                 if (cur.valid) {
-                    p.x = __fadd_rn(p.x, cur.ox);
-                    p.y = __fadd_rn(p.y, cur.oy);
-                    p.z = __fadd_rn(p.z, cur.oz);
+                    // sc (p + o), rounded once: sc is a power of two
+                    p.x = __fmaf_rn(p.x, sc, cur.ox * sc);
+                    p.y = __fmaf_rn(p.y, sc, cur.oy * sc);
+                    p.z = __fmaf_rn(p.z, sc, cur.oz * sc);
                     const float qx = fmaxf(fabsf(p.x) - gh.x, 0.f);
                     const float qy = fmaxf(fabsf(p.y) - gh.y, 0.f);
                     const float qz = fmaxf(fabsf(p.z) - gh.z, 0.f);
@@ -693,6 +746,7 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
             const int gx = ground / (ns * ns), gy = (ground / ns) % ns, gz = ground % ns;
             const float4 gc = a.group_c4[g];
             const float hc = (float)bx.h;
+            const float rfb = bx.rfilt2;   // of the boxes (not scaled)
             int l0 = 0, cnt = 0;
             if (lane < 27) {
                 const int dx = lane / 9 - 1, dy = (lane / 3) % 3 - 1, dz = lane % 3 - 1;
@@ -701,10 +755,10 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
                 const int sy = ay < 0 ? -1 : (ay >= ns ? 1 : 0);
                 const int sz = az < 0 ? -1 : (az >= ns ? 1 : 0);
                 const int nc = bx.cell_base + ((ax - sx * ns) * ns + (ay - sy * ns)) * ns + (az - sz * ns);
-                const float qx = fmaxf(fmaxf(dx * hc - (gc.x + gh.x), (gc.x - gh.x) - (dx + 1) * hc), 0.f);
-                const float qy = fmaxf(fmaxf(dy * hc - (gc.y + gh.y), (gc.y - gh.y) - (dy + 1) * hc), 0.f);
-                const float qz = fmaxf(fmaxf(dz * hc - (gc.z + gh.z), (gc.z - gh.z) - (dz + 1) * hc), 0.f);
-                if (qx * qx + qy * qy + qz * qz < rf2 * 1.0001f) {
+                const float qx = fmaxf(fmaxf(dx * hc - (gc.x + gh0.x), (gc.x - gh0.x) - (dx + 1) * hc), 0.f);
+                const float qy = fmaxf(fmaxf(dy * hc - (gc.y + gh0.y), (gc.y - gh0.y) - (dy + 1) * hc), 0.f);
+                const float qz = fmaxf(fmaxf(dz * hc - (gc.z + gh0.z), (gc.z - gh0.z) - (dz + 1) * hc), 0.f);
+                if (qx * qx + qy * qy + qz * qz < rfb * 1.0001f) {
                     l0 = a.cell_leaf_first[nc];
                     cnt = a.cell_leaf_first[nc + 1] - l0;
                 }
@@ -733,10 +787,10 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
                 if (q < ctotal) {
                     const int l = ru.y + q;
                     const float4 lc = a.leaf_c4[l], lh = a.leaf_h4[l];
-                    const float px = fmaxf(fabsf((lc.x + odx * hc) - gc.x) - (gh.x + lh.x), 0.f);
-                    const float py = fmaxf(fabsf((lc.y + ody * hc) - gc.y) - (gh.y + lh.y), 0.f);
-                    const float pz = fmaxf(fabsf((lc.z + odz * hc) - gc.z) - (gh.z + lh.z), 0.f);
-                    acc = px * px + py * py + pz * pz < rf2;
+                    const float px = fmaxf(fabsf((lc.x + odx * hc) - gc.x) - (gh0.x + lh.x), 0.f);
+                    const float py = fmaxf(fabsf((lc.y + ody * hc) - gc.y) - (gh0.y + lh.y), 0.f);
+                    const float pz = fmaxf(fabsf((lc.z + odz * hc) - gc.z) - (gh0.z + lh.z), 0.f);
+                    acc = px * px + py * py + pz * pz < rfb;
                     if (acc) {
                         const int ax = gx + odx, ay = gy + ody, az = gz + odz;
                         const int sx = ax < 0 ? -1 : (ax >= ns ? 1 : 0);
@@ -804,7 +858,7 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
         }
         if (hs == 0 && ti < ni) {
             const int64_t o = a.perm[i0 + ti];
-            const float Gc = bx.c_g;
+            const float Gc = NPOLY == kInvDeg ? bx.inv_g : bx.c_g;
             a.acc[3 * o + 0] = Gc * tx;
             a.acc[3 * o + 1] = Gc * ty;
             a.acc[3 * o + 2] = Gc * tz;
@@ -835,8 +889,10 @@ __global__ void __launch_bounds__(kPPThreads) k_count_within(PPArgs a)
         if (g >= ng) break;
         const int i0 = a.group_first[g], ni = a.group_first[g + 1] - i0;
         const BoxDev &bx = a.boxes[a.group_box[g]];
-        const float rcut2 = bx.rcut2;
-        const float4 xi = lane < ni ? a.pos_group[i0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float sc = a.inverse ? bx.sc : 1.f, eps2 = a.inverse ? bx.eps2s : 0.f;
+        const float cut = a.inverse ? bx.inv_cut : bx.rcut2;
+        float4 xi = lane < ni ? a.pos_group[i0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+        xi.x *= sc; xi.y *= sc; xi.z *= sc;
         const int64_t e1 = a.group_off[g + 1] < a.cap ? a.group_off[g + 1] : a.cap;
         for (int64_t e = a.group_off[g]; e < e1; e++) {
             const float4 ent = a.entries[e];
@@ -848,9 +904,9 @@ __global__ void __launch_bounds__(kPPThreads) k_count_within(PPArgs a)
                 float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (ok) {
                     p = a.pos_leaf[j];
-                    p.x = __fadd_rn(p.x, ent.x);
-                    p.y = __fadd_rn(p.y, ent.y);
-                    p.z = __fadd_rn(p.z, ent.z);
+                    p.x = __fmaf_rn(p.x, sc, ent.x * sc);
+                    p.y = __fmaf_rn(p.y, sc, ent.y * sc);
+                    p.z = __fmaf_rn(p.z, sc, ent.z * sc);
                 }
                 const unsigned bal = __ballot_sync(0xffffffffu, ok);
                 __syncwarp();
@@ -860,8 +916,8 @@ __global__ void __launch_bounds__(kPPThreads) k_count_within(PPArgs a)
                 for (int jj = 0; jj < nb; jj++) {
                     const float4 pj = buf[jj];
                     const float dx = pj.x - xi.x, dy = pj.y - xi.y, dz = pj.z - xi.z;
-                    const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-                    if (lane < ni && r2 < rcut2 && jb + jj != i0 + lane) cnt_within++;   // not the self pair
+                    const float r2 = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, eps2)));
+                    if (lane < ni && r2 < cut && jb + jj != i0 + lane) cnt_within++;   // not the self pair
                 }
             }
         }
@@ -915,12 +971,14 @@ static void pp_args(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, PPArg
     a.n_inter = reinterpret_cast<unsigned long long *>(work + 8);
     a.n_staged = reinterpret_cast<unsigned long long *>(work + 16);
     a.acc = d_acc;
+    a.inverse = lv->poly_degree == kInvDeg;
 }
 
 template <bool kLearned, int kMinBlocks, int kSplit, bool kUniform>
 static void launch_pp(int npoly, int grid, cudaStream_t s, const PPArgs &a)
 {
     switch (npoly) {
+    case kInvDeg: k_pp<kInvDeg, kLearned, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
     case 10: k_pp<10, kLearned, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
     case 12: k_pp<12, kLearned, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
     case 14: k_pp<14, kLearned, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
@@ -932,6 +990,7 @@ template <int kMinBlocks, int kSplit, bool kUniform>
 static void launch_walk_one(int npoly, int grid, cudaStream_t s, const PPArgs &a)
 {
     switch (npoly) {
+    case kInvDeg: k_pp_walk<kInvDeg, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
     case 10: k_pp_walk<10, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
     case 12: k_pp_walk<12, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
     case 14: k_pp_walk<14, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
@@ -1011,15 +1070,18 @@ int pp_learned_device(const ph_leaves *lv, const ph_pairs *pr, const float *mlp_
 }
 
 // true if every box has the same factor constants (then the kernel reads
-// them from its parameter bank)
-static bool uniform_consts(const ph_leaves *lv, PairConsts &uc)
+// them from its parameter bank); general: those of the general form, which
+// the tabulated factor's kernel uses whatever the exact kernel does
+static bool uniform_consts(const ph_leaves *lv, PairConsts &uc, bool general)
 {
     if ((int)lv->boxes_host.size() < lv->n_boxes || lv->n_boxes < 1) return false;   // no host copy of the boxes
     const BoxDev &b0 = lv->boxes_host[0];
     for (int b = 1; b < lv->n_boxes; b++) {
         const BoxDev &bx = lv->boxes_host[b];
         if (memcmp(bx.poly, b0.poly, sizeof b0.poly) || bx.s2 != b0.s2 || bx.eps2s != b0.eps2s || bx.c_t != b0.c_t ||
-            bx.c_e != b0.c_e || bx.rcut2 != b0.rcut2 || bx.rfilt2 != b0.rfilt2)
+            bx.c_e != b0.c_e || bx.rcut2 != b0.rcut2 || bx.rfilt2 != b0.rfilt2 ||
+            memcmp(bx.inv_poly, b0.inv_poly, sizeof b0.inv_poly) || bx.inv_b1 != b0.inv_b1 ||
+            bx.inv_b2 != b0.inv_b2 || bx.inv_zc != b0.inv_zc || bx.inv_cut != b0.inv_cut)
             return false;
     }
     auto dup = [](float v) {
@@ -1029,14 +1091,20 @@ static bool uniform_consts(const ph_leaves *lv, PairConsts &uc)
         u = ((uint64_t)bits << 32) | bits;
         return (f2_t)u;
     };
-    for (int q = 0; q <= kMaxPoly; q++) uc.poly[q] = dup(b0.poly[q]);
+    const bool inv = lv->poly_degree == kInvDeg && !general;
+    for (int q = 0; q <= kMaxPoly; q++) uc.poly[q] = dup(!inv ? b0.poly[q] : q <= kInvDeg ? b0.inv_poly[q] : 0.f);
     uc.s2 = dup(b0.s2);
     uc.eps2s = dup(b0.eps2s);
     uc.c_t = dup(b0.c_t);
     uc.c_e = dup(b0.c_e);
     uc.m1 = dup(-1.f);
-    uc.rcut2 = b0.rcut2;
-    uc.rfilt2 = b0.rfilt2;
+    uc.rcut2 = inv ? b0.inv_cut : b0.rcut2;
+    uc.rfilt2 = inv ? b0.rfilt2 * b0.s2 : b0.rfilt2;
+    uc.zc = dup(b0.inv_zc);
+    uc.b1 = dup(b0.inv_b1);
+    uc.b2 = dup(b0.inv_b2);
+    uc.m53 = dup(-kInvK);
+    uc.sc = inv ? b0.sc : 1.f;
     return true;
 }
 
@@ -1047,7 +1115,7 @@ int pp_table_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaS
     PPArgs a;
     pp_args(lv, pr, d_acc, a);
     a.mlp_w = nullptr;
-    if (!uniform_consts(lv, a.uc)) return fail(PH_ERR_ARG, "the tabulated factor needs one rcut and rs for all boxes");
+    if (!uniform_consts(lv, a.uc, true)) return fail(PH_ERR_ARG, "the tabulated factor needs one rcut and rs for all boxes");
     a.table = static_cast<const float2 *>(lv->table.p);
     a.tab_scale2 = (float)((kTabN / lv->table_rcut) * (kTabN / lv->table_rcut));
     int rc2 = cuda_check(cudaMemsetAsync(pr->work.p, 0, 24, s), "reset work queue");
@@ -1068,9 +1136,9 @@ int pp_exact_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaS
     int rc = cuda_check(cudaMemsetAsync(pr ? pr->work.p : lv->work.p, 0, 24, s), "reset work queue");
     if (rc) return rc;
     const int npoly = lv->poly_degree;
-    if (npoly != 10 && npoly != 12 && npoly != 14 && npoly != 16)
+    if (npoly != kInvDeg && npoly != 10 && npoly != 12 && npoly != 14 && npoly != 16)
         return fail(PH_ERR_STATE, "unsupported polynomial degree %d", npoly);
-    const bool uni = uniform_consts(lv, a.uc);
+    const bool uni = uniform_consts(lv, a.uc, false);
     if (!pr) {
         launch_walk(lv, npoly, uni, s, a);
         count_launch();
