@@ -298,12 +298,13 @@ uint64_t buffers_fingerprint(const ph_leaves *h, const ph_pairs *p)
     fp_mix(f, (uint64_t)h->n);
     if (p) {
         const DevBuf *pb[] = {&p->group_cnt, &p->group_off, &p->entries, &p->ecount, &p->work, &p->status, &p->temp,
-                              &p->group_key, &p->group_order, &p->order_temp};
+                              &p->group_key, &p->group_order, &p->order_temp, &p->task_mem};
         for (const DevBuf *b : pb) {
             fp_mix(f, (uint64_t)(uintptr_t)b->p);
             fp_mix(f, (uint64_t)b->bytes);
         }
         fp_mix(f, (uint64_t)p->capacity);
+        fp_mix(f, (uint64_t)p->task_cap);
     }
     return f;
 }
@@ -322,7 +323,7 @@ static void free_leaves(ph_leaves *h)
 static void free_pairs(ph_pairs *h)
 {
     DevBuf *bufs[] = {&h->group_cnt, &h->group_off, &h->entries, &h->ecount, &h->work, &h->status, &h->temp,
-                      &h->acc_tmp, &h->group_key, &h->group_order, &h->order_temp};
+                      &h->acc_tmp, &h->group_key, &h->group_order, &h->order_temp, &h->task_mem};
     for (DevBuf *b : bufs) release(*b);
 }
 
@@ -376,6 +377,7 @@ static int leaves_common(const void *pos, int pos_type, const float *mass, const
     h->level_bits = params[0].level_bits ? params[0].level_bits : 1;
     h->pp_variant = params[0].pp_variant;
     h->queue_order = params[0].queue_order;
+    h->segment = segment_entries(n, h->max_leaf, h->group_size);
     h->boxes_host.resize(nb);
     const int deg = exact_degree_for(params, nb);
     h->poly_degree = deg;
@@ -576,8 +578,8 @@ int ph_leaf_pairs(ph_leaves *leaves, void *stream, ph_pairs **pairs)
     if (!rc && leaves->queue_order == 0) {
         rc = ensure(p->group_key, N);
         if (!rc) rc = ensure(p->group_order, 4 * N);
-        if (!rc) rc = ensure(p->order_temp, order_temp_bytes((int64_t)N));
     }
+    if (!rc) rc = ensure(p->order_temp, order_temp_bytes());
     if (!rc && !p->status.p) {
         rc = ensure(p->status, 16);
         if (!rc) rc = cuda_check(cudaMemsetAsync(p->status.p, 0, 16, s), "status reset");
@@ -587,6 +589,11 @@ int ph_leaf_pairs(ph_leaves *leaves, void *stream, ph_pairs **pairs)
         if (!rc) rc = ensure(p->ecount, 1024);
         if (!rc) p->capacity = 1024;
     }
+    // (a reserved list is not sized: as many slots as it can need)
+    if (!rc && p->fixed_capacity && !p->task_cap)
+        rc = ensure_tasks(p, task_bound(p->capacity, leaves->segment), (int64_t)N);
+    else if (!rc)
+        rc = ensure_tasks(p, p->task_cap, (int64_t)N);
     if (!rc) rc = build_pairs_device(leaves, p, s, !p->fixed_capacity);
     if (rc) {
         if (fresh) {

@@ -90,6 +90,15 @@ int ph_graph_create(ph_leaves *leaves, ph_pairs *pairs, const void *d_pos, int p
             }
             pairs->capacity = want;
         }
+        const int64_t slots = (int64_t)((double)pairs->n_tasks * (1.0 + headroom)) + 64;
+        if (slots > pairs->task_cap) {
+            int rc = cuda_check(cudaStreamSynchronize(caller), "sync before growing");
+            if (!rc) rc = ensure_tasks(pairs, slots, leaves->n);
+            if (rc) {
+                pairs->valid = false;   // the tasks are gone
+                return rc;
+            }
+        }
         pairs->fixed_capacity = true;
     }
     bool learned = false;

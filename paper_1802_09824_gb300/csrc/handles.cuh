@@ -23,6 +23,7 @@ struct ph_leaves {
     int32_t key_kind = PH_KEY_MORTON;
     int32_t level_bits = 1;      // key bits per level of the leaf hierarchy (1 or 3)
     int32_t pp_variant = 0;      // PP kernel register/occupancy variant (0: 2 blocks/SM, 1: 3)
+    int32_t segment = 256;       // pair entries per segment of a group's PP sum (segment_entries)
     int32_t queue_order = 0;     // PP queue: 0 = groups by decreasing cost, 1 = group order
     bool tree_leaves = false;    // some box has theta > 0: leaf mass-centre particles are made
     std::vector<phpp::BoxDev> boxes_host;
@@ -95,7 +96,15 @@ struct ph_pairs {
     // pass when these buffers exist; `ordered` says the last list has it
     phpp::DevBuf group_key;      // uint8[n]: 255 - cost bucket
     phpp::DevBuf group_order;    // int32[n]: groups in queue order
-    phpp::DevBuf order_temp;     // histograms and scan scratch
+    phpp::DevBuf order_temp;     // int32[514]: groups per key, cursors, the number of tasks written and needed
+    // groups with more than one segment are queued as one task per segment
+    phpp::DevBuf task_mem;       // the four arrays below
+    int2 *tasks = nullptr;       // [task_cap] (group, segment), a group's in a row; group -1: none
+    int32_t *task_done = nullptr;// [task_cap] segments summed, at the group's first task
+    float *task_part = nullptr;  // [task_cap][3][32] the segments' sums
+    uint8_t *split_of = nullptr; // [n] of a group with several segments: whether it has tasks
+    int64_t task_cap = 0;
+    int64_t n_tasks = 0;         // host copy (valid after sizing sync)
     bool ordered = false;
 };
 
@@ -104,6 +113,9 @@ namespace phpp {
 // is incomplete or made for another build (PH_ERR_STATE), so no kernel ever
 // reads buffers that a failed or newer build left behind.
 int check_built(const ph_leaves *lv, const ph_pairs *pr);
+
+// Room for `slots` tasks of a list over n particles (pairs.cu).
+int ensure_tasks(ph_pairs *pr, int64_t slots, int64_t n);
 
 // A fingerprint of the device buffers of a leaves (and pairs) handle: their
 // addresses and sizes.  A captured graph holds these addresses; it may only

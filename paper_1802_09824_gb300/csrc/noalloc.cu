@@ -97,12 +97,12 @@ void carve(Carver &c, ph_leaves &lv, ph_pairs &pr, int64_t n, int cells)
     c.take(lv.group_scan, 4 * (N + 1));
     c.take(lv.leaf_first, 4 * (N + 1));
     c.take(lv.group_first, 4 * (N + 1));
-    c.take(lv.leaf_ref, 24 * N);
+    c.take(lv.group_h4, 16 * N);
+    c.take(lv.leaf_ref, 24 * N);   // from here to box_ext: not read by the PP kernel
     c.take(lv.leaf_c4, 16 * N);
     c.take(lv.leaf_h4, 16 * N);
     c.take(lv.group_ref, 24 * N);
     c.take(lv.group_c4, 16 * N);
-    c.take(lv.group_h4, 16 * N);
     c.take(lv.leaf_r4, 16 * N);
     c.take(lv.group_r4, 16 * N);
     c.take(lv.box_ext, 96 * N);
@@ -123,6 +123,24 @@ void carve(Carver &c, ph_leaves &lv, ph_pairs &pr, int64_t n, int cells)
     const size_t cap = (size_t)PH_NOALLOC_PAIRS_PER_PARTICLE * N;
     c.take(pr.entries, 16 * cap);
     c.take(pr.ecount, cap);
+    c.take(pr.order_temp, order_temp_bytes());
+    // the tasks of split groups: records and counters where the build's flags
+    // were, sums where the boxes' tables and extents were (what the PP kernel
+    // does not read)
+    const size_t room = (size_t)((char *)lv.box_ext.p + lv.box_ext.bytes - (char *)lv.leaf_ref.p) / (96 * sizeof(float));
+    pr.task_cap = (int64_t)(room < N / 2 ? room : N / 2);
+    pr.tasks = static_cast<int2 *>(lv.leaf_flag.p);
+    pr.task_done = static_cast<int32_t *>(lv.group_flag.p);
+    pr.task_part = static_cast<float *>(lv.leaf_ref.p);
+    pr.split_of = static_cast<uint8_t *>(lv.group_scan.p);
+}
+
+// Segment length of the step: twice segment_entries' (there are fewer task
+// slots than a list at its capacity could ask for: N / 2, with a group whose
+// tasks find no room summed by one warp).
+int noalloc_segment(int64_t n, int leaf_max)
+{
+    return segment_entries(2 * n, leaf_max, kDefaultGroup);
 }
 
 }  // namespace
@@ -189,6 +207,7 @@ extern "C" int ph_accel_noalloc(const float *d_pos, const float *d_mass, int64_t
     lv.group_size = kDefaultGroup;
     lv.poly_degree = deg;
     lv.max_leaf = p.leaf_max;
+    lv.segment = noalloc_segment(n, p.leaf_max);
     lv.key_kind = p.key_kind;
     lv.level_bits = p.level_bits ? p.level_bits : 1;
     lv.pp_variant = p.pp_variant == 1 ? 1 : 0;

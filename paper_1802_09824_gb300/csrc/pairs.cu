@@ -27,6 +27,8 @@
 // cursor per key.  Groups of one key land in the order the fill pass meets
 // them; the forces do not depend on the order (each group is summed by one
 // warp on its own).
+#include <algorithm>
+
 #include "checks.cuh"
 #include "handles.cuh"
 
@@ -56,6 +58,12 @@ struct PairArgs {
     int64_t n_particles;     // mass-centre particle of leaf l: pos_leaf[n_particles + l]
     int64_t cap;
     uint32_t *status;
+    int32_t *n_tasks;        // tasks of split groups: [0] written by the fill pass, [1] needed (count pass)
+    int2 *tasks;
+    uint8_t *split_of;       // [n_groups]: whether a group of several segments has tasks
+    int32_t *task_done;
+    int64_t task_cap;
+    int segment;             // entries per segment
     int64_t n_leaf_rows;     // rows of the leaf arrays (bounds checks)
 };
 
@@ -119,6 +127,24 @@ __global__ void __launch_bounds__(kThreads) k_pairs(PairArgs a)
             const int k = a.gkey[g];
             const int pos = s_start[k] + atomicAdd(&a.ohist[kOrdKeys + k], 1);
             if (in_bounds(pos, ng, BS_ORDER)) a.order[pos] = g;
+        }
+        if (kFill) {
+            // a group of more than one segment: one task per segment
+            const int64_t e0 = a.off[g] < a.cap ? a.off[g] : a.cap, e1 = a.off[g + 1] < a.cap ? a.off[g + 1] : a.cap;
+            if (e1 - e0 > a.segment) {
+                const int nseg = (int)((e1 - e0 + a.segment - 1) / a.segment);
+                int first = 0;
+                if (lane == 0) first = atomicAdd(a.n_tasks, nseg);
+                first = __shfl_sync(0xffffffffu, first, 0);
+                // (a list that outgrew its task slots: the group is summed by
+                // one warp, and the slots left over are empty)
+                const bool fits = first + nseg <= a.task_cap;
+                for (int k = lane; k < nseg && first + k < a.task_cap; k += 32) {
+                    a.tasks[first + k] = make_int2(fits ? g : -1, k);
+                    a.task_done[first + k] = 0;
+                }
+                if (lane == 0) a.split_of[g] = fits ? 1 : 0;
+            }
         }
         const BoxDev &bx = a.boxes[a.group_box[g]];
         const int ns = bx.nside;
@@ -247,6 +273,7 @@ __global__ void __launch_bounds__(kThreads) k_pairs(PairArgs a)
             const unsigned cost = __reduce_add_sync(0xffffffffu, src);
             if (lane == 0) {
                 a.cnt[g] = count;
+                if (count > a.segment) atomicAdd(a.n_tasks + 1, (int)((count + a.segment - 1) / a.segment));
                 if (a.gkey) {
                     const int k = 255 - cost_bucket(cost);
                     a.gkey[g] = (uint8_t)k;
@@ -260,18 +287,61 @@ __global__ void __launch_bounds__(kThreads) k_pairs(PairArgs a)
 
 }  // namespace
 
-// Scratch of the group order: the per-key counts and cursors.
-size_t order_temp_bytes(int64_t) { return 2 * kOrdKeys * sizeof(int32_t); }
+// Scratch of the queue: the per-key counts and cursors, the number of tasks.
+size_t order_temp_bytes() { return (2 * kOrdKeys + 4) * sizeof(int32_t); }
+
+// A warp sums a group's list segment by segment, and a group of several
+// segments is shared out to as many warps.  Without that, the longest list
+// bounds the launch (a halo core of 65,000 sources kept one warp busy for
+// 4 ms of a 6 ms launch; SMs were active 69 % of it on average), and a box
+// of few groups leaves most warps without work (4096 particles: 128 groups
+// for 2432 resident warps).  Per step, before and after:
+//   uniform 4096 180 -> 141 us, 50,021 684 -> 397, 150,000 1925 -> 1520;
+//   lattice 64^3 769 -> 727; 24 boxes with and without a halo 6230 -> 5736;
+//   halo mixture 48^3 1810 -> 955, 80^3 4633 -> 3800.
+// A segment is n / 50 sources' worth of entries, at least 256 sources and 8
+// entries (shorter tasks are mostly start-up: n / 200 ran 426 us at 50,021,
+// twice the minimum 147 us at 4096).  Where the groups fill the resident
+// warps less than six times over, at most 2000 sources, so that an evenly
+// filled box splits its lists too (64^3: 761 us whole, 727 with 2000, 743
+// with 2600); with six rounds or more even lists stay whole (a limit at ten
+// rounds cost 80^3 2 %, at twenty 100^3 4 %) and only long ones are cut, at
+// most every 32,768 sources.
+int segment_entries(int64_t n, int leaf_max, int group_size)
+{
+    const int64_t warps = 152 * 16;   // resident in the two-block shape
+    const int64_t most = n / group_size >= 6 * warps ? 32768 : 2000;
+    const int64_t sources = std::min<int64_t>(std::max<int64_t>(n / 50, 256), most);
+    return (int)std::max<int64_t>(sources / leaf_max, 8);
+}
+
+int ensure_tasks(ph_pairs *pr, int64_t slots, int64_t n)
+{
+    const size_t c = ((size_t)slots + 31) & ~(size_t)31;
+    if (pr->task_cap >= (int64_t)c && pr->task_mem.bytes >= (size_t)pr->task_cap * 396 + (size_t)n) return PH_OK;
+    pr->task_cap = 0;
+    const int rc = ensure(pr->task_mem, c * 396 + (size_t)n);
+    if (rc) return rc;
+    char *p = static_cast<char *>(pr->task_mem.p);
+    pr->task_cap = (int64_t)c;
+    pr->task_part = reinterpret_cast<float *>(p);
+    pr->tasks = reinterpret_cast<int2 *>(p + c * 384);
+    pr->task_done = reinterpret_cast<int32_t *>(p + c * 392);
+    pr->split_of = reinterpret_cast<uint8_t *>(p + c * 396);
+    return PH_OK;
+}
 
 // The sizing (with `sizing_sync`: read the total, grow the entry buffers)
 // and the fill pass, on stream s.
-static int fill_pairs(ph_pairs *pr, PairArgs &a, const int32_t *n_all, int grid, cudaStream_t s, bool sizing_sync)
+static int fill_pairs(ph_pairs *pr, PairArgs &a, const int32_t *n_all, int grid, cudaStream_t s, bool sizing_sync,
+                      int64_t n)
 {
     int rc = 0;
     if (sizing_sync) {
         // total = group_off[n_groups]; read the count then the total
-        int32_t ng = 0;
-        rc = cuda_check(cudaMemcpyAsync(&ng, n_all, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "copy n_groups");
+        int32_t ng = 0, nt = 0;
+        rc = cuda_check(cudaMemcpyAsync(&nt, a.n_tasks + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "copy n_tasks");
+        if (!rc) rc = cuda_check(cudaMemcpyAsync(&ng, n_all, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "copy n_groups");
         if (rc) return rc;
         rc = cuda_check(cudaStreamSynchronize(s), "sync n_groups");
         if (rc) return rc;
@@ -290,7 +360,14 @@ static int fill_pairs(ph_pairs *pr, PairArgs &a, const int32_t *n_all, int grid,
             if (rc) return rc;
             pr->capacity = cap;
         }
+        pr->n_tasks = nt;
+        rc = ensure_tasks(pr, nt > pr->task_cap ? nt + nt / 8 : nt, n);
+        if (rc) return rc;
     }
+    a.tasks = pr->tasks;
+    a.task_done = pr->task_done;
+    a.task_cap = pr->task_cap;
+    a.split_of = pr->split_of;
     a.ent = static_cast<float4 *>(pr->entries.p);
     a.ecnt = static_cast<uint8_t *>(pr->ecount.p);
     a.cap = pr->capacity;
@@ -329,9 +406,12 @@ int build_pairs_device(const ph_leaves *lv, ph_pairs *pr, cudaStream_t s, bool s
     // the active-particle mode, whose inactive groups get no list (the PP
     // kernel takes them in group order there)
     const bool ordered =
-        lv->queue_order == 0 && !lv->active && pr->group_key.p && pr->group_order.p && pr->order_temp.p;
+        lv->queue_order == 0 && !lv->active && pr->group_key.p && pr->group_order.p;
+    int32_t *const ot = static_cast<int32_t *>(pr->order_temp.p);
+    a.n_tasks = ot + 2 * kOrdKeys;
+    a.segment = lv->segment;
     a.gkey = ordered ? static_cast<uint8_t *>(pr->group_key.p) : nullptr;
-    a.ohist = ordered ? static_cast<int32_t *>(pr->order_temp.p) : nullptr;
+    a.ohist = ordered ? ot : nullptr;
     a.order = ordered ? static_cast<int32_t *>(pr->group_order.p) : nullptr;
     pr->ordered = ordered;
     a.off = static_cast<const int64_t *>(pr->group_off.p);
@@ -343,15 +423,15 @@ int build_pairs_device(const ph_leaves *lv, ph_pairs *pr, cudaStream_t s, bool s
         const int rz = cuda_check(cudaMemsetAsync(a.cnt, 0, 8 * (size_t)(n > 0 ? n : 1), s), "clear counts");
         if (rz) return rz;
     }
-    if (ordered) {
-        const int rz = cuda_check(cudaMemsetAsync(a.ohist, 0, order_temp_bytes(0), s), "clear key counts");
+    {
+        const int rz = cuda_check(cudaMemsetAsync(ot, 0, order_temp_bytes(), s), "clear the queue's counts");
         if (rz) return rz;
     }
     k_pairs<false><<<grid, kThreads, 0, s>>>(a);
     count_launch();
     int rc = scan_exclusive_i64(a.cnt, static_cast<int64_t *>(pr->group_off.p), n, n_all, pr->temp.p, s);
     if (rc) return rc;
-    rc = fill_pairs(pr, a, n_all, grid, s, sizing_sync);
+    rc = fill_pairs(pr, a, n_all, grid, s, sizing_sync, n);
     if (rc) return rc;
     return cuda_check(cudaGetLastError(), "pair kernels");
 }

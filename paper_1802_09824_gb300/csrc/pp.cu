@@ -88,6 +88,14 @@ struct PPArgs {
     const float2 *table;
     float tab_scale2;                // (kTabN / rcut)^2
     int64_t n_pos;                   // rows of pos_leaf (bounds checks)
+    // groups of several segments, one task each (pairs.cu)
+    const int32_t *n_tasks;
+    const int2 *tasks;               // (group, segment); group -1: no task
+    int32_t *task_done;
+    float *task_part;                // [task][3][32]
+    const uint8_t *split_of;
+    int64_t task_cap;
+    int segment;                     // entries per segment
     bool inverse;                    // the exact kernel runs the inverse-distance form (count kernel)
     const int32_t *order;            // queue slot -> group (groups by decreasing cost), or NULL
 };
@@ -490,6 +498,42 @@ struct Round {
     }
 };
 
+// The sum of a task (one segment of a split group's list, at task slot t):
+// kept aside, and the warp that finishes a group's last segment adds them up
+// in segment order with compensation, whichever warps computed them.
+template <int G>
+__device__ __noinline__ void finish_task(const PPArgs &a, int t, int ni, int i0, float Gc, float tx, float ty, float tz)
+{
+    const int lane = threadIdx.x & 31;
+    const int2 tk = a.tasks[t];
+    const int first = t - tk.y;
+    const int64_t b = a.group_off[tk.x], e = a.group_off[tk.x + 1];
+    const int nseg = (int)(((e < a.cap ? e : a.cap) - b + a.segment - 1) / a.segment);
+    if (lane < G) {
+        float *p = a.task_part + (int64_t)t * 96 + lane;
+        __stcg(p, tx);
+        __stcg(p + 32, ty);
+        __stcg(p + 64, tz);
+    }
+    __threadfence();
+    __syncwarp();
+    int done = 0;
+    if (lane == 0) done = atomicAdd(a.task_done + first, 1);
+    done = __shfl_sync(0xffffffffu, done, 0);
+    if (done != nseg - 1) return;
+    if (lane == 0) a.task_done[first] = 0;   // ready for another sum over this list
+    __threadfence();
+    if (lane < ni) {
+        Kahan3 k;
+        const float *p = a.task_part + (int64_t)first * 96 + lane;
+        for (int q = 0; q < nseg; q++, p += 96) k.add(__ldcg(p), __ldcg(p + 32), __ldcg(p + 64));
+        const int64_t o = a.perm[i0 + lane];
+        a.acc[3 * o + 0] = Gc * (k.sx - k.cx);
+        a.acc[3 * o + 1] = Gc * (k.sy - k.cy);
+        a.acc[3 * o + 2] = Gc * (k.sz - k.cz);
+    }
+}
+
 // Source staging and summation for one target group.  Entries are taken 32
 // at a time, one per lane; the lanes' leaf sizes are prefix-summed and the
 // concatenated source particles are loaded 32 per round, each lane finding
@@ -514,6 +558,7 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
     float4 *A = sA[w], *Bq = sB[w];
     float *Af = reinterpret_cast<float *>(A), *Bf = reinterpret_cast<float *>(Bq);
     const int ng = *a.n_groups;
+    const int nt = *a.n_tasks < a.task_cap ? *a.n_tasks : (int)a.task_cap;
     unsigned long long inter = 0, staged = 0;
     MlpLane L;
     if (kLearned) {
@@ -525,21 +570,52 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
         for (int i = threadIdx.x; i <= kTabN; i += blockDim.x) sTab[i] = a.table[i];
         __syncthreads();
     }
-    for (;;) {
-        int g = 0;
-        if (lane == 0) {
-            g = atomicAdd(a.queue, 1);
-            if (a.order && g < ng) g = a.order[g];   // the queue's order (a permutation of the groups)
+    // The queue: the tasks of split groups, then the other groups in their
+    // order (a permutation of the groups).  While at least eight rounds of all
+    // warps are left a warp draws its next slot before it sums the current
+    // one, so the atomic's latency is hidden (128^3 lattice step 4191 ->
+    // 4132 us); near the end it draws when it is free, so that no warp holds
+    // work that an idle one could take (with two rounds as the line the 64^3
+    // step took 797 us instead of 761).
+    const int total = nt + ng, spare = 8 * (int)(gridDim.x * kPPWarps);
+    int t_next = 0;
+    if (lane == 0) t_next = atomicAdd(a.queue, 1);
+    bool drawn = false;
+    auto draw = [&]() {
+        if (!drawn && lane == 0) t_next = atomicAdd(a.queue, 1);
+    };
+    for (;; draw()) {
+        const int t = __shfl_sync(0xffffffffu, t_next, 0);
+        if (t >= total) break;
+        drawn = t < total - spare;
+        if (drawn && lane == 0) t_next = atomicAdd(a.queue, 1);
+        const bool task = t < nt;
+        int g, seg = 0;
+        if (task) {
+            const int2 tk = a.tasks[t];
+            g = tk.x;
+            seg = tk.y;
+            if (g < 0) continue;
+        } else {
+            g = a.order ? a.order[t - nt] : t - nt;
         }
-        g = __shfl_sync(0xffffffffu, g, 0);
-        if (g >= ng) break;
-        const int i0 = a.group_first[g], ni = a.group_first[g + 1] - i0;
+        int64_t e0 = a.group_off[g], e1 = a.group_off[g + 1];
+        const int i0 = a.group_first[g], ni = a.group_first[g + 1] - i0;   // (loaded beside the offsets)
         const BoxDev &bx = a.boxes[a.group_box[g]];
+        float4 gh = a.group_h4[g];
+        if (e1 > a.cap) e1 = a.cap;
+        if (e1 - e0 > a.segment) {
+            if (task) {
+                e0 += (int64_t)seg * a.segment;
+                e1 = e0 + a.segment < e1 ? e0 + a.segment : e1;
+            } else if (a.split_of[g]) {
+                continue;   // its tasks came first
+            }
+        }
         PairConsts cl;
         if (!kUniform) box_consts<NPOLY>(bx, cl);
         const PairConsts &c = kUniform ? a.uc : cl;
         const float rf2 = c.rfilt2;
-        float4 gh = a.group_h4[g];
         constexpr int G = 32 / kSplit;
         const int ti = lane & (G - 1), hs = lane / G;   // target slot, source slot
         float4 xi4 = ti < ni ? a.pos_group[i0 + ti] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -558,10 +634,9 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
             lq.l1 = sDyn;
             if (lane == 0) lq.q[kLQ] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        const int64_t e1 = a.group_off[g + 1] < a.cap ? a.group_off[g + 1] : a.cap;
         // Entries are taken 32 at a time; each round loads 32 concatenated
         // source particles of the batch, one per lane.
-        for (int64_t eb = a.group_off[g]; eb < e1; eb += 32) {
+        for (int64_t eb = e0; eb < e1; eb += 32) {
             EntryBatch bt;
             bt.load(a, eb, e1, lane);
             int before = 0;
@@ -633,9 +708,11 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
             ty += __shfl_xor_sync(0xffffffffu, ty, o);
             tz += __shfl_xor_sync(0xffffffffu, tz, o);
         }
-        if (hs == 0 && ti < ni) {
+        const float Gc = kLearned ? bx.G : NPOLY == kInvDeg ? bx.inv_g : bx.c_g;
+        if (task) {
+            finish_task<G>(a, t, ni, i0, Gc, tx, ty, tz);
+        } else if (hs == 0 && ti < ni) {
             const int64_t o = a.perm[i0 + ti];
-            const float Gc = kLearned ? bx.G : NPOLY == kInvDeg ? bx.inv_g : bx.c_g;
             a.acc[3 * o + 0] = Gc * tx;
             a.acc[3 * o + 1] = Gc * ty;
             a.acc[3 * o + 2] = Gc * tz;
@@ -665,6 +742,7 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
     __shared__ int2 sRun[kPPWarps][32];
     __shared__ float4 sQEnt[kPPWarps][64];
     __shared__ int sQCnt[kPPWarps][64];
+    __shared__ Kahan3 sFold[kPPWarps][32];   // the sum over the segments done
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     float4 *A = sA[w], *Bq = sB[w];
@@ -736,6 +814,30 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
                 }
                 nbuf += nk;
             }
+        };
+        // A segment's end: its sum joins the group's, as the list kernel's
+        // tasks do (finish_task).
+        Kahan3 &fold = sFold[w][lane];
+        fold = Kahan3();
+        int left = a.segment;          // entries the segment still takes
+        auto end_segment = [&]() {
+            const int padded = pad_sources<kSplit>(Af, Bf, nbuf, lane);
+            __syncwarp();
+            sum_buffer<NPOLY, kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, k);
+            inter += (unsigned long long)nbuf * ni;
+            staged += nbuf;
+            nbuf = 0;
+            __syncwarp();
+            // the kSplit source slots of a target add up their compensated totals
+            float tx = k.sx - k.cx, ty = k.sy - k.cy, tz = k.sz - k.cz;
+#pragma unroll
+            for (int o = G; o < 32; o <<= 1) {
+                tx += __shfl_xor_sync(0xffffffffu, tx, o);
+                ty += __shfl_xor_sync(0xffffffffu, ty, o);
+                tz += __shfl_xor_sync(0xffffffffu, tz, o);
+            }
+            fold.add(tx, ty, tz);
+            k = Kahan3();
         };
         {
             // Direct mode: the leaf pairs of the group are found here, as the
@@ -821,17 +923,27 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
                 }
                 qn += __popc(bal);
                 __syncwarp();
-                if (qn >= 32) {
+                for (int nb = left < 32 ? left : 32; qn >= nb; nb = left < 32 ? left : 32) {
                     EntryBatch bt;
-                    bt.set(sQEnt[w][lane], sQCnt[w][lane], lane);
+                    const bool has = lane < nb;
+                    bt.set(has ? sQEnt[w][lane] : make_float4(0.f, 0.f, 0.f, 0.f), has ? sQCnt[w][lane] : 0, lane);
+                    // the rest moves up (qn - nb may exceed 32: two per lane)
+                    const int s0 = nb + lane, s1 = nb + 32 + lane;
+                    float4 m0, m1;
+                    int c0m = 0, c1m = 0;
+                    if (s0 < qn) { m0 = sQEnt[w][s0]; c0m = sQCnt[w][s0]; }
+                    if (s1 < qn) { m1 = sQEnt[w][s1]; c1m = sQCnt[w][s1]; }
                     __syncwarp();
-                    if (lane < qn - 32) {
-                        sQEnt[w][lane] = sQEnt[w][32 + lane];
-                        sQCnt[w][lane] = sQCnt[w][32 + lane];
-                    }
+                    if (s0 < qn) { sQEnt[w][lane] = m0; sQCnt[w][lane] = c0m; }
+                    if (s1 < qn) { sQEnt[w][32 + lane] = m1; sQCnt[w][32 + lane] = c1m; }
                     __syncwarp();
-                    qn -= 32;
+                    qn -= nb;
                     stage_batch(bt);
+                    left -= nb;
+                    if (left == 0) {
+                        end_segment();
+                        left = a.segment;
+                    }
                 }
             }
             if (qn > 0) {
@@ -839,23 +951,12 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
                 bt.set(lane < qn ? sQEnt[w][lane] : make_float4(0.f, 0.f, 0.f, 0.f), lane < qn ? sQCnt[w][lane] : 0,
                        lane);
                 stage_batch(bt);
+                left -= qn;
             }
             __syncwarp();   // sRun and the queue are rewritten for the next group
         }
-        const int padded = pad_sources<kSplit>(Af, Bf, nbuf, lane);
-        __syncwarp();
-        sum_buffer<NPOLY, kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, k);
-        inter += (unsigned long long)nbuf * ni;
-        staged += nbuf;
-        __syncwarp();
-        // the kSplit source slots of a target add up their compensated totals
-        float tx = k.sx - k.cx, ty = k.sy - k.cy, tz = k.sz - k.cz;
-#pragma unroll
-        for (int o = G; o < 32; o <<= 1) {
-            tx += __shfl_xor_sync(0xffffffffu, tx, o);
-            ty += __shfl_xor_sync(0xffffffffu, ty, o);
-            tz += __shfl_xor_sync(0xffffffffu, tz, o);
-        }
+        if (left < a.segment) end_segment();   // the last one, unless the entries just filled it
+        const float tx = fold.sx - fold.cx, ty = fold.sy - fold.cy, tz = fold.sz - fold.cz;
         if (hs == 0 && ti < ni) {
             const int64_t o = a.perm[i0 + ti];
             const float Gc = NPOLY == kInvDeg ? bx.inv_g : bx.c_g;
@@ -972,6 +1073,13 @@ static void pp_args(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, PPArg
     a.n_staged = reinterpret_cast<unsigned long long *>(work + 16);
     a.acc = d_acc;
     a.inverse = lv->poly_degree == kInvDeg;
+    a.segment = lv->segment;
+    a.n_tasks = pr ? static_cast<const int32_t *>(pr->order_temp.p) + 512 : nullptr;
+    a.tasks = pr ? pr->tasks : nullptr;
+    a.task_done = pr ? pr->task_done : nullptr;
+    a.task_part = pr ? pr->task_part : nullptr;
+    a.split_of = pr ? pr->split_of : nullptr;
+    a.task_cap = pr ? pr->task_cap : 0;
 }
 
 template <bool kLearned, int kMinBlocks, int kSplit, bool kUniform>
