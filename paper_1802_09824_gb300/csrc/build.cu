@@ -96,7 +96,7 @@ __device__ __forceinline__ void wrapped_pos(const void *pos, int64_t i, const Bo
 
 template <int kPosType>
 __global__ void k_keys(const void *pos, int64_t n, const int32_t *box_first, int nb, const BoxDev *boxes, int T,
-                       int key_kind, uint64_t *keys, int32_t *vals, uint32_t *status)
+                       int key_kind, uint64_t *keys, int32_t *vals, SortCounts sc, uint32_t *status)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int bi = nb > 1 ? find_box(box_first, nb, i) : 0;
@@ -114,8 +114,10 @@ __global__ void k_keys(const void *pos, int64_t n, const int32_t *box_first, int
         uint64_t local = key_kind == PH_KEY_HILBERT ? hilbert3(qx & lm, qy & lm, qz & lm, b)
                                                     : interleave3(qx & lm, qy & lm, qz & lm);
         uint64_t boxbits = 3 * T < 64 ? ((uint64_t)bi << (3 * T)) : 0ull;
-        keys[i] = boxbits | (ground << (3 * b)) | local;
+        const uint64_t key = boxbits | (ground << (3 * b)) | local;
+        keys[i] = key;
         vals[i] = (int32_t)i;
+        atomicAdd(sc.hist + (int64_t)(key & ((1u << kSortBits) - 1u)) * sc.row + (i >> sc.tile_shift), 1);
     }
 }
 
@@ -605,19 +607,22 @@ int build_leaves_device(ph_leaves *h, const void *pos, int pos_type, const float
     uint64_t *keys = static_cast<uint64_t *>(h->keys.p);
     int32_t *vals = static_cast<int32_t *>(h->vals.p);
     if (n > 0) {
+        int rc = sort_begin(n, h->temp.p, s);
+        if (rc) return rc;
+        const SortCounts sc = sort_counts(n, h->temp.p);
         if (pos_type == PH_F64)
             k_keys<PH_F64><<<grid_for(n), kThreads, 0, s>>>(pos, n, box_first, nb, boxes, T, h->key_kind, keys, vals,
-                                                            status);
+                                                            sc, status);
         else
             k_keys<PH_F32><<<grid_for(n), kThreads, 0, s>>>(pos, n, box_first, nb, boxes, T, h->key_kind, keys, vals,
-                                                            status);
+                                                            sc, status);
         count_launch();
         bool alt = false;
         int box_bits = 0;
         while ((1 << box_bits) < nb) box_bits++;
         int bits = 3 * T + box_bits;
         bits = (bits + kSortBits - 1) / kSortBits * kSortBits;
-        int rc = radix_sort_pairs(keys, vals, static_cast<uint64_t *>(h->keys_alt.p),
+        rc = radix_sort_pairs(keys, vals, static_cast<uint64_t *>(h->keys_alt.p),
                                   static_cast<int32_t *>(h->vals_alt.p), n, bits, h->temp.p, s, &alt);
         if (rc) return rc;
         h->keys_in_alt = alt;

@@ -205,7 +205,15 @@ int segment_entries(int64_t n, int leaf_max, int group_size);
 inline int64_t task_bound(int64_t capacity, int segment) { return 2 * (capacity / segment) + 2; }
 
 // sort.cu: stable LSD radix sort of (key, value) pairs on the low `bits` bits.
+// The caller clears the digit counts (sort_begin) and counts each key's lowest
+// digit d at hist[d * row + (index >> tile_shift)] as it writes the keys.
+struct SortCounts {
+    int32_t *hist;
+    int row, tile_shift;
+};
 size_t sort_temp_bytes(int64_t n);
+SortCounts sort_counts(int64_t n, void *temp);
+int sort_begin(int64_t n, void *temp, cudaStream_t s);
 int radix_sort_pairs(uint64_t *keys, int32_t *vals, uint64_t *keys_alt, int32_t *vals_alt, int64_t n, int bits,
                      void *temp, cudaStream_t s, bool *result_in_alt);
 
