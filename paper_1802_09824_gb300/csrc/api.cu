@@ -285,8 +285,8 @@ uint64_t buffers_fingerprint(const ph_leaves *h, const ph_pairs *p)
 {
     uint64_t f = 1469598103934665603ull;
     const DevBuf *lb[] = {&h->boxes, &h->box_first, &h->keys, &h->keys_alt, &h->vals, &h->vals_alt, &h->xw,
-                          &h->mass_sorted, &h->cell_first, &h->leaf_flag, &h->group_flag, &h->leaf_scan,
-                          &h->group_scan, &h->leaf_first, &h->group_first, &h->leaf_ref, &h->leaf_c4, &h->leaf_h4,
+                          &h->mass_sorted, &h->cell_first, &h->starts, &h->leaf_of,
+                          &h->group_of, &h->leaf_first, &h->group_first, &h->leaf_ref, &h->leaf_c4, &h->leaf_h4,
                           &h->group_ref, &h->group_c4, &h->group_h4, &h->leaf_r4, &h->group_r4, &h->box_ext,
                           &h->work, &h->group_cell, &h->group_box, &h->pos_leaf, &h->pos_group,
                           &h->cell_leaf_first, &h->counts, &h->status, &h->temp, &h->group_act, &h->group_act_scan,
@@ -297,7 +297,7 @@ uint64_t buffers_fingerprint(const ph_leaves *h, const ph_pairs *p)
     }
     fp_mix(f, (uint64_t)h->n);
     if (p) {
-        const DevBuf *pb[] = {&p->group_cnt, &p->group_off, &p->entries, &p->ecount, &p->work, &p->status, &p->temp,
+        const DevBuf *pb[] = {&p->group_cnt, &p->group_off, &p->entries, &p->ecount, &p->work, &p->status,
                               &p->group_key, &p->group_order, &p->order_temp, &p->task_mem};
         for (const DevBuf *b : pb) {
             fp_mix(f, (uint64_t)(uintptr_t)b->p);
@@ -312,8 +312,8 @@ uint64_t buffers_fingerprint(const ph_leaves *h, const ph_pairs *p)
 static void free_leaves(ph_leaves *h)
 {
     DevBuf *bufs[] = {&h->boxes, &h->box_first, &h->in_pos, &h->in_mass, &h->keys, &h->keys_alt, &h->vals,
-                      &h->vals_alt, &h->xw, &h->mass_sorted, &h->cell_first, &h->leaf_flag, &h->group_flag,
-                      &h->leaf_scan, &h->group_scan, &h->leaf_first, &h->group_first, &h->leaf_ref, &h->leaf_c4,
+                      &h->vals_alt, &h->xw, &h->mass_sorted, &h->cell_first, &h->starts,
+                      &h->leaf_of, &h->group_of, &h->leaf_first, &h->group_first, &h->leaf_ref, &h->leaf_c4,
                       &h->leaf_h4, &h->group_ref, &h->group_c4, &h->group_h4, &h->leaf_r4, &h->group_r4, &h->box_ext, &h->work, &h->acc_tmp, &h->table, &h->group_cell, &h->group_box,
                       &h->pos_leaf, &h->pos_group, &h->cell_leaf_first, &h->counts, &h->status, &h->temp,
                       &h->group_act, &h->group_act_scan, &h->active_list};
@@ -322,7 +322,7 @@ static void free_leaves(ph_leaves *h)
 
 static void free_pairs(ph_pairs *h)
 {
-    DevBuf *bufs[] = {&h->group_cnt, &h->group_off, &h->entries, &h->ecount, &h->work, &h->status, &h->temp,
+    DevBuf *bufs[] = {&h->group_cnt, &h->group_off, &h->entries, &h->ecount, &h->work, &h->status,
                       &h->acc_tmp, &h->group_key, &h->group_order, &h->order_temp, &h->task_mem};
     for (DevBuf *b : bufs) release(*b);
 }
@@ -408,10 +408,9 @@ static int leaves_common(const void *pos, int pos_type, const float *mass, const
     ENS(h->xw, 24 * N);
     ENS(h->mass_sorted, 4 * N);
     ENS(h->cell_first, 4 * (size_t)(cells + 1));
-    ENS(h->leaf_flag, 4 * N);
-    ENS(h->group_flag, 4 * N);
-    ENS(h->leaf_scan, 4 * (N + 1));
-    ENS(h->group_scan, 4 * (N + 1));
+    ENS(h->starts, N);
+    ENS(h->leaf_of, 4 * N);
+    ENS(h->group_of, 4 * N);
     ENS(h->leaf_first, 4 * (N + 1));
     ENS(h->group_first, 4 * (N + 1));
     ENS(h->leaf_ref, 24 * N);
@@ -433,7 +432,7 @@ static int leaves_common(const void *pos, int pos_type, const float *mass, const
     ENS(h->status, 16);
     size_t tb = sort_temp_bytes(n);
     size_t ts = scan_temp_bytes(n);
-    ENS(h->temp, tb > ts ? tb : ts);
+    ENS(h->temp, std::max(std::max(tb, ts), build_temp_bytes()));
     if (h->active) {
         ENS(h->group_act, 4 * (N + 1));
         ENS(h->group_act_scan, 4 * (N + 1));
@@ -574,12 +573,11 @@ int ph_leaf_pairs(ph_leaves *leaves, void *stream, ph_pairs **pairs)
     if (!rc) rc = ensure(p->group_cnt, 8 * (N + 1));
     if (!rc) rc = ensure(p->group_off, 8 * (N + 1));
     if (!rc) rc = ensure(p->work, 64);
-    if (!rc) rc = ensure(p->temp, scan_temp_bytes((int64_t)N));
     if (!rc && leaves->queue_order == 0) {
         rc = ensure(p->group_key, N);
         if (!rc) rc = ensure(p->group_order, 4 * N);
     }
-    if (!rc) rc = ensure(p->order_temp, order_temp_bytes());
+    if (!rc) rc = ensure(p->order_temp, order_temp_bytes((int64_t)N));
     if (!rc && !p->status.p) {
         rc = ensure(p->status, 16);
         if (!rc) rc = cuda_check(cudaMemsetAsync(p->status.p, 0, 16, s), "status reset");

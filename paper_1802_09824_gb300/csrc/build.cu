@@ -121,30 +121,6 @@ __global__ void k_keys(const void *pos, int64_t n, const int32_t *box_first, int
     }
 }
 
-template <int kPosType>
-__global__ void k_gather(const void *pos, const float *mass, int64_t n, const uint64_t *keys, const int32_t *perm,
-                         const BoxDev *boxes, int T, double *xw, float *mass_sorted, uint32_t *status)
-{
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        int64_t i = perm[k];
-        if (!in_bounds(i, n, BS_BUILD_ROW)) i = 0;
-        const int bi = 3 * T < 64 ? (int)(keys[k] >> (3 * T)) : 0;
-        const BoxDev &bx = boxes[bi];
-        double x, y, z;
-        bool bad;
-        wrapped_pos<kPosType>(pos, i, bx, x, y, z, bad);
-        xw[3 * k + 0] = x;
-        xw[3 * k + 1] = y;
-        xw[3 * k + 2] = z;
-        float m = mass ? mass[i] : bx.mass_default;
-        if (!isfinite(m)) {
-            atomicOr(status, ST_NONFINITE);
-            m = 0.f;
-        }
-        mass_sorted[k] = m;
-    }
-}
-
 __device__ __forceinline__ int box_of_cell(const BoxDev *boxes, int nb, int c)
 {
     int lo = 0, hi = nb - 1;
@@ -164,27 +140,101 @@ __device__ __forceinline__ int64_t lower_bound_u64(const uint64_t *a, int64_t lo
     return lo;
 }
 
-__global__ void k_cell_first(const uint64_t *keys, int64_t n, const BoxDev *boxes, int nb, int n_cells, int T,
-                             int32_t *cell_first)
+// First particle of every ground cell (a search in the sorted keys).
+__device__ __forceinline__ void cell_starts(const uint64_t *keys, int64_t n, const BoxDev *boxes, int nb, int n_cells,
+                                            int T, int c, int32_t *cell_first)
 {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c <= n_cells; c += gridDim.x * blockDim.x) {
-        if (c == n_cells) {
-            cell_first[c] = (int32_t)n;
-            continue;
-        }
-        const int bi = box_of_cell(boxes, nb, c);
+    if (c >= n_cells) {
+        if (c == n_cells) cell_first[c] = (int32_t)n;
+        return;
+    }
+    const int bi = box_of_cell(boxes, nb, c);
+    const BoxDev &bx = boxes[bi];
+    const uint64_t boxbits = 3 * T < 64 ? ((uint64_t)bi << (3 * T)) : 0ull;
+    const uint64_t pre = boxbits | ((uint64_t)(c - bx.cell_base) << (3 * bx.b));
+    cell_first[c] = (int32_t)lower_bound_u64(keys, bx.first, (int64_t)bx.first + bx.n, pre);
+}
+
+// The particles in sorted order, wrapped, and (the last blocks, one thread a
+// cell) the first particle of every ground cell: both read only the sorted
+// keys and rows, so they share a launch.
+template <int kPosType>
+__global__ void k_gather(const void *pos, const float *mass, int64_t n, const uint64_t *keys, const int32_t *perm,
+                         const BoxDev *boxes, int T, double *xw, float *mass_sorted, uint32_t *status, int cell_blocks,
+                         int nb, int n_cells, int32_t *cell_first)
+{
+    const int blocks = (int)gridDim.x - cell_blocks;
+    if ((int)blockIdx.x >= blocks) {
+        cell_starts(keys, n, boxes, nb, n_cells, T, ((int)blockIdx.x - blocks) * (int)blockDim.x + (int)threadIdx.x,
+                    cell_first);
+        return;
+    }
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)blocks * blockDim.x) {
+        int64_t i = perm[k];
+        if (!in_bounds(i, n, BS_BUILD_ROW)) i = 0;
+        const int bi = 3 * T < 64 ? (int)(keys[k] >> (3 * T)) : 0;
         const BoxDev &bx = boxes[bi];
-        const uint64_t boxbits = 3 * T < 64 ? ((uint64_t)bi << (3 * T)) : 0ull;
-        const uint64_t pre = boxbits | ((uint64_t)(c - bx.cell_base) << (3 * bx.b));
-        cell_first[c] = (int32_t)lower_bound_u64(keys, bx.first, (int64_t)bx.first + bx.n, pre);
+        double x, y, z;
+        bool bad;
+        wrapped_pos<kPosType>(pos, i, bx, x, y, z, bad);
+        xw[3 * k + 0] = x;
+        xw[3 * k + 1] = y;
+        xw[3 * k + 2] = z;
+        float m = mass ? mass[i] : bx.mass_default;
+        if (!isfinite(m)) {
+            atomicOr(status, ST_NONFINITE);
+            m = 0.f;
+        }
+        mass_sorted[k] = m;
     }
 }
 
-// Leaf and group start flags (see the leaf rule in the file comment).
-__global__ void k_flags(const uint64_t *keys, int64_t n, const BoxDev *boxes, int T, int leaf_max, int level_bits,
-                        const int32_t *cell_first, int32_t *leaf_flag, int32_t *group_flag)
+// The leaves and groups are numbered in two passes over the particles, one
+// contiguous chunk a block: k_flags marks the starts (see the leaf rule in the
+// file comment) and counts them per chunk, k_starts adds up the counts of the
+// chunks before its own and numbers them.  Two launches where flags, two
+// three-kernel scans and a kernel for the first particles took eight (with the
+// merged launches below and k_offsets, per step: 1000 particles 187 -> 132 us,
+// 4096 102 -> 77 us, 50,021 472 -> 413 us, 128^3 lattice 4121 -> 4079 us).
+constexpr int kMaxChunks = 2048;
+
+struct Chunks {
+    int blocks;
+    int64_t size;            // particles a block, a multiple of kThreads
+};
+
+inline Chunks chunks_of(int64_t n)
 {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t tiles = (n + kThreads - 1) / kThreads;
+    const int64_t per = (tiles + kMaxChunks - 1) / kMaxChunks;
+    return Chunks{(int)((tiles + per - 1) / per), per * kThreads};
+}
+
+// Sums of two values over the block (every thread gets them).
+__device__ __forceinline__ int2 block_sum2(int a, int b)
+{
+    __shared__ int2 s_w[kThreads / 32];
+    a = __reduce_add_sync(0xffffffffu, a);
+    b = __reduce_add_sync(0xffffffffu, b);
+    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = make_int2(a, b);
+    __syncthreads();
+    int2 t = make_int2(0, 0);
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; w++) {
+        t.x += s_w[w].x;
+        t.y += s_w[w].y;
+    }
+    __syncthreads();
+    return t;
+}
+
+__global__ void __launch_bounds__(kThreads) k_flags(const uint64_t *keys, int64_t n, int64_t chunk, const BoxDev *boxes,
+                                                    int T, int leaf_max, int level_bits, const int32_t *cell_first,
+                                                    uint8_t *starts, int2 *chunk_count)
+{
+    const int64_t lo = blockIdx.x * chunk, end = lo + chunk < n ? lo + chunk : n;
+    int nl = 0, ngr = 0;
+    for (int64_t k = lo + threadIdx.x; k < end; k += kThreads) {
         const uint64_t Bk = keys[k];
         const int bi = 3 * T < 64 ? (int)(Bk >> (3 * T)) : 0;
         const BoxDev &bx = boxes[bi];
@@ -193,7 +243,7 @@ __global__ void k_flags(const uint64_t *keys, int64_t n, const BoxDev *boxes, in
         const int cell = bx.cell_base + (int)(cellpre & ((1ull << (3 * bx.g)) - 1ull));
         // target groups: runs of group_size inside each ground cell
         const int64_t cf = cell_first[cell];
-        group_flag[k] = ((k - cf) % bx.group_size) == 0 ? 1 : 0;
+        const int gf = (int)(k - cf) % bx.group_size == 0 ? 1 : 0;
         int lf;
         if (k == 0) {
             lf = 1;
@@ -237,38 +287,79 @@ __global__ void k_flags(const uint64_t *keys, int64_t n, const BoxDev *boxes, in
                 }
             }
         }
-        leaf_flag[k] = lf;
+        starts[k] = (uint8_t)(lf | (gf << 1));
+        nl += lf;
+        ngr += gf;
+    }
+    const int2 t = block_sum2(nl, ngr);
+    if (threadIdx.x == 0) chunk_count[blockIdx.x] = t;
+}
+
+// The leaf and the group of every particle, the first particle of every leaf
+// and group, and their numbers; also resets the boxes' extent accumulators
+// (ordered-integer min and max per axis) for k_extents.
+__device__ __forceinline__ void reset_extent(long long *e)
+{
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        e[d] = LLONG_MAX;
+        e[3 + d] = LLONG_MIN;
     }
 }
 
-// First particle of every leaf and every group; also resets the boxes'
-// extent accumulators (ordered-integer min and max per axis) for k_extents.
-__global__ void k_firsts(const int32_t *lflag, const int32_t *lscan, const int32_t *gflag, const int32_t *gscan,
-                         int64_t n, int32_t *lfirst, int32_t *gfirst, long long *lext, long long *gext)
+__global__ void __launch_bounds__(kThreads) k_starts(const uint8_t *starts, int64_t n, int64_t chunk,
+                                                     const int2 *chunk_count, int32_t *leaf_of, int32_t *group_of,
+                                                     int32_t *lfirst, int32_t *gfirst, long long *lext,
+                                                     long long *gext, int32_t *counts)
 {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        if (lflag[k] && in_bounds(lscan[k], n, BS_BUILD_ROW)) {
-            const int64_t l = lscan[k];
-            lfirst[l] = (int32_t)k;
+    __shared__ int2 s_w[2][kThreads / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned le = 0xffffffffu >> (31 - lane);
+    int2 run = make_int2(0, 0);
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kThreads) {
+        const int2 c = chunk_count[b];
+        run.x += c.x;
+        run.y += c.y;
+    }
+    run = block_sum2(run.x, run.y);   // starts before this chunk
+    const int64_t lo = blockIdx.x * chunk, end = lo + chunk < n ? lo + chunk : n;
+    for (int64_t base = lo; base < end; base += kThreads) {
+        const int64_t k = base + threadIdx.x;
+        const int f = k < end ? starts[k] : 0;
+        const unsigned lb = __ballot_sync(0xffffffffu, f & 1), gb = __ballot_sync(0xffffffffu, f & 2);
+        int2 *sw = s_w[((base - lo) / kThreads) & 1];   // alternating, so one barrier a tile
+        if (lane == 0) sw[w] = make_int2(__popc(lb), __popc(gb));
+        __syncthreads();
+        int2 at = run;
 #pragma unroll
-            for (int d = 0; d < 3; d++) {
-                lext[6 * l + d] = LLONG_MAX;
-                lext[6 * l + 3 + d] = LLONG_MIN;
+        for (int ww = 0; ww < kThreads / 32; ww++) {
+            const int2 c = sw[ww];
+            if (ww < w) {
+                at.x += c.x;
+                at.y += c.y;
+            }
+            run.x += c.x;
+            run.y += c.y;
+        }
+        if (k < end) {
+            const int l = at.x + __popc(lb & le) - 1, g = at.y + __popc(gb & le) - 1;
+            leaf_of[k] = l;
+            group_of[k] = g;
+            if ((f & 1) && in_bounds(l, n, BS_BUILD_ROW)) {
+                lfirst[l] = (int32_t)k;
+                reset_extent(lext + 6 * (int64_t)l);
+            }
+            if ((f & 2) && in_bounds(g, n, BS_BUILD_ROW)) {
+                gfirst[g] = (int32_t)k;
+                reset_extent(gext + 6 * (int64_t)g);
             }
         }
-        if (gflag[k] && in_bounds(gscan[k], n, BS_BUILD_ROW)) {
-            const int64_t l = gscan[k];
-            gfirst[l] = (int32_t)k;
-#pragma unroll
-            for (int d = 0; d < 3; d++) {
-                gext[6 * l + d] = LLONG_MAX;
-                gext[6 * l + 3 + d] = LLONG_MIN;
-            }
-        }
-        if (k == n - 1) {
-            lfirst[lscan[n]] = (int32_t)n;
-            gfirst[gscan[n]] = (int32_t)n;
-        }
+    }
+    if (end == n && threadIdx.x == 0) {
+        lfirst[run.x] = (int32_t)n;
+        gfirst[run.y] = (int32_t)n;
+        counts[0] = run.x;
+        counts[1] = run.y;
     }
 }
 
@@ -318,7 +409,7 @@ __device__ __forceinline__ void segment_extent(const long long v[3], int l, int 
     }
 }
 
-__global__ void k_extents(const double *xw, int64_t n, const int32_t *lscan, const int32_t *gscan, long long *lext,
+__global__ void k_extents(const double *xw, int64_t n, const int32_t *leaf_of, const int32_t *group_of, long long *lext,
                           long long *gext)
 {
     const int lane = threadIdx.x & 31;
@@ -329,8 +420,8 @@ __global__ void k_extents(const double *xw, int64_t n, const int32_t *lscan, con
         long long v[3];
 #pragma unroll
         for (int d = 0; d < 3; d++) v[d] = in ? dkey(xw[3 * k + d]) : 0;
-        segment_extent(v, in ? lscan[k + 1] - 1 : -1, lane, lext);
-        segment_extent(v, in ? gscan[k + 1] - 1 : -1, lane, gext);
+        segment_extent(v, in ? leaf_of[k] : -1, lane, lext);
+        segment_extent(v, in ? group_of[k] : -1, lane, gext);
     }
 }
 
@@ -345,12 +436,24 @@ __global__ void k_extents(const double *xw, int64_t n, const int32_t *lscan, con
 // is done as (c + 1.5 2^52 U) - 1.5 2^52 U (round half to even).  Being a
 // multiple of U below 2^e in magnitude, it is itself an FP32 number: r4
 // holds that exact FP32 copy.
-__global__ void k_boxes(const int32_t *first, const int32_t *scan_total, const long long *ext, const uint64_t *keys,
-                        const BoxDev *boxes, int T, double *ref, float4 *r4, float4 *c4, float4 *h4,
-                        int32_t *cell_of, int32_t *box_of)
+struct BoxTable {
+    const int32_t *first, *count;
+    const long long *ext;
+    double *ref;
+    float4 *r4, *c4, *h4;
+    int32_t *cell_of, *box_of;   // groups only
+};
+
+__device__ __forceinline__ void make_boxes(const BoxTable &t, const uint64_t *keys, const BoxDev *boxes, int T, int l0,
+                                           int step)
 {
-    const int count = *scan_total;
-    for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < count; l += gridDim.x * blockDim.x) {
+    const int32_t *first = t.first;
+    const long long *ext = t.ext;
+    double *ref = t.ref;
+    float4 *r4 = t.r4, *c4 = t.c4, *h4 = t.h4;
+    int32_t *cell_of = t.cell_of, *box_of = t.box_of;
+    const int count = *t.count;
+    for (int l = l0; l < count; l += step) {
         long long lo[3], hi[3];
 #pragma unroll
         for (int d = 0; d < 3; d++) {
@@ -387,15 +490,34 @@ __global__ void k_boxes(const int32_t *first, const int32_t *scan_total, const l
     }
 }
 
+// The boxes of the leaves (the first `blocks` blocks) and of the groups (the
+// next), and the first leaf of every ground cell (the rest): independent of
+// each other, one launch.  A cell's first particle starts a leaf; an empty
+// cell takes the next cell's.
+__global__ void k_boxes(BoxTable leaves, BoxTable groups, int blocks, const uint64_t *keys, const BoxDev *boxes, int T,
+                        int64_t n, const int32_t *cell_first, const int32_t *leaf_of, int n_cells,
+                        int32_t *cell_leaf_first)
+{
+    const int b = blockIdx.x, t = threadIdx.x;
+    if (b < blocks) {
+        make_boxes(leaves, keys, boxes, T, b * blockDim.x + t, blocks * blockDim.x);
+    } else if (b < 2 * blocks) {
+        make_boxes(groups, keys, boxes, T, (b - blocks) * blockDim.x + t, blocks * blockDim.x);
+    } else {
+        const int c = (b - 2 * blocks) * blockDim.x + t;
+        if (c <= n_cells) cell_leaf_first[c] = cell_first[c] < n ? leaf_of[cell_first[c]] : *leaves.count;
+    }
+}
+
 // Tree part (theta > 0): one particle per leaf carrying the leaf's mass at
 // its mass centre, sum(m x) / sum(m) over the leaf's wrapped positions in
 // FP64 (summed in particle order), stored after the N particles of pos_leaf
 // relative to the leaf's reference point like the leaf's own particles.  A
 // massless leaf keeps its reference point.
-__global__ void k_leaf_mass(const int32_t *first, const int32_t *scan_total, const double *xw, const float *mass,
+__global__ void k_leaf_mass(const int32_t *first, const int32_t *n_leaves, const double *xw, const float *mass,
                             const double *ref, int64_t n, float4 *pos_leaf)
 {
-    const int count = *scan_total;
+    const int count = *n_leaves;
     for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < count; l += gridDim.x * blockDim.x) {
         const int a = first[l], e = first[l + 1];
         double M = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
@@ -418,13 +540,13 @@ __global__ void k_leaf_mass(const int32_t *first, const int32_t *scan_total, con
     }
 }
 
-__global__ void k_pos(int64_t n, const double *xw, const float *mass_sorted, const int32_t *leaf_scan,
-                      const int32_t *group_scan, const double *leaf_ref, const float4 *leaf_r4, const float4 *group_r4,
+__global__ void k_pos(int64_t n, const double *xw, const float *mass_sorted, const int32_t *leaf_of,
+                      const int32_t *group_of, const double *leaf_ref, const float4 *leaf_r4, const float4 *group_r4,
                       float4 *pos_leaf, float4 *pos_group)
 {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        int64_t l = leaf_scan[k + 1] - 1;
-        int64_t g = group_scan[k + 1] - 1;
+        int64_t l = leaf_of[k];
+        int64_t g = group_of[k];
         if (!in_bounds(l, n, BS_BUILD_ROW)) l = 0;
         if (!in_bounds(g, n, BS_BUILD_ROW)) g = 0;
         const float4 lr4 = leaf_r4[l], gr4 = group_r4[g];
@@ -442,13 +564,6 @@ __global__ void k_pos(int64_t n, const double *xw, const float *mass_sorted, con
         pos_leaf[k] = make_float4(p[0], p[1], p[2], m);
         pos_group[k] = make_float4(q[0], q[1], q[2], m);
     }
-}
-
-__global__ void k_cell_leaf_first(const int32_t *cell_first, const int32_t *leaf_scan, int n_cells,
-                                  int32_t *cell_leaf_first)
-{
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c <= n_cells; c += gridDim.x * blockDim.x)
-        cell_leaf_first[c] = leaf_scan[cell_first[c]];
 }
 
 inline int grid_for(int64_t n, int threads = kThreads, int cap = 152 * 16)
@@ -594,6 +709,8 @@ void fit_inverse_form(BoxDev &bx, double G, double rcut, double rs)
     bx.inv_g = (float)(-G * s2 / mk);
 }
 
+size_t build_temp_bytes() { return kMaxChunks * sizeof(int2); }
+
 // Enqueue the whole leaf/group build for the particles already in device
 // memory (pos, mass).  The handle's box table and buffers are set up.
 int build_leaves_device(ph_leaves *h, const void *pos, int pos_type, const float *mass, cudaStream_t s)
@@ -634,71 +751,62 @@ int build_leaves_device(ph_leaves *h, const void *pos, int pos_type, const float
     double *xw = static_cast<double *>(h->xw.p);
     float *ms = static_cast<float *>(h->mass_sorted.p);
     int32_t *cell_first = static_cast<int32_t *>(h->cell_first.p);
-    int32_t *lflag = static_cast<int32_t *>(h->leaf_flag.p), *gflag = static_cast<int32_t *>(h->group_flag.p);
-    int32_t *lscan = static_cast<int32_t *>(h->leaf_scan.p), *gscan = static_cast<int32_t *>(h->group_scan.p);
-    if (n > 0)
-        if (pos_type == PH_F64)
-            k_gather<PH_F64><<<grid_for(n), kThreads, 0, s>>>(pos, mass, n, sk, perm, boxes, T, xw, ms, status);
-        else
-            k_gather<PH_F32><<<grid_for(n), kThreads, 0, s>>>(pos, mass, n, sk, perm, boxes, T, xw, ms, status);
-        count_launch();
-    k_cell_first<<<grid_for(h->n_cells + 1), kThreads, 0, s>>>(sk, n, boxes, nb, h->n_cells, T, cell_first);
-    count_launch();
-    if (n > 0)
-        k_flags<<<grid_for(n), kThreads, 0, s>>>(sk, n, boxes, T, h->max_leaf, h->level_bits, cell_first, lflag,
-                                                 gflag);
-        count_launch();
-    int rc = scan_exclusive_i32(lflag, lscan, n, nullptr, h->temp.p, s);
-    if (rc) return rc;
-    rc = scan_exclusive_i32(gflag, gscan, n, nullptr, h->temp.p, s);
-    if (rc) return rc;
+    int32_t *cell_leaf_first = static_cast<int32_t *>(h->cell_leaf_first.p);
     int32_t *lfirst = static_cast<int32_t *>(h->leaf_first.p), *gfirst = static_cast<int32_t *>(h->group_first.p);
+    int32_t *cnt = static_cast<int32_t *>(h->counts.p);   // leaves, groups, active groups
+    if (n == 0) {
+        // no particles: no leaves, no groups, every cell empty
+        int rc = cuda_check(cudaMemsetAsync(cnt, 0, 2 * sizeof(int32_t), s), "clear counts");
+        if (!rc) rc = cuda_check(cudaMemsetAsync(lfirst, 0, sizeof(int32_t), s), "clear leaves");
+        if (!rc) rc = cuda_check(cudaMemsetAsync(gfirst, 0, sizeof(int32_t), s), "clear groups");
+        if (!rc) rc = cuda_check(cudaMemsetAsync(cell_first, 0, 4 * (size_t)(h->n_cells + 1), s), "clear cells");
+        if (!rc) rc = cuda_check(cudaMemsetAsync(cell_leaf_first, 0, 4 * (size_t)(h->n_cells + 1), s), "clear cells");
+        return rc;
+    }
+    const int cell_blocks = (h->n_cells + kThreads) / kThreads;   // one thread a cell, and one for the end
+    if (pos_type == PH_F64)
+        k_gather<PH_F64><<<grid_for(n) + cell_blocks, kThreads, 0, s>>>(pos, mass, n, sk, perm, boxes, T, xw, ms, status,
+                                                                       cell_blocks, nb, h->n_cells, cell_first);
+    else
+        k_gather<PH_F32><<<grid_for(n) + cell_blocks, kThreads, 0, s>>>(pos, mass, n, sk, perm, boxes, T, xw, ms, status,
+                                                                       cell_blocks, nb, h->n_cells, cell_first);
+    count_launch();
+    const Chunks ch = chunks_of(n);
+    uint8_t *starts = static_cast<uint8_t *>(h->starts.p);
+    int2 *chunk_count = static_cast<int2 *>(h->temp.p);   // (the sort is done with it)
+    k_flags<<<ch.blocks, kThreads, 0, s>>>(sk, n, ch.size, boxes, T, h->max_leaf, h->level_bits, cell_first, starts,
+                                           chunk_count);
+    count_launch();
+    int32_t *leaf_of = static_cast<int32_t *>(h->leaf_of.p), *group_of = static_cast<int32_t *>(h->group_of.p);
     long long *lext = static_cast<long long *>(h->box_ext.p), *gext = lext + 6 * (size_t)n;
-    // first particles (and extent reset), extents, then the boxes of leaves and groups
-    if (n > 0) {
-        k_firsts<<<grid_for(n), kThreads, 0, s>>>(lflag, lscan, gflag, gscan, n, lfirst, gfirst, lext, gext);
-        count_launch();
-        k_extents<<<grid_for(n), kThreads, 0, s>>>(xw, n, lscan, gscan, lext, gext);
-        count_launch();
-    } else {
-        cudaMemsetAsync(lfirst, 0, sizeof(int32_t), s);
-        cudaMemsetAsync(gfirst, 0, sizeof(int32_t), s);
-    }
-    k_boxes<<<grid_for(n), kThreads, 0, s>>>(lfirst, lscan + n, lext, sk, boxes, T, static_cast<double *>(h->leaf_ref.p),
-                                             static_cast<float4 *>(h->leaf_r4.p), static_cast<float4 *>(h->leaf_c4.p),
-                                             static_cast<float4 *>(h->leaf_h4.p), nullptr, nullptr);
+    k_starts<<<ch.blocks, kThreads, 0, s>>>(starts, n, ch.size, chunk_count, leaf_of, group_of, lfirst, gfirst, lext,
+                                            gext, cnt);
     count_launch();
-    k_boxes<<<grid_for(n), kThreads, 0, s>>>(gfirst, gscan + n, gext, sk, boxes, T,
-                                             static_cast<double *>(h->group_ref.p),
-                                             static_cast<float4 *>(h->group_r4.p),
-                                             static_cast<float4 *>(h->group_c4.p),
-                                             static_cast<float4 *>(h->group_h4.p),
-                                             static_cast<int32_t *>(h->group_cell.p),
-                                             static_cast<int32_t *>(h->group_box.p));
+    k_extents<<<grid_for(n), kThreads, 0, s>>>(xw, n, leaf_of, group_of, lext, gext);
     count_launch();
-    if (n > 0 && h->tree_leaves) {
-        k_leaf_mass<<<grid_for(n), kThreads, 0, s>>>(lfirst, lscan + n, xw, ms, static_cast<const double *>(h->leaf_ref.p),
-                                                     n, static_cast<float4 *>(h->pos_leaf.p));
+    double *lref = static_cast<double *>(h->leaf_ref.p);
+    float4 *lr4 = static_cast<float4 *>(h->leaf_r4.p), *gr4 = static_cast<float4 *>(h->group_r4.p);
+    float4 *pos_leaf = static_cast<float4 *>(h->pos_leaf.p);
+    const BoxTable lt{lfirst, cnt, lext, lref, lr4, static_cast<float4 *>(h->leaf_c4.p),
+                      static_cast<float4 *>(h->leaf_h4.p), nullptr, nullptr};
+    const BoxTable gt{gfirst, cnt + 1, gext, static_cast<double *>(h->group_ref.p), gr4,
+                      static_cast<float4 *>(h->group_c4.p), static_cast<float4 *>(h->group_h4.p),
+                      static_cast<int32_t *>(h->group_cell.p), static_cast<int32_t *>(h->group_box.p)};
+    const int bb = grid_for(n, kThreads, 152 * 4);
+    k_boxes<<<2 * bb + cell_blocks, kThreads, 0, s>>>(lt, gt, bb, sk, boxes, T, n, cell_first, leaf_of, h->n_cells,
+                                                     cell_leaf_first);
+    count_launch();
+    if (h->tree_leaves) {
+        k_leaf_mass<<<grid_for(n), kThreads, 0, s>>>(lfirst, cnt, xw, ms, lref, n, pos_leaf);
         count_launch();
     }
-    if (n > 0)
-        k_pos<<<grid_for(n), kThreads, 0, s>>>(n, xw, ms, lscan, gscan, static_cast<const double *>(h->leaf_ref.p),
-                                               static_cast<const float4 *>(h->leaf_r4.p),
-                                               static_cast<const float4 *>(h->group_r4.p),
-                                               static_cast<float4 *>(h->pos_leaf.p),
-                                               static_cast<float4 *>(h->pos_group.p));
-        count_launch();
-    k_cell_leaf_first<<<grid_for(h->n_cells + 1), kThreads, 0, s>>>(cell_first, lscan, h->n_cells,
-                                                                    static_cast<int32_t *>(h->cell_leaf_first.p));
+    k_pos<<<grid_for(n), kThreads, 0, s>>>(n, xw, ms, leaf_of, group_of, lref, lr4, gr4, pos_leaf,
+                                           static_cast<float4 *>(h->pos_group.p));
     count_launch();
-    // device copies of the counts
-    int32_t *cnt = static_cast<int32_t *>(h->counts.p);
-    cudaMemcpyAsync(cnt + 0, lscan + n, sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
-    cudaMemcpyAsync(cnt + 1, gscan + n, sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
-    if (h->active && n > 0) {
+    int rc = 0;
+    if (h->active) {
         // the groups to sum in active-particle mode (buffers sized by the caller)
         int32_t *gact = static_cast<int32_t *>(h->group_act.p), *gacts = static_cast<int32_t *>(h->group_act_scan.p);
-        const int32_t *perm = static_cast<const int32_t *>(h->keys_in_alt ? h->vals_alt.p : h->vals.p);
         k_group_active<<<grid_for(n), kThreads, 0, s>>>(gfirst, cnt + 1, perm, h->active, gact);
         count_launch();
         rc = scan_exclusive_i32(gact, gacts, n, cnt + 1, h->temp.p, s);

@@ -37,8 +37,8 @@ struct ph_leaves {
     phpp::DevBuf xw;             // double[3n] wrapped positions in sorted order
     phpp::DevBuf mass_sorted;    // float[n]
     phpp::DevBuf cell_first;     // int32[n_cells + 1]
-    phpp::DevBuf leaf_flag, group_flag;   // int32[n]
-    phpp::DevBuf leaf_scan, group_scan;   // int32[n + 1]
+    phpp::DevBuf starts;         // uint8[n]: bit 0 starts a leaf, bit 1 a group
+    phpp::DevBuf leaf_of, group_of;       // int32[n]: leaf and group of every particle
     phpp::DevBuf leaf_first;     // int32[n + 1]
     phpp::DevBuf group_first;    // int32[n + 1]
     phpp::DevBuf leaf_ref;       // double[3 n]
@@ -90,13 +90,12 @@ struct ph_pairs {
     phpp::DevBuf ecount;         // uint8[capacity]: particles in the entry's leaf - 1
     phpp::DevBuf work;           // int32 queue counter + int64 work counters
     phpp::DevBuf status;         // uint32
-    phpp::DevBuf temp;
     phpp::DevBuf acc_tmp;        // float[3n] when the caller passes host memory
     // the PP queue's order (groups by decreasing cost), made by the count
     // pass when these buffers exist; `ordered` says the last list has it
     phpp::DevBuf group_key;      // uint8[n]: 255 - cost bucket
     phpp::DevBuf group_order;    // int32[n]: groups in queue order
-    phpp::DevBuf order_temp;     // int32[514]: groups per key, cursors, the number of tasks written and needed
+    phpp::DevBuf order_temp;     // groups per key, cursors, the number of tasks written and needed, entries per run of groups
     // groups with more than one segment are queued as one task per segment
     phpp::DevBuf task_mem;       // the four arrays below
     int2 *tasks = nullptr;       // [task_cap] (group, segment), a group's in a row; group -1: none

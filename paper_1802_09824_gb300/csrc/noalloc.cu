@@ -14,6 +14,7 @@
 // shadow symbol); its device address is looked up once per device with
 // cudaGetSymbolAddress, with that device current, on the first call made on
 // that device.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -91,10 +92,9 @@ void carve(Carver &c, ph_leaves &lv, ph_pairs &pr, int64_t n, int cells)
     c.take(lv.xw, 24 * N);
     c.take(lv.mass_sorted, 4 * N);
     c.take(lv.cell_first, 4 * (size_t)(cells + 1));
-    c.take(lv.leaf_flag, 4 * N);
-    c.take(lv.group_flag, 4 * N);
-    c.take(lv.leaf_scan, 4 * (N + 1));
-    c.take(lv.group_scan, 4 * (N + 1));
+    c.take(lv.starts, N);
+    c.take(lv.leaf_of, 4 * N);
+    c.take(lv.group_of, 4 * N);
     c.take(lv.leaf_first, 4 * (N + 1));
     c.take(lv.group_first, 4 * (N + 1));
     c.take(lv.group_h4, 16 * N);
@@ -114,25 +114,24 @@ void carve(Carver &c, ph_leaves &lv, ph_pairs &pr, int64_t n, int cells)
     c.take(lv.counts, 16);
     c.take(lv.status, 16);
     const size_t tsort = sort_temp_bytes(n), tscan = scan_temp_bytes(n);
-    c.take(lv.temp, tsort > tscan ? tsort : tscan);
+    c.take(lv.temp, std::max(std::max(tsort, tscan), build_temp_bytes()));
     c.take(pr.group_cnt, 8 * (N + 1));
     c.take(pr.group_off, 8 * (N + 1));
     c.take(pr.work, 64);
     c.take(pr.status, 16);
-    c.take(pr.temp, tscan);
     const size_t cap = (size_t)PH_NOALLOC_PAIRS_PER_PARTICLE * N;
     c.take(pr.entries, 16 * cap);
     c.take(pr.ecount, cap);
-    c.take(pr.order_temp, order_temp_bytes());
-    // the tasks of split groups: records and counters where the build's flags
+    c.take(pr.order_temp, order_temp_bytes(n));
+    // the tasks of split groups: records and counters where the sort's keys
     // were, sums where the boxes' tables and extents were (what the PP kernel
     // does not read)
     const size_t room = (size_t)((char *)lv.box_ext.p + lv.box_ext.bytes - (char *)lv.leaf_ref.p) / (96 * sizeof(float));
     pr.task_cap = (int64_t)(room < N / 2 ? room : N / 2);
-    pr.tasks = static_cast<int2 *>(lv.leaf_flag.p);
-    pr.task_done = static_cast<int32_t *>(lv.group_flag.p);
+    pr.tasks = static_cast<int2 *>(lv.keys.p);
+    pr.task_done = static_cast<int32_t *>(lv.keys_alt.p);
     pr.task_part = static_cast<float *>(lv.leaf_ref.p);
-    pr.split_of = static_cast<uint8_t *>(lv.group_scan.p);
+    pr.split_of = static_cast<uint8_t *>(lv.starts.p);
 }
 
 // Segment length of the step: twice segment_entries' (there are fewer task

@@ -59,6 +59,7 @@ struct PairArgs {
     int64_t cap;
     uint32_t *status;
     int32_t *n_tasks;        // tasks of split groups: [0] written by the fill pass, [1] needed (count pass)
+    unsigned long long *chunk_sum;   // entries of every kOffChunk groups (count pass)
     int2 *tasks;
     uint8_t *split_of;       // [n_groups]: whether a group of several segments has tasks
     int32_t *task_done;
@@ -87,6 +88,7 @@ __device__ __forceinline__ int warp_incl_scan_i(int v, int lane)
 // minus one (lanes with no leaves start no run).  Candidates keep the order
 // (neighbour, leaf), so the list is deterministic.
 constexpr int kOrdKeys = 256;   // queue keys (8 bits)
+constexpr int kOffChunk = 4 * kThreads;   // groups a block of k_offsets takes
 
 // Quarter-octave bucket of a cost: 0 for 0, else 1 + 4 e + f with e the
 // position of the leading bit and f the next two bits (1 .. 128).
@@ -273,6 +275,7 @@ __global__ void __launch_bounds__(kThreads) k_pairs(PairArgs a)
             const unsigned cost = __reduce_add_sync(0xffffffffu, src);
             if (lane == 0) {
                 a.cnt[g] = count;
+                atomicAdd(a.chunk_sum + g / kOffChunk, (unsigned long long)count);
                 if (count > a.segment) atomicAdd(a.n_tasks + 1, (int)((count + a.segment - 1) / a.segment));
                 if (a.gkey) {
                     const int k = 255 - cost_bucket(cost);
@@ -285,10 +288,61 @@ __global__ void __launch_bounds__(kThreads) k_pairs(PairArgs a)
     }
 }
 
+// The list's offsets: exclusive prefix of the groups' counts (off[n_groups]:
+// all entries), one block per kOffChunk groups; the chunks before its own it
+// adds up from the count pass's sums.
+__global__ void __launch_bounds__(kThreads) k_offsets(const int64_t *cnt, const int32_t *n_groups,
+                                                      const unsigned long long *chunk_sum, int64_t *off)
+{
+    __shared__ long long s_w[kThreads / 32];
+    const int ng = *n_groups, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int g0 = blockIdx.x * kOffChunk;
+    if (g0 > ng) return;
+    auto block_sum = [&](long long v) {   // over the block, every thread
+#pragma unroll
+        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) s_w[w] = v;
+        __syncthreads();
+        long long t = 0;
+#pragma unroll
+        for (int k = 0; k < kThreads / 32; k++) t += s_w[k];
+        __syncthreads();
+        return t;
+    };
+    long long mine = 0;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kThreads) mine += (long long)chunk_sum[b];
+    const long long before = block_sum(mine);
+    const int g = g0 + 4 * threadIdx.x;
+    long long v[4], t = 0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        v[k] = g + k < ng ? cnt[g + k] : 0;
+        t += v[k];
+    }
+    long long incl = t;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    if (lane == 31) s_w[w] = incl;
+    __syncthreads();
+    long long e = before + incl - t;
+#pragma unroll
+    for (int k = 0; k < kThreads / 32; k++) e += k < w ? s_w[k] : 0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        if (g + k <= ng) off[g + k] = e;
+        e += v[k];
+    }
+}
+
 }  // namespace
 
-// Scratch of the queue: the per-key counts and cursors, the number of tasks.
-size_t order_temp_bytes() { return (2 * kOrdKeys + 4) * sizeof(int32_t); }
+// Scratch of the queue: the per-key counts and cursors, the number of tasks;
+// then the chunk sums of k_offsets.
+constexpr int kOrdInts = 2 * kOrdKeys + 4;
+size_t order_temp_bytes(int64_t n) { return kOrdInts * sizeof(int32_t) + (n / kOffChunk + 2) * sizeof(int64_t); }
 
 // A warp sums a group's list segment by segment, and a group of several
 // segments is shared out to as many warps.  Without that, the longest list
@@ -409,6 +463,7 @@ int build_pairs_device(const ph_leaves *lv, ph_pairs *pr, cudaStream_t s, bool s
         lv->queue_order == 0 && !lv->active && pr->group_key.p && pr->group_order.p;
     int32_t *const ot = static_cast<int32_t *>(pr->order_temp.p);
     a.n_tasks = ot + 2 * kOrdKeys;
+    a.chunk_sum = reinterpret_cast<unsigned long long *>(ot + kOrdInts);
     a.segment = lv->segment;
     a.gkey = ordered ? static_cast<uint8_t *>(pr->group_key.p) : nullptr;
     a.ohist = ordered ? ot : nullptr;
@@ -424,14 +479,17 @@ int build_pairs_device(const ph_leaves *lv, ph_pairs *pr, cudaStream_t s, bool s
         if (rz) return rz;
     }
     {
-        const int rz = cuda_check(cudaMemsetAsync(ot, 0, order_temp_bytes(), s), "clear the queue's counts");
+        const int rz = cuda_check(cudaMemsetAsync(ot, 0, order_temp_bytes(n), s), "clear the queue's counts");
         if (rz) return rz;
     }
     k_pairs<false><<<grid, kThreads, 0, s>>>(a);
     count_launch();
-    int rc = scan_exclusive_i64(a.cnt, static_cast<int64_t *>(pr->group_off.p), n, n_all, pr->temp.p, s);
-    if (rc) return rc;
-    rc = fill_pairs(pr, a, n_all, grid, s, sizing_sync, n);
+    // at most one part-filled group a ground cell
+    const int64_t most = std::min<int64_t>(n, n / lv->group_size + lv->n_cells);
+    k_offsets<<<(int)(most / kOffChunk) + 1, kThreads, 0, s>>>(a.cnt, n_all, a.chunk_sum,
+                                                              static_cast<int64_t *>(pr->group_off.p));
+    count_launch();
+    int rc = fill_pairs(pr, a, n_all, grid, s, sizing_sync, n);
     if (rc) return rc;
     return cuda_check(cudaGetLastError(), "pair kernels");
 }

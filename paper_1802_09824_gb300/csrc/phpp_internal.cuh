@@ -189,12 +189,10 @@ void register_bounds_reader(int (*read)(unsigned int *hits, unsigned int *site))
 size_t scan_temp_bytes(int64_t max_n);
 int scan_exclusive_i32(const int32_t *in, int32_t *out, int64_t n, const int32_t *d_n, void *temp,
                        cudaStream_t s);
-int scan_exclusive_i64(const int64_t *in, int64_t *out, int64_t n, const int32_t *d_n, void *temp,
-                       cudaStream_t s);
 
-// pairs.cu: scratch of the PP queue (per-key counts and cursors, the number
-// of tasks of split groups).
-size_t order_temp_bytes();
+// pairs.cu: scratch of the pair passes for n particles (per-key counts and
+// cursors, the number of tasks of split groups, entries per run of groups).
+size_t order_temp_bytes(int64_t n);
 
 // pairs.cu: pair entries per segment of a group's source list for n particles,
 // a largest leaf and a group size: the PP sum of a group is the compensated sum of its
@@ -203,6 +201,9 @@ int segment_entries(int64_t n, int leaf_max, int group_size);
 
 // pairs.cu: task slots that a list of `capacity` entries can need at most.
 inline int64_t task_bound(int64_t capacity, int segment) { return 2 * (capacity / segment) + 2; }
+
+// build.cu: scratch of the leaf and group numbering.
+size_t build_temp_bytes();
 
 // sort.cu: stable LSD radix sort of (key, value) pairs on the low `bits` bits.
 // The caller clears the digit counts (sort_begin) and counts each key's lowest

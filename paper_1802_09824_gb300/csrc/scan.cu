@@ -140,9 +140,4 @@ int scan_exclusive_i32(const int32_t *in, int32_t *out, int64_t n, const int32_t
     return scan_impl<int32_t>(in, out, n, d_n, temp, s);
 }
 
-int scan_exclusive_i64(const int64_t *in, int64_t *out, int64_t n, const int32_t *d_n, void *temp, cudaStream_t s)
-{
-    return scan_impl<int64_t>(in, out, n, d_n, temp, s);
-}
-
 }  // namespace phpp
