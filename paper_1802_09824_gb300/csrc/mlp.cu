@@ -12,11 +12,15 @@
 // Validation evaluates the trained network exactly as the learned PP kernel
 // does (warp-level BF16 tensor-core MMAs) on a dense grid of r in [0, rcut)
 // and records the largest relative deviation from the exact factor.
+#include <algorithm>
 #include <cstdio>
+#include <type_traits>
 #include <cmath>
 #include <cstring>
 #include <new>
 #include <vector>
+
+#include <cooperative_groups.h>
 
 #include "factor.cuh"
 #include "handles.cuh"
@@ -33,6 +37,11 @@ namespace {
 constexpr int kTrainThreads = 128;
 constexpr int kTrainWarps = kTrainThreads / 32;
 constexpr int kGraphSteps = 64;
+// Largest batch of k_train_run: 16 SMs hold it, so a step grows with the batch
+// (512 steps: 2.5 ms at 300, 4.5 at 4096, 7.4 at 9000, 11.2 at 16,384), where
+// the gradient kernel spreads over all SMs (8.4, 8.9, 9.8 and 10.1 ms).
+constexpr int kRunBatch = 12288;
+constexpr int kRunSteps = 2048;     // steps a launch of k_train_run (~10 ms)
 constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
 
 __host__ __device__ __forceinline__ uint64_t splitmix64(uint64_t stream, uint64_t k)
@@ -226,6 +235,274 @@ __global__ void k_adam(AdamArgs a)
     }
     __syncthreads();
     if (e == 0) *a.step = step + 1;
+}
+
+// A run of training steps in one launch, by one thread-block cluster that
+// keeps the weights in shared memory.  A half-warp takes one sample at a time,
+// lane j the hidden units j of both layers: row and column j of W2 and the
+// gradients of row j stay in registers, the activations cross the lanes
+// through shared memory.  After a step's samples the blocks' gradient sums
+// are exchanged over distributed shared memory: each block adds up its share
+// of the parameters, applies Adam and writes the new weights into every
+// block.  Two cluster barriers a step instead of two dependent launches (a
+// gradient kernel and a one-block Adam kernel, 16.5 us a step at a batch of
+// 4096); now 7.8 us.  All sums run in a fixed order.  Bound by the latency
+// of a sample's chain (two exchanges, two 16-term sums, two sigmoids; 0.9 us
+// for two samples a half-warp) and of the barriers and the exchange of the
+// sums (4 us).
+namespace cg = cooperative_groups;
+constexpr int kRunThreads = 512;
+constexpr int kRunWarps = kRunThreads / 32;
+constexpr int kRunCluster = 16;
+constexpr int kRunSums = kMlpParams + 1;   // gradient, then the loss
+
+// Parameters in shared memory: the flat order with the rows of W2 20 floats
+// apart, so that 16 lanes read their rows as float4 without bank conflicts.
+constexpr int kRunFloats = kMlpParams + 64;
+__device__ __forceinline__ int run_at(int e) { return e < 32 ? e : e < 288 ? e + 4 * ((e - 32) >> 4) : e + 64; }
+
+struct RunArgs {
+    TrainArgs t;             // samples and streams (theta, step and partial unused)
+    AdamArgs a;              // parameters, moments, schedule (partial and step unused)
+    int step0, step1;        // the steps of this launch
+};
+
+__global__ void __launch_bounds__(kRunThreads, 1) k_train_run(RunArgs r)
+{
+    __shared__ __align__(16) float th[kRunFloats + 3];
+    __shared__ __align__(16) float s_part[kRunWarps][kRunFloats + 3];   // (run_at, then the loss)
+    __shared__ float s_sum[kRunSums];
+    __shared__ float s_m[kMlpParams], s_v[kMlpParams];      // (this block's share is used)
+    __shared__ __align__(16) float s_x[kRunWarps][2][2][2][16];
+    cg::cluster_group cl = cg::this_cluster();
+    const int nc = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = lane & 15, half = lane >> 4;
+    const int per = (kRunSums + nc - 1) / nc;                // parameters a block owns
+    for (int e = threadIdx.x; e < kMlpParams; e += kRunThreads) {
+        th[run_at(e)] = r.a.theta[e];
+        s_m[e] = r.a.m[e];
+        s_v[e] = r.a.v[e];
+    }
+    cl.sync();
+    const int nhw = nc * kRunWarps * 2;                      // half-warps of the cluster
+    const int hw = (rank * kRunWarps + w) * 2 + half;
+    const int iters = (r.t.batch + nhw - 1) / nhw;
+    const float batch_f = (float)r.t.batch;
+    // lane q of a half-warp holds the sample of its iteration it0 + q
+    auto fetch = [&](int step, int it0, float &z, float &tg) {
+        const int s = hw + (it0 + j) * nhw;
+        z = 0.f;
+        tg = 1.f;
+        if (it0 + j < iters && s < r.t.batch) {
+            const int64_t idx = (int64_t)(splitmix64(r.t.batch_stream, (uint64_t)step * (uint64_t)r.t.batch + (uint64_t)s) %
+                                          (uint64_t)r.t.n_samples);
+            z = r.t.z0[idx];
+            tg = r.t.tgt[idx];
+        }
+    };
+    float zq, tq;
+    fetch(r.step0, 0, zq, tq);
+    for (int step = r.step0; step < r.step1; step++) {
+        float row[16], col[16], g2[16];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const float4 v = *reinterpret_cast<const float4 *>(th + 32 + 20 * j + 4 * q);
+            row[4 * q] = v.x;
+            row[4 * q + 1] = v.y;
+            row[4 * q + 2] = v.z;
+            row[4 * q + 3] = v.w;
+        }
+#pragma unroll
+        for (int k = 0; k < 16; k++) {
+            col[k] = th[32 + 20 * k + j];
+            g2[k] = 0.f;
+        }
+        const float w1 = th[j], b1 = th[16 + j], b2 = th[352 + j], w3 = th[368 + j], b3 = th[384];
+        float gw1 = 0.f, gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f, loss = 0.f;
+        // kN samples at a time, so that one's exchanges run under the other's arithmetic
+        auto samples = [&](int it, auto count) {
+            constexpr int kN = decltype(count)::value;
+            float z[kN], a1[kN], s1[kN], a2[kN], s2[kN], dy[kN], h2[kN], d2[kN], hk[kN][16];
+#pragma unroll
+            for (int c = 0; c < kN; c++) {
+                z[c] = __shfl_sync(0xffffffffu, zq, (it + c) & 15, 16);
+                a1[c] = fmaf(w1, z[c], b1);
+                s1[c] = 1.f / (1.f + __expf(-a1[c]));
+                s_x[w][half][c][0][j] = a1[c] * s1[c];
+            }
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < kN; c++) {
+                const float4 *x = reinterpret_cast<const float4 *>(s_x[w][half][c][0]);
+                a2[c] = b2;
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const float4 v = x[q];
+                    hk[c][4 * q] = v.x;
+                    hk[c][4 * q + 1] = v.y;
+                    hk[c][4 * q + 2] = v.z;
+                    hk[c][4 * q + 3] = v.w;
+                }
+#pragma unroll
+                for (int k = 0; k < 16; k++) a2[c] = fmaf(row[k], hk[c][k], a2[c]);
+                s2[c] = 1.f / (1.f + __expf(-a2[c]));
+                h2[c] = a2[c] * s2[c];
+            }
+#pragma unroll
+            for (int c = 0; c < kN; c++) {
+                float y = w3 * h2[c];
+#pragma unroll
+                for (int o = 8; o; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+                y += b3;
+                const float tg = __shfl_sync(0xffffffffu, tq, (it + c) & 15, 16);
+                dy[c] = 0.f;
+                if (hw + (it + c) * nhw < r.t.batch) {
+                    const float rel = (y - tg) / tg;
+                    loss += rel * rel;
+                    dy[c] = 2.f * rel / tg / batch_f;
+                }
+                d2[c] = dy[c] * w3 * (s2[c] * (1.f + a2[c] * (1.f - s2[c])));
+                s_x[w][half][c][1][j] = d2[c];
+                gw3 = fmaf(dy[c], h2[c], gw3);
+                gb3 += dy[c];
+                gb2 += d2[c];
+#pragma unroll
+                for (int k = 0; k < 16; k++) g2[k] = fmaf(d2[c], hk[c][k], g2[k]);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < kN; c++) {
+                const float4 *x = reinterpret_cast<const float4 *>(s_x[w][half][c][1]);
+                float dh = 0.f;
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const float4 v = x[q];
+                    dh = fmaf(col[4 * q], v.x, dh);
+                    dh = fmaf(col[4 * q + 1], v.y, dh);
+                    dh = fmaf(col[4 * q + 2], v.z, dh);
+                    dh = fmaf(col[4 * q + 3], v.w, dh);
+                }
+                const float d1 = dh * (s1[c] * (1.f + a1[c] * (1.f - s1[c])));
+                gw1 = fmaf(d1, z[c], gw1);
+                gb1 += d1;
+            }
+            // (the next write of an activation follows every lane's read of
+            // this one by the second barrier, that of a gradient by the next first)
+        };
+        int it = 0;
+        for (; it + 2 <= iters; it += 2) {
+            if (it && (it & 15) == 0) fetch(step, it, zq, tq);
+            samples(it, std::integral_constant<int, 2>());
+        }
+        if (it < iters) {
+            if (it && (it & 15) == 0) fetch(step, it, zq, tq);
+            samples(it, std::integral_constant<int, 1>());
+        }
+        // the block's sums: the two halves of a warp, then the warps in order
+        auto halves = [&](float v) { return v + __shfl_xor_sync(0xffffffffu, v, 16); };
+#pragma unroll
+        for (int k = 0; k < 16; k++) g2[k] = halves(g2[k]);
+        gw1 = halves(gw1);
+        gb1 = halves(gb1);
+        gb2 = halves(gb2);
+        gw3 = halves(gw3);
+        gb3 = halves(gb3);
+        loss = halves(loss);
+        if (half == 0) {
+            float *p = s_part[w];
+            p[j] = gw1;
+            p[16 + j] = gb1;
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                *reinterpret_cast<float4 *>(p + 32 + 20 * j + 4 * q) =
+                    make_float4(g2[4 * q], g2[4 * q + 1], g2[4 * q + 2], g2[4 * q + 3]);
+            p[352 + j] = gb2;
+            p[368 + j] = gw3;
+            if (j == 0) {
+                p[384] = gb3;
+                p[385] = loss;
+            }
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < kRunSums; e += kRunThreads) {
+            float t = 0.f;
+#pragma unroll
+            for (int k = 0; k < kRunWarps; k++) t += s_part[k][run_at(e)];
+            s_sum[e] = t;
+        }
+        if (step + 1 < r.step1) fetch(step + 1, 0, zq, tq);   // (its loads run under the barriers)
+        const float t1 = (float)(step + 1);
+        const float c1 = 1.f - powf(r.a.b1, t1), c2 = 1.f - powf(r.a.b2, t1);
+        const float lr = r.a.lr_min + 0.5f * (r.a.lr0 - r.a.lr_min) *
+                                          (1.f + cosf(3.14159265358979f * (float)step / (float)max(r.a.steps, 1)));
+        cl.sync();
+        // this block's parameters: a half-warp each, lane q with block q's sum
+        for (int p0 = 2 * w; p0 < per; p0 += 2 * kRunWarps) {
+            const int p = p0 + half, e = rank * per + p;
+            const bool mine = p < per && e < kRunSums;
+            const bool par = mine && e < kMlpParams;
+            float g = mine && j < nc ? cl.map_shared_rank(s_sum, j)[e] : 0.f;
+            const float m0 = par ? s_m[e] : 0.f, v0 = par ? s_v[e] : 0.f, t0 = par ? th[run_at(e)] : 0.f;
+            __syncwarp();   // read by every lane before one of them writes
+#pragma unroll
+            for (int o = 8; o; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+            if (par) {
+                const float m = r.a.b1 * m0 + (1.f - r.a.b1) * g;
+                const float v = r.a.b2 * v0 + (1.f - r.a.b2) * g * g;
+                const float nt = t0 - lr * (m / c1) / (sqrtf(v / c2) + r.a.eps);
+                if (j == 0) {
+                    s_m[e] = m;
+                    s_v[e] = v;
+                }
+                if (j < nc) cl.map_shared_rank(th, j)[run_at(e)] = nt;
+            } else if (mine && j == 0 && r.a.loss_hist && step < r.a.steps) {
+                r.a.loss_hist[step] = g / (float)r.a.batch;
+            }
+        }
+        cl.sync();
+    }
+    for (int e = rank * per + threadIdx.x; e < min((rank + 1) * per, kMlpParams); e += kRunThreads) {
+        r.a.theta[e] = th[run_at(e)];
+        r.a.m[e] = s_m[e];
+        r.a.v[e] = s_v[e];
+    }
+}
+
+// Blocks of the cluster that k_train_run can be launched with (0: none).
+int train_cluster()
+{
+    cudaFuncSetAttribute(k_train_run, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int c : {kRunCluster, 8}) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(c);
+        cfg.blockDim = dim3(kRunThreads);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = c;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, k_train_run, &cfg) == cudaSuccess && fit > 0) return c;
+        cudaGetLastError();
+    }
+    return 0;
+}
+
+int launch_train_run(const RunArgs &r, int cluster, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cluster);
+    cfg.blockDim = dim3(kRunThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cluster;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    count_launch();
+    return cuda_check(cudaLaunchKernelEx(&cfg, k_train_run, r), "training run");
 }
 
 // Largest |g_hat / g - 1| over n_grid points r in [0, rcut), g_hat evaluated
@@ -488,8 +765,24 @@ int ph_mlp_train(const ph_train_params *tp, double rs, double rcut, const float 
     aa.eps = 1e-8f;
     aa.batch = tp->batch;
     aa.loss_hist = static_cast<float *>(h->loss_hist.p);
-    // a graph of kGraphSteps steps, replayed; the remainder launched directly
-    const int full = tp->steps / kGraphSteps, rest = tp->steps % kGraphSteps;
+    // batches up to kRunBatch: whole runs of steps by one cluster, at most
+    // kRunSteps a launch
+    int done = 0;
+    const int cluster = !rc && tp->batch <= kRunBatch ? train_cluster() : 0;
+    if (cluster > 0) {
+        for (; !rc && done < tp->steps; done += std::min(kRunSteps, tp->steps - done)) {
+            RunArgs r;
+            r.t = ta;
+            r.a = aa;
+            r.step0 = done;
+            r.step1 = done + std::min(kRunSteps, tp->steps - done);
+            rc = launch_train_run(r, cluster, s);
+        }
+        done = tp->steps;
+    }
+    // larger ones: a graph of kGraphSteps steps, replayed; the remainder
+    // launched directly
+    const int full = (tp->steps - done) / kGraphSteps, rest = (tp->steps - done) % kGraphSteps;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     if (!rc && full > 0) {
