@@ -4,7 +4,7 @@
 // of a pass's digits per tile are made by whoever writes its input: the
 // caller counts the first digit as it makes the keys, each pass counts the
 // next digit at the tile a key lands in (one L2 atomic a key).  A tile ranks
-// its keys stably (warp by warp, 32 keys at a time, with __match_any_sync),
+// its keys stably (warp by warp, 32 keys at a time),
 // reorders them by digit in shared memory and writes each digit's run after
 // the keys of earlier tiles, with consecutive threads on consecutive
 // positions.  The earlier tiles' counts it adds up itself (up to
@@ -12,7 +12,7 @@
 // the counts (k_digit_scan) that runs between the passes.
 // Bound by latency up to ~10^5 keys and by L2 traffic and atomics above.
 // Measured against one count, three scan and one scatter kernel a pass: a
-// pass of 4096 keys 27 -> 9 us, of 2 M keys 46 -> 33 us; per step, 1000
+// pass of 4096 keys 27 -> 9 us, of 2 M keys 46 -> 26 us; per step, 1000
 // particles 253 -> 187 us, 4096 140 -> 102 us, 50,021 552 -> 472 us.
 #include <algorithm>
 #include <utility>
@@ -27,6 +27,19 @@ constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kBins = 1 << kSortBits;
 constexpr int kDirectTiles = 64;
+
+// The lanes holding the same digit (0 .. kBins): one ballot a bit (a pass of
+// 2 M keys took 7 us longer with __match_any_sync).
+__device__ __forceinline__ unsigned same_digit(int d)
+{
+    unsigned m = 0xffffffffu;
+#pragma unroll
+    for (int b = 0; b <= kSortBits; b++) {
+        const unsigned set = __ballot_sync(0xffffffffu, (d >> b) & 1);
+        m &= (d >> b) & 1 ? set : ~set;
+    }
+    return m;
+}
 
 // Exclusive scan of one int per thread over the block.
 __device__ __forceinline__ int block_excl(int v, int *s_wsum)
@@ -89,7 +102,7 @@ template <int kItems, bool kDirect>
 __global__ void __launch_bounds__(kSortThreads) k_radix_pass(PassArgs a)
 {
     constexpr int kTile = kSortThreads * kItems;
-    __shared__ int32_t cnt[kSortWarps][kBins];
+    __shared__ uint16_t cnt[kSortWarps][kBins];   // (a tile has at most 2048 keys)
     __shared__ int32_t s_off[kBins];            // output position of the tile's first key of each digit
     __shared__ int32_t s_start[kBins];          // its first slot in the tile
     __shared__ int32_t s_wsum[kSortWarps];
@@ -135,12 +148,12 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_pass(PassArgs a)
     const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
     for (int r = 0; r < kItems; r++) {
-        const unsigned peers = __match_any_sync(0xffffffffu, d_[r]);
+        const unsigned peers = same_digit(d_[r]);
         const int leader = __ffs(peers) - 1;
         int old = 0;
         if (d_[r] < kBins && lane == leader) {
             old = cnt[w][d_[r]];
-            cnt[w][d_[r]] = old + __popc(peers);
+            cnt[w][d_[r]] = (uint16_t)(old + __popc(peers));
         }
         r_[r] = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & lt);
         __syncwarp();
@@ -153,7 +166,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_pass(PassArgs a)
 #pragma unroll
         for (int ww = 0; ww < kSortWarps; ww++) {
             const int c = cnt[ww][d];
-            cnt[ww][d] = run;
+            cnt[ww][d] = (uint16_t)run;
             run += c;
         }
         s_start[d] = block_excl(run, s_wsum);
