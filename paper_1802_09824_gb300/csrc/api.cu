@@ -242,6 +242,8 @@ void fill_box(BoxDev &bx, const ph_params &p, int key_bits, int poly_degree, int
     bx.b = key_bits - bx.g;
     bx.nside = 1 << bx.g;
     bx.S = std::ldexp(1.0, key_bits) / p.L;
+    bx.S_hi = (float)bx.S;
+    bx.S_lo = (float)(bx.S - (double)bx.S_hi);
     bx.h = p.L / bx.nside;
     set_softening(bx, p.G, p.eps, p.rcut);
     bx.rcut2 = (float)(p.rcut * p.rcut);
@@ -287,7 +289,7 @@ uint64_t buffers_fingerprint(const ph_leaves *h, const ph_pairs *p)
     const DevBuf *lb[] = {&h->boxes, &h->box_first, &h->keys, &h->keys_alt, &h->vals, &h->vals_alt, &h->xw,
                           &h->mass_sorted, &h->cell_first, &h->starts, &h->leaf_of,
                           &h->group_of, &h->leaf_first, &h->group_first, &h->leaf_ref, &h->leaf_c4, &h->leaf_h4,
-                          &h->group_ref, &h->group_c4, &h->group_h4, &h->leaf_r4, &h->group_r4, &h->box_ext,
+                          &h->group_ref, &h->group_c4, &h->group_h4, &h->leaf_r4, &h->group_r4,
                           &h->work, &h->group_cell, &h->group_box, &h->pos_leaf, &h->pos_group,
                           &h->cell_leaf_first, &h->counts, &h->status, &h->temp, &h->group_act, &h->group_act_scan,
                           &h->active_list};
@@ -314,7 +316,7 @@ static void free_leaves(ph_leaves *h)
     DevBuf *bufs[] = {&h->boxes, &h->box_first, &h->in_pos, &h->in_mass, &h->keys, &h->keys_alt, &h->vals,
                       &h->vals_alt, &h->xw, &h->mass_sorted, &h->cell_first, &h->starts,
                       &h->leaf_of, &h->group_of, &h->leaf_first, &h->group_first, &h->leaf_ref, &h->leaf_c4,
-                      &h->leaf_h4, &h->group_ref, &h->group_c4, &h->group_h4, &h->leaf_r4, &h->group_r4, &h->box_ext, &h->work, &h->acc_tmp, &h->table, &h->group_cell, &h->group_box,
+                      &h->leaf_h4, &h->group_ref, &h->group_c4, &h->group_h4, &h->leaf_r4, &h->group_r4, &h->work, &h->acc_tmp, &h->table, &h->group_cell, &h->group_box,
                       &h->pos_leaf, &h->pos_group, &h->cell_leaf_first, &h->counts, &h->status, &h->temp,
                       &h->group_act, &h->group_act_scan, &h->active_list};
     for (DevBuf *b : bufs) release(*b);
@@ -421,7 +423,6 @@ static int leaves_common(const void *pos, int pos_type, const float *mass, const
     ENS(h->group_h4, 16 * N);
     ENS(h->leaf_r4, 16 * N);
     ENS(h->group_r4, 16 * N);
-    ENS(h->box_ext, 96 * N);
     ENS(h->work, 64);
     ENS(h->group_cell, 4 * N);
     ENS(h->group_box, 4 * N);

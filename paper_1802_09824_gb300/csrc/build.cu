@@ -22,6 +22,7 @@
 // group, derived from the first by one FP32 add of the FP64-computed offset,
 // exactly as the PP kernel shifts source particles, so that a particle seen
 // as target and as source has bitwise the same coordinates.
+#include <algorithm>
 #include <climits>
 #include <cmath>
 
@@ -60,13 +61,55 @@ __device__ __forceinline__ uint32_t quant_coord(double xw, double S, int T)
     return (uint32_t)(q < 0 ? 0 : (q > top ? top : q));
 }
 
+// The widening of an FP32 number with integer operations (the FP64 pipe, which
+// conversions share, has two lanes an SM here; a subnormal still goes there).
+__device__ __forceinline__ double widen(float x)
+{
+    const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+    if (e == 0 && (b & 0x7fffffu)) return (double)x;
+    const uint32_t hi = (b & 0x80000000u) | (e ? ((e + 896u) << 20) | ((b & 0x7fffffu) >> 3) : 0u);
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+
+// The reverse where it is exact: true if x is a normal FP32 number or zero.
+__device__ __forceinline__ bool narrow(double x, float &f)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x), e = (hi >> 20) & 0x7ffu;
+    const bool zero = !((hi & 0x7fffffffu) | lo);
+    f = __uint_as_float((hi & 0x80000000u) | (zero ? 0u : ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29)));
+    return zero || (!(lo & 0x1fffffffu) && e >= 897u && e <= 1150u);
+}
+
 // Wrapped coordinate of an FP32 input: the in-box test runs in FP32 (x < L
 // exactly when x < L_up), so only the multiply of the key and the widening
 // to FP64 remain on the FP64 pipe for particles already in the box.
 __device__ __forceinline__ double wrap_f32(float x, const BoxDev &bx)
 {
-    if (x >= 0.f && x < bx.L_up) return (double)x;
+    if (x >= 0.f && x < bx.L_up) return widen(x);
     return wrap_coord((double)x, bx.L);
+}
+
+// quant_coord of an FP32 coordinate in [0, L) without FP64: x S as a
+// double-float product (the product's rounding error taken exactly by an FMA),
+// off by at most 2^-25 (S_lo's rounding and one FP32 rounding of the low
+// part, x S < 2^21).  The floor is taken from it when its fraction lies at
+// least 1e-6 off an integer, 40 times that, else the FP64 product decides
+// (false).
+__device__ __forceinline__ bool quant_f32(float x, const BoxDev &bx, int T, uint32_t &q)
+{
+    const float p = x * bx.S_hi;
+    const float lo = fmaf(x, bx.S_lo, fmaf(x, bx.S_hi, -p));
+    float fl = floorf(p), fr = (p - fl) + lo;
+    if (fr < 0.f) {
+        fr += 1.f;
+        fl -= 1.f;
+    } else if (fr >= 1.f) {
+        fr -= 1.f;
+        fl += 1.f;
+    }
+    const int i = (int)fl, top = (1 << T) - 1;
+    q = (uint32_t)(i < 0 ? 0 : (i > top ? top : i));
+    return fr >= 1e-6f && fr <= 1.f - 1e-6f;
 }
 
 // Particle i's coordinates wrapped into [0, L) in FP64 (non-finite input
@@ -101,13 +144,23 @@ __global__ void k_keys(const void *pos, int64_t n, const int32_t *box_first, int
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int bi = nb > 1 ? find_box(box_first, nb, i) : 0;
         const BoxDev &bx = boxes[bi];
-        double x, y, z;
-        bool bad;
-        wrapped_pos<kPosType>(pos, i, bx, x, y, z, bad);
-        if (bad) atomicOr(status, ST_NONFINITE);
-        const uint32_t qx = quant_coord(x, bx.S, T);
-        const uint32_t qy = quant_coord(y, bx.S, T);
-        const uint32_t qz = quant_coord(z, bx.S, T);
+        uint32_t qx = 0, qy = 0, qz = 0;
+        bool done = false;
+        if (kPosType == PH_F32) {
+            const float *p = static_cast<const float *>(pos) + 3 * i;
+            const float x = p[0], y = p[1], z = p[2];
+            done = x >= 0.f && x < bx.L_up && y >= 0.f && y < bx.L_up && z >= 0.f && z < bx.L_up;   // (NaN: no)
+            done = done && quant_f32(x, bx, T, qx) && quant_f32(y, bx, T, qy) && quant_f32(z, bx, T, qz);
+        }
+        if (!done) {
+            double x, y, z;
+            bool bad;
+            wrapped_pos<kPosType>(pos, i, bx, x, y, z, bad);
+            if (bad) atomicOr(status, ST_NONFINITE);
+            qx = quant_coord(x, bx.S, T);
+            qy = quant_coord(y, bx.S, T);
+            qz = quant_coord(z, bx.S, T);
+        }
         const int b = bx.b;
         const uint32_t lm = (1u << b) - 1u;
         uint64_t ground = ((uint64_t)(qx >> b) * bx.nside + (qy >> b)) * bx.nside + (qz >> b);
@@ -296,21 +349,10 @@ __global__ void __launch_bounds__(kThreads) k_flags(const uint64_t *keys, int64_
 }
 
 // The leaf and the group of every particle, the first particle of every leaf
-// and group, and their numbers; also resets the boxes' extent accumulators
-// (ordered-integer min and max per axis) for k_extents.
-__device__ __forceinline__ void reset_extent(long long *e)
-{
-#pragma unroll
-    for (int d = 0; d < 3; d++) {
-        e[d] = LLONG_MAX;
-        e[3 + d] = LLONG_MIN;
-    }
-}
-
+// and group, and their numbers.
 __global__ void __launch_bounds__(kThreads) k_starts(const uint8_t *starts, int64_t n, int64_t chunk,
                                                      const int2 *chunk_count, int32_t *leaf_of, int32_t *group_of,
-                                                     int32_t *lfirst, int32_t *gfirst, long long *lext,
-                                                     long long *gext, int32_t *counts)
+                                                     int32_t *lfirst, int32_t *gfirst, int32_t *counts)
 {
     __shared__ int2 s_w[2][kThreads / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -345,14 +387,8 @@ __global__ void __launch_bounds__(kThreads) k_starts(const uint8_t *starts, int6
             const int l = at.x + __popc(lb & le) - 1, g = at.y + __popc(gb & le) - 1;
             leaf_of[k] = l;
             group_of[k] = g;
-            if ((f & 1) && in_bounds(l, n, BS_BUILD_ROW)) {
-                lfirst[l] = (int32_t)k;
-                reset_extent(lext + 6 * (int64_t)l);
-            }
-            if ((f & 2) && in_bounds(g, n, BS_BUILD_ROW)) {
-                gfirst[g] = (int32_t)k;
-                reset_extent(gext + 6 * (int64_t)g);
-            }
+            if ((f & 1) && in_bounds(l, n, BS_BUILD_ROW)) lfirst[l] = (int32_t)k;
+            if ((f & 2) && in_bounds(g, n, BS_BUILD_ROW)) gfirst[g] = (int32_t)k;
         }
     }
     if (end == n && threadIdx.x == 0) {
@@ -375,60 +411,42 @@ __device__ __forceinline__ double dkey_inv(long long k)
     return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
 }
 
-// Per-axis extents of every leaf and every group, one thread per particle:
-// the particles of a box are consecutive, so a warp combines each box's part
-// of its 32 particles by a segmented reduction (shuffle down within runs of
-// the same box), and the first lane of each run folds that into the box's
-// accumulators with 64-bit atomic min/max (boxes may straddle warps).
-// Coordinates enter as ordered integers (dkey), so the integer order is the
-// FP64 order.
-__device__ __forceinline__ void segment_extent(const long long v[3], int l, int lane, long long *ext)
+// Smallest and largest of the lanes' values, 64-bit integers, by two 32-bit
+// warp reductions each: the high words, then the low words of those that hold
+// the extreme one.
+__device__ __forceinline__ long long warp_min(long long v)
 {
-    long long lo[3] = {v[0], v[1], v[2]}, hi[3] = {v[0], v[1], v[2]};
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int lo_l = __shfl_down_sync(0xffffffffu, l, o);
-        const bool same = lane + o < 32 && lo_l == l;
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-            const long long vl = __shfl_down_sync(0xffffffffu, lo[d], o);
-            const long long vh = __shfl_down_sync(0xffffffffu, hi[d], o);
-            if (same) {
-                lo[d] = vl < lo[d] ? vl : lo[d];
-                hi[d] = vh > hi[d] ? vh : hi[d];
-            }
-        }
-    }
-    const int prev = __shfl_up_sync(0xffffffffu, l, 1);
-    if (l >= 0 && (lane == 0 || prev != l)) {
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-            atomicMin(ext + 6 * (int64_t)l + d, lo[d]);
-            atomicMax(ext + 6 * (int64_t)l + 3 + d, hi[d]);
-        }
-    }
+    const int h = (int)(v >> 32), mh = __reduce_min_sync(0xffffffffu, h);
+    const unsigned ml = __reduce_min_sync(0xffffffffu, h == mh ? (unsigned)v : 0xffffffffu);
+    return ((long long)mh << 32) | ml;
 }
 
-__global__ void k_extents(const double *xw, int64_t n, const int32_t *leaf_of, const int32_t *group_of, long long *lext,
-                          long long *gext)
+__device__ __forceinline__ long long warp_max(long long v)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t k0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
-    for (int64_t base = k0; base < n; base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = base + lane;
-        const bool in = k < n;
-        long long v[3];
-#pragma unroll
-        for (int d = 0; d < 3; d++) v[d] = in ? dkey(xw[3 * k + d]) : 0;
-        segment_extent(v, in ? leaf_of[k] : -1, lane, lext);
-        segment_extent(v, in ? group_of[k] : -1, lane, gext);
-    }
+    const int h = (int)(v >> 32), mh = __reduce_max_sync(0xffffffffu, h);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, h == mh ? (unsigned)v : 0u);
+    return ((long long)mh << 32) | ml;
 }
 
-// Bounding box of each leaf (or group) from its extents, one thread per box:
-// FP64 reference point near the box centre, FP32 half extents around it
-// rounded up, FP32 reference point relative to the ground cell's lower
-// corner.
+struct BoxTable {
+    const int32_t *first, *count;
+    double *ref;
+    float4 *r4, *c4, *h4;
+    int32_t *cell_of, *box_of;   // groups only
+};
+
+struct FrameArgs {               // leaves only: the particles in their frames
+    const float *mass_sorted;
+    const int32_t *leaf_of, *group_of;
+    const float4 *group_r4;
+    float4 *pos_leaf, *pos_group;
+    int64_t n;
+};
+
+// Bounding box of each leaf (or group): FP64 reference point near the box
+// centre, FP32 half extents around it rounded up, FP32 reference point
+// relative to the ground cell's lower corner; and for the leaves the
+// particles' positions in their leaf's and group's frames.
 //
 // The reference point is the centre rounded to a multiple of U = 2^(e-24),
 // the FP32 spacing of the box's largest |coordinate| (2^(e-1) <= m < 2^e),
@@ -436,77 +454,159 @@ __global__ void k_extents(const double *xw, int64_t n, const int32_t *leaf_of, c
 // is done as (c + 1.5 2^52 U) - 1.5 2^52 U (round half to even).  Being a
 // multiple of U below 2^e in magnitude, it is itself an FP32 number: r4
 // holds that exact FP32 copy.
-struct BoxTable {
-    const int32_t *first, *count;
-    const long long *ext;
-    double *ref;
-    float4 *r4, *c4, *h4;
-    int32_t *cell_of, *box_of;   // groups only
-};
+//
+// A block takes kBoxes consecutive boxes: a warp reduces the extents of four
+// of them (coordinates as integers ordered like the doubles, dkey), then one
+// thread an axis does the FP64 arithmetic of all (a warp per box would spend
+// the narrow FP64 pipe on idle lanes), then the leaves' particles, one
+// contiguous run, are written in their frames.  An FP32 coordinate takes an
+// FP32 subtraction there: the difference of two FP32 numbers rounded once,
+// as the FP64 one rounded to FP32 is.  (Extents by segmented warp reductions
+// and global atomics, the boxes and the frames as three launches took 88 us
+// for 2 M particles, now 62 us; the 128^3 lattice step 4046 -> 4014 us.)
+constexpr int kBoxes = 32;
 
-__device__ __forceinline__ void make_boxes(const BoxTable &t, const uint64_t *keys, const BoxDev *boxes, int T, int l0,
-                                           int step)
+template <bool kLeaves>
+__device__ __forceinline__ void box_block(const BoxTable &t, const FrameArgs &fr, const uint64_t *keys,
+                                          const BoxDev *boxes, int T, const double *xw, int block, int blocks)
 {
-    const int32_t *first = t.first;
-    const long long *ext = t.ext;
-    double *ref = t.ref;
-    float4 *r4 = t.r4, *c4 = t.c4, *h4 = t.h4;
-    int32_t *cell_of = t.cell_of, *box_of = t.box_of;
+    __shared__ int s_first[kBoxes + 1];
+    __shared__ long long s_ext[kBoxes][6];
+    __shared__ float s_ref[kBoxes][3], s_c[kBoxes][3], s_h[kBoxes][3];
+    __shared__ double s_refd[kLeaves ? kBoxes : 1][3];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int count = *t.count;
-    for (int l = l0; l < count; l += step) {
-        long long lo[3], hi[3];
+    for (int l0 = block * kBoxes; l0 < count; l0 += blocks * kBoxes) {
+        const int nb = count - l0 < kBoxes ? count - l0 : kBoxes;
+        if (threadIdx.x <= nb) s_first[threadIdx.x] = t.first[l0 + threadIdx.x];
+        __syncthreads();
+        constexpr int kPer = kBoxes / (kThreads / 32);
+        // the first 32 particles of the warp's boxes in flight together
+        double x[kPer][3];
 #pragma unroll
-        for (int d = 0; d < 3; d++) {
-            lo[d] = ext[6 * (int64_t)l + d];
-            hi[d] = ext[6 * (int64_t)l + 3 + d];
+        for (int q = 0; q < kPer; q++) {
+            const int b = w * kPer + q;
+            const int k = b < nb ? s_first[b] + lane : 0;
+            const bool in = b < nb && k < s_first[b + 1];
+#pragma unroll
+            for (int d = 0; d < 3; d++) x[q][d] = in ? xw[3 * (int64_t)k + d] : 0.0;
         }
-        const uint64_t key = keys[first[l]];
-        const int bi = 3 * T < 64 ? (int)(key >> (3 * T)) : 0;
-        const BoxDev &bx = boxes[bi];
-        const uint32_t ground = (uint32_t)((key >> (3 * bx.b)) & ((1ull << (3 * bx.g)) - 1ull));
-        const uint32_t gz = ground % bx.nside, gy = (ground / bx.nside) % bx.nside, gx = ground / (bx.nside * bx.nside);
-        const uint32_t gc[3] = {gx, gy, gz};
-        float c[3], hh[3], rf[3];
 #pragma unroll
-        for (int d = 0; d < 3; d++) {
-            const double vlo = dkey_inv(lo[d]), vhi = dkey_inv(hi[d]);
+        for (int q = 0; q < kPer; q++) {
+            const int b = w * kPer + q;
+            if (b >= nb) break;
+            const int f1 = s_first[b + 1];
+            int k = s_first[b] + lane;
+            long long lo[3], hi[3];
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                lo[d] = k < f1 ? dkey(x[q][d]) : LLONG_MAX;
+                hi[d] = k < f1 ? lo[d] : LLONG_MIN;
+            }
+            for (k += 32; k < f1; k += 32)
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    const long long v = dkey(xw[3 * (int64_t)k + d]);
+                    lo[d] = v < lo[d] ? v : lo[d];
+                    hi[d] = v > hi[d] ? v : hi[d];
+                }
+            __syncwarp();
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                lo[d] = warp_min(lo[d]);
+                hi[d] = warp_max(hi[d]);
+            }
+            if (lane == 0) {
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    s_ext[b][d] = lo[d];
+                    s_ext[b][3 + d] = hi[d];
+                }
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x < 3 * nb) {
+            const int b = threadIdx.x / 3, d = threadIdx.x % 3;
+            const uint64_t key = keys[s_first[b]];
+            const int bi = 3 * T < 64 ? (int)(key >> (3 * T)) : 0;
+            const BoxDev &bx = boxes[bi];
+            const uint32_t ground = (uint32_t)((key >> (3 * bx.b)) & ((1ull << (3 * bx.g)) - 1ull));
+            const uint32_t gc = d == 2 ? ground % bx.nside
+                                       : d == 1 ? (ground / bx.nside) % bx.nside : ground / (bx.nside * bx.nside);
+            const double vlo = dkey_inv(s_ext[b][d]), vhi = dkey_inv(s_ext[b][3 + d]);
             const double m = fmax(fabs(vlo), fabs(vhi));
             const int ex = (int)((__double_as_longlong(m) >> 52) & 0x7ff) - 1022;   // m = f 2^ex, f in [0.5, 1)
             const double C = __longlong_as_double(((long long)(ex + 28 + 1023) << 52) | (1ll << 51));
             const double cen = __dmul_rn(0.5, __dadd_rn(vlo, vhi));
             const double r = __dsub_rn(__dadd_rn(cen, C), C);
             const double half = fmax(__dsub_rn(vhi, r), __dsub_rn(r, vlo));
-            ref[3 * (int64_t)l + d] = r;
-            rf[d] = __double2float_rn(r);   // exact
-            c[d] = __double2float_rn(__dsub_rn(r, __dmul_rn((double)gc[d], bx.h)));
-            hh[d] = __double2float_ru(half);
+            t.ref[3 * (int64_t)(l0 + b) + d] = r;
+            if (kLeaves) s_refd[kLeaves ? b : 0][d] = r;
+            s_ref[b][d] = __double2float_rn(r);   // exact
+            s_c[b][d] = __double2float_rn(__dsub_rn(r, __dmul_rn((double)gc, bx.h)));
+            s_h[b][d] = __double2float_ru(half);
+            if (!kLeaves && d == 0) {
+                t.cell_of[l0 + b] = bx.cell_base + (int)ground;
+                t.box_of[l0 + b] = bi;
+            }
         }
-        r4[l] = make_float4(rf[0], rf[1], rf[2], 0.f);
-        const int f0 = first[l];
-        c4[l] = make_float4(c[0], c[1], c[2], __int_as_float(f0));              // w: first particle
-        h4[l] = make_float4(hh[0], hh[1], hh[2], __int_as_float(first[l + 1] - f0));   // w: particles
-        if (cell_of) cell_of[l] = bx.cell_base + (int)ground;
-        if (box_of) box_of[l] = bi;
+        __syncthreads();
+        if (threadIdx.x < nb) {
+            const int b = threadIdx.x, l = l0 + b, f0 = s_first[b];
+            t.r4[l] = make_float4(s_ref[b][0], s_ref[b][1], s_ref[b][2], 0.f);
+            t.c4[l] = make_float4(s_c[b][0], s_c[b][1], s_c[b][2], __int_as_float(f0));   // w: first particle
+            t.h4[l] = make_float4(s_h[b][0], s_h[b][1], s_h[b][2], __int_as_float(s_first[b + 1] - f0));   // w: particles
+        }
+        if (kLeaves) {
+            for (int k = s_first[0] + threadIdx.x; k < s_first[nb]; k += kThreads) {
+                int b = fr.leaf_of[k] - l0;
+                int64_t g = fr.group_of[k];
+                if (!in_bounds(b, nb, BS_BUILD_ROW)) b = 0;
+                if (!in_bounds(g, fr.n, BS_BUILD_ROW)) g = 0;
+                const float4 gr4 = fr.group_r4[g];
+                const float grf[3] = {gr4.x, gr4.y, gr4.z};
+                float p[3], q[3];
+#pragma unroll
+                for (int d = 0; d < 3; d++) {
+                    const double v = xw[3 * (int64_t)k + d];
+                    float vf;
+                    p[d] = narrow(v, vf) ? __fsub_rn(vf, s_ref[b][d])
+                                         : __double2float_rn(__dsub_rn(v, s_refd[kLeaves ? b : 0][d]));
+                    // the same FP32 offset (the rounded difference of the two exact FP32
+                    // reference points) and FP32 add as the PP kernel's source shift
+                    q[d] = __fadd_rn(p[d], __fsub_rn(s_ref[b][d], grf[d]));
+                }
+                const float m = fr.mass_sorted[k];
+                fr.pos_leaf[k] = make_float4(p[0], p[1], p[2], m);
+                fr.pos_group[k] = make_float4(q[0], q[1], q[2], m);
+            }
+        }
+        __syncthreads();   // the tables are rewritten for the next boxes
     }
 }
 
-// The boxes of the leaves (the first `blocks` blocks) and of the groups (the
-// next), and the first leaf of every ground cell (the rest): independent of
-// each other, one launch.  A cell's first particle starts a leaf; an empty
-// cell takes the next cell's.
-__global__ void k_boxes(BoxTable leaves, BoxTable groups, int blocks, const uint64_t *keys, const BoxDev *boxes, int T,
-                        int64_t n, const int32_t *cell_first, const int32_t *leaf_of, int n_cells,
-                        int32_t *cell_leaf_first)
+// The boxes of the groups (the first `blocks` blocks) and the first leaf of
+// every ground cell (the rest, one thread a cell): independent of each other,
+// one launch.  A cell's first particle starts a leaf; an empty cell takes the
+// next cell's.
+__global__ void __launch_bounds__(kThreads) k_groups(BoxTable groups, int blocks, const uint64_t *keys,
+                                                     const BoxDev *boxes, int T, const double *xw, int64_t n,
+                                                     const int32_t *cell_first, const int32_t *leaf_of,
+                                                     const int32_t *n_leaves, int n_cells, int32_t *cell_leaf_first)
 {
-    const int b = blockIdx.x, t = threadIdx.x;
-    if (b < blocks) {
-        make_boxes(leaves, keys, boxes, T, b * blockDim.x + t, blocks * blockDim.x);
-    } else if (b < 2 * blocks) {
-        make_boxes(groups, keys, boxes, T, (b - blocks) * blockDim.x + t, blocks * blockDim.x);
+    if ((int)blockIdx.x < blocks) {
+        box_block<false>(groups, FrameArgs{}, keys, boxes, T, xw, blockIdx.x, blocks);
     } else {
-        const int c = (b - 2 * blocks) * blockDim.x + t;
-        if (c <= n_cells) cell_leaf_first[c] = cell_first[c] < n ? leaf_of[cell_first[c]] : *leaves.count;
+        const int c = ((int)blockIdx.x - blocks) * (int)blockDim.x + (int)threadIdx.x;
+        if (c <= n_cells) cell_leaf_first[c] = cell_first[c] < n ? leaf_of[cell_first[c]] : *n_leaves;
     }
+}
+
+// The boxes of the leaves and the particles in their frames (after k_groups).
+__global__ void __launch_bounds__(kThreads) k_leaves(BoxTable leaves, FrameArgs fr, const uint64_t *keys,
+                                                     const BoxDev *boxes, int T, const double *xw)
+{
+    box_block<true>(leaves, fr, keys, boxes, T, xw, blockIdx.x, gridDim.x);
 }
 
 // Tree part (theta > 0): one particle per leaf carrying the leaf's mass at
@@ -537,32 +637,6 @@ __global__ void k_leaf_mass(const int32_t *first, const int32_t *n_leaves, const
             q.w = __double2float_rn(M);
         }
         pos_leaf[n + l] = q;
-    }
-}
-
-__global__ void k_pos(int64_t n, const double *xw, const float *mass_sorted, const int32_t *leaf_of,
-                      const int32_t *group_of, const double *leaf_ref, const float4 *leaf_r4, const float4 *group_r4,
-                      float4 *pos_leaf, float4 *pos_group)
-{
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        int64_t l = leaf_of[k];
-        int64_t g = group_of[k];
-        if (!in_bounds(l, n, BS_BUILD_ROW)) l = 0;
-        if (!in_bounds(g, n, BS_BUILD_ROW)) g = 0;
-        const float4 lr4 = leaf_r4[l], gr4 = group_r4[g];
-        const float lrf[3] = {lr4.x, lr4.y, lr4.z}, grf[3] = {gr4.x, gr4.y, gr4.z};
-        float p[3], q[3];
-#pragma unroll
-        for (int d = 0; d < 3; d++) {
-            p[d] = __double2float_rn(__dsub_rn(xw[3 * k + d], leaf_ref[3 * l + d]));
-            // the same FP32 offset (the rounded difference of the two exact FP32
-            // reference points) and FP32 add as the PP kernel's source shift
-            const float off = __fsub_rn(lrf[d], grf[d]);
-            q[d] = __fadd_rn(p[d], off);
-        }
-        const float m = mass_sorted[k];
-        pos_leaf[k] = make_float4(p[0], p[1], p[2], m);
-        pos_group[k] = make_float4(q[0], q[1], q[2], m);
     }
 }
 
@@ -778,31 +852,29 @@ int build_leaves_device(ph_leaves *h, const void *pos, int pos_type, const float
                                            chunk_count);
     count_launch();
     int32_t *leaf_of = static_cast<int32_t *>(h->leaf_of.p), *group_of = static_cast<int32_t *>(h->group_of.p);
-    long long *lext = static_cast<long long *>(h->box_ext.p), *gext = lext + 6 * (size_t)n;
-    k_starts<<<ch.blocks, kThreads, 0, s>>>(starts, n, ch.size, chunk_count, leaf_of, group_of, lfirst, gfirst, lext,
-                                            gext, cnt);
-    count_launch();
-    k_extents<<<grid_for(n), kThreads, 0, s>>>(xw, n, leaf_of, group_of, lext, gext);
+    k_starts<<<ch.blocks, kThreads, 0, s>>>(starts, n, ch.size, chunk_count, leaf_of, group_of, lfirst, gfirst, cnt);
     count_launch();
     double *lref = static_cast<double *>(h->leaf_ref.p);
     float4 *lr4 = static_cast<float4 *>(h->leaf_r4.p), *gr4 = static_cast<float4 *>(h->group_r4.p);
     float4 *pos_leaf = static_cast<float4 *>(h->pos_leaf.p);
-    const BoxTable lt{lfirst, cnt, lext, lref, lr4, static_cast<float4 *>(h->leaf_c4.p),
+    const BoxTable lt{lfirst, cnt, lref, lr4, static_cast<float4 *>(h->leaf_c4.p),
                       static_cast<float4 *>(h->leaf_h4.p), nullptr, nullptr};
-    const BoxTable gt{gfirst, cnt + 1, gext, static_cast<double *>(h->group_ref.p), gr4,
+    const BoxTable gt{gfirst, cnt + 1, static_cast<double *>(h->group_ref.p), gr4,
                       static_cast<float4 *>(h->group_c4.p), static_cast<float4 *>(h->group_h4.p),
                       static_cast<int32_t *>(h->group_cell.p), static_cast<int32_t *>(h->group_box.p)};
-    const int bb = grid_for(n, kThreads, 152 * 4);
-    k_boxes<<<2 * bb + cell_blocks, kThreads, 0, s>>>(lt, gt, bb, sk, boxes, T, n, cell_first, leaf_of, h->n_cells,
-                                                     cell_leaf_first);
+    const FrameArgs fr{ms, leaf_of, group_of, gr4, pos_leaf, static_cast<float4 *>(h->pos_group.p), n};
+    // at most one part-filled group a ground cell; up to n leaves
+    const int64_t most = std::min<int64_t>(n, n / h->group_size + h->n_cells);
+    const int gb = grid_for(most, kBoxes), lb = grid_for(n, kBoxes);
+    k_groups<<<gb + cell_blocks, kThreads, 0, s>>>(gt, gb, sk, boxes, T, xw, n, cell_first, leaf_of, cnt, h->n_cells,
+                                                   cell_leaf_first);
+    count_launch();
+    k_leaves<<<lb, kThreads, 0, s>>>(lt, fr, sk, boxes, T, xw);
     count_launch();
     if (h->tree_leaves) {
         k_leaf_mass<<<grid_for(n), kThreads, 0, s>>>(lfirst, cnt, xw, ms, lref, n, pos_leaf);
         count_launch();
     }
-    k_pos<<<grid_for(n), kThreads, 0, s>>>(n, xw, ms, leaf_of, group_of, lref, lr4, gr4, pos_leaf,
-                                           static_cast<float4 *>(h->pos_group.p));
-    count_launch();
     int rc = 0;
     if (h->active) {
         // the groups to sum in active-particle mode (buffers sized by the caller)

@@ -98,14 +98,14 @@ void carve(Carver &c, ph_leaves &lv, ph_pairs &pr, int64_t n, int cells)
     c.take(lv.leaf_first, 4 * (N + 1));
     c.take(lv.group_first, 4 * (N + 1));
     c.take(lv.group_h4, 16 * N);
-    c.take(lv.leaf_ref, 24 * N);   // from here to box_ext: not read by the PP kernel
+    c.take(lv.leaf_ref, 24 * N);   // from here to task_mem: not read by the PP kernel
     c.take(lv.leaf_c4, 16 * N);
     c.take(lv.leaf_h4, 16 * N);
     c.take(lv.group_ref, 24 * N);
     c.take(lv.group_c4, 16 * N);
     c.take(lv.leaf_r4, 16 * N);
     c.take(lv.group_r4, 16 * N);
-    c.take(lv.box_ext, 96 * N);
+    c.take(pr.task_mem, 96 * N);
     c.take(lv.group_cell, 4 * N);
     c.take(lv.group_box, 4 * N);
     c.take(lv.pos_leaf, 16 * N);
@@ -124,9 +124,9 @@ void carve(Carver &c, ph_leaves &lv, ph_pairs &pr, int64_t n, int cells)
     c.take(pr.ecount, cap);
     c.take(pr.order_temp, order_temp_bytes(n));
     // the tasks of split groups: records and counters where the sort's keys
-    // were, sums where the boxes' tables and extents were (what the PP kernel
-    // does not read)
-    const size_t room = (size_t)((char *)lv.box_ext.p + lv.box_ext.bytes - (char *)lv.leaf_ref.p) / (96 * sizeof(float));
+    // were, sums in task_mem and where the boxes' tables were (what the PP
+    // kernel does not read)
+    const size_t room = (size_t)((char *)pr.task_mem.p + pr.task_mem.bytes - (char *)lv.leaf_ref.p) / (96 * sizeof(float));
     pr.task_cap = (int64_t)(room < N / 2 ? room : N / 2);
     pr.tasks = static_cast<int2 *>(lv.keys.p);
     pr.task_done = static_cast<int32_t *>(lv.keys_alt.p);

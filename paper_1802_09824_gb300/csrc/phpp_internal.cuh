@@ -63,6 +63,7 @@ struct BoxDev {
     float s2;
     float eps2s;       // max(eps^2 s2, 1e-12)
     float c_g;
+    float S_hi, S_lo;  // S as a double-float (FP32 cell decisions of the key kernel)
     float L_up;        // smallest FP32 number >= L: an FP32 x is below L iff x < L_up
     float c_acc;       // 1 / theta of the tree part (infinite: every leaf pair by PP)
     // The exact kernel's inverse-distance form of the factor (fit_inverse_form;
