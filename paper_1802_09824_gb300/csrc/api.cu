@@ -17,10 +17,11 @@ namespace phpp {
 
 int build_leaves_device(ph_leaves *h, const void *pos, int pos_type, const float *mass, cudaStream_t s);
 int build_pairs_device(const ph_leaves *lv, ph_pairs *pr, cudaStream_t s, bool sizing_sync);
-int pp_exact_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s);
+int pp_exact_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s, bool chained);
 int count_within_device(const ph_leaves *lv, const ph_pairs *pr, cudaStream_t s);
-int pp_learned_device(const ph_leaves *lv, const ph_pairs *pr, const float *mlp_w, float *d_acc, cudaStream_t s);
-int pp_table_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s);
+int pp_learned_device(const ph_leaves *lv, const ph_pairs *pr, const float *mlp_w, float *d_acc, cudaStream_t s,
+                      bool chained);
+int pp_table_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s, bool chained);
 
 // The tabulated factor of PH_G_TABLE for the handle's (single) rs and rcut:
 // f(r_i) = erfc(u) + (2u / sqrt(pi)) exp(-u^2), u = r_i / (2 rs), at
@@ -663,10 +664,10 @@ int ph_pp_accel(const ph_leaves *leaves, const ph_pairs *pairs, int g_mode, cons
     }
     if (g_mode == PH_G_TABLE) {
         rc = ensure_table(lvm, s);
-        if (!rc) rc = pp_table_device(leaves, pairs, dacc, s);
+        if (!rc) rc = pp_table_device(leaves, pairs, dacc, s, false);
     } else {
-        rc = use_learned ? pp_learned_device(leaves, pairs, static_cast<const float *>(mlp->theta.p), dacc, s)
-                         : pp_exact_device(leaves, pairs, dacc, s);
+        rc = use_learned ? pp_learned_device(leaves, pairs, static_cast<const float *>(mlp->theta.p), dacc, s, false)
+                         : pp_exact_device(leaves, pairs, dacc, s, false);
     }
     if (!rc && !dev)
         rc = cuda_check(cudaMemcpyAsync(acc, dacc, (size_t)leaves->n * 12, cudaMemcpyDeviceToHost, s), "copy acc");

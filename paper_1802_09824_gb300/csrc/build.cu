@@ -141,6 +141,7 @@ template <int kPosType>
 __global__ void k_keys(const void *pos, int64_t n, const int32_t *box_first, int nb, const BoxDev *boxes, int T,
                        int key_kind, uint64_t *keys, int32_t *vals, SortCounts sc, uint32_t *status)
 {
+    chain_begin();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int bi = nb > 1 ? find_box(box_first, nb, i) : 0;
         const BoxDev &bx = boxes[bi];
@@ -216,6 +217,7 @@ __global__ void k_gather(const void *pos, const float *mass, int64_t n, const ui
                          const BoxDev *boxes, int T, double *xw, float *mass_sorted, uint32_t *status, int cell_blocks,
                          int nb, int n_cells, int32_t *cell_first)
 {
+    chain_begin();
     const int blocks = (int)gridDim.x - cell_blocks;
     if ((int)blockIdx.x >= blocks) {
         cell_starts(keys, n, boxes, nb, n_cells, T, ((int)blockIdx.x - blocks) * (int)blockDim.x + (int)threadIdx.x,
@@ -285,6 +287,7 @@ __global__ void __launch_bounds__(kThreads) k_flags(const uint64_t *keys, int64_
                                                     int T, int leaf_max, int level_bits, const int32_t *cell_first,
                                                     uint8_t *starts, int2 *chunk_count)
 {
+    chain_begin();
     const int64_t lo = blockIdx.x * chunk, end = lo + chunk < n ? lo + chunk : n;
     int nl = 0, ngr = 0;
     for (int64_t k = lo + threadIdx.x; k < end; k += kThreads) {
@@ -354,6 +357,7 @@ __global__ void __launch_bounds__(kThreads) k_starts(const uint8_t *starts, int6
                                                      const int2 *chunk_count, int32_t *leaf_of, int32_t *group_of,
                                                      int32_t *lfirst, int32_t *gfirst, int32_t *counts)
 {
+    chain_begin();
     __shared__ int2 s_w[2][kThreads / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned le = 0xffffffffu >> (31 - lane);
@@ -594,6 +598,7 @@ __global__ void __launch_bounds__(kThreads) k_groups(BoxTable groups, int blocks
                                                      const int32_t *cell_first, const int32_t *leaf_of,
                                                      const int32_t *n_leaves, int n_cells, int32_t *cell_leaf_first)
 {
+    chain_begin();
     if ((int)blockIdx.x < blocks) {
         box_block<false>(groups, FrameArgs{}, keys, boxes, T, xw, blockIdx.x, blocks);
     } else {
@@ -606,6 +611,7 @@ __global__ void __launch_bounds__(kThreads) k_groups(BoxTable groups, int blocks
 __global__ void __launch_bounds__(kThreads) k_leaves(BoxTable leaves, FrameArgs fr, const uint64_t *keys,
                                                      const BoxDev *boxes, int T, const double *xw)
 {
+    chain_begin();
     box_block<true>(leaves, fr, keys, boxes, T, xw, blockIdx.x, gridDim.x);
 }
 
@@ -617,6 +623,7 @@ __global__ void __launch_bounds__(kThreads) k_leaves(BoxTable leaves, FrameArgs 
 __global__ void k_leaf_mass(const int32_t *first, const int32_t *n_leaves, const double *xw, const float *mass,
                             const double *ref, int64_t n, float4 *pos_leaf)
 {
+    chain_begin();
     const int count = *n_leaves;
     for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < count; l += gridDim.x * blockDim.x) {
         const int a = first[l], e = first[l + 1];
@@ -802,12 +809,11 @@ int build_leaves_device(ph_leaves *h, const void *pos, int pos_type, const float
         if (rc) return rc;
         const SortCounts sc = sort_counts(n, h->temp.p);
         if (pos_type == PH_F64)
-            k_keys<PH_F64><<<grid_for(n), kThreads, 0, s>>>(pos, n, box_first, nb, boxes, T, h->key_kind, keys, vals,
-                                                            sc, status);
+            launch_chained(true, k_keys<PH_F64>, grid_for(n), kThreads, 0, s, pos, n, box_first, nb, boxes, T,
+                           h->key_kind, keys, vals, sc, status);
         else
-            k_keys<PH_F32><<<grid_for(n), kThreads, 0, s>>>(pos, n, box_first, nb, boxes, T, h->key_kind, keys, vals,
-                                                            sc, status);
-        count_launch();
+            launch_chained(true, k_keys<PH_F32>, grid_for(n), kThreads, 0, s, pos, n, box_first, nb, boxes, T,
+                           h->key_kind, keys, vals, sc, status);
         bool alt = false;
         int box_bits = 0;
         while ((1 << box_bits) < nb) box_bits++;
@@ -839,21 +845,19 @@ int build_leaves_device(ph_leaves *h, const void *pos, int pos_type, const float
     }
     const int cell_blocks = (h->n_cells + kThreads) / kThreads;   // one thread a cell, and one for the end
     if (pos_type == PH_F64)
-        k_gather<PH_F64><<<grid_for(n) + cell_blocks, kThreads, 0, s>>>(pos, mass, n, sk, perm, boxes, T, xw, ms, status,
-                                                                       cell_blocks, nb, h->n_cells, cell_first);
+        launch_chained(true, k_gather<PH_F64>, grid_for(n) + cell_blocks, kThreads, 0, s, pos, mass, n, sk, perm, boxes,
+                       T, xw, ms, status, cell_blocks, nb, h->n_cells, cell_first);
     else
-        k_gather<PH_F32><<<grid_for(n) + cell_blocks, kThreads, 0, s>>>(pos, mass, n, sk, perm, boxes, T, xw, ms, status,
-                                                                       cell_blocks, nb, h->n_cells, cell_first);
-    count_launch();
+        launch_chained(true, k_gather<PH_F32>, grid_for(n) + cell_blocks, kThreads, 0, s, pos, mass, n, sk, perm, boxes,
+                       T, xw, ms, status, cell_blocks, nb, h->n_cells, cell_first);
     const Chunks ch = chunks_of(n);
     uint8_t *starts = static_cast<uint8_t *>(h->starts.p);
     int2 *chunk_count = static_cast<int2 *>(h->temp.p);   // (the sort is done with it)
-    k_flags<<<ch.blocks, kThreads, 0, s>>>(sk, n, ch.size, boxes, T, h->max_leaf, h->level_bits, cell_first, starts,
-                                           chunk_count);
-    count_launch();
+    launch_chained(true, k_flags, ch.blocks, kThreads, 0, s, sk, n, ch.size, boxes, T, h->max_leaf, h->level_bits,
+                   cell_first, starts, chunk_count);
     int32_t *leaf_of = static_cast<int32_t *>(h->leaf_of.p), *group_of = static_cast<int32_t *>(h->group_of.p);
-    k_starts<<<ch.blocks, kThreads, 0, s>>>(starts, n, ch.size, chunk_count, leaf_of, group_of, lfirst, gfirst, cnt);
-    count_launch();
+    launch_chained(true, k_starts, ch.blocks, kThreads, 0, s, starts, n, ch.size, chunk_count, leaf_of, group_of, lfirst,
+                   gfirst, cnt);
     double *lref = static_cast<double *>(h->leaf_ref.p);
     float4 *lr4 = static_cast<float4 *>(h->leaf_r4.p), *gr4 = static_cast<float4 *>(h->group_r4.p);
     float4 *pos_leaf = static_cast<float4 *>(h->pos_leaf.p);
@@ -866,14 +870,11 @@ int build_leaves_device(ph_leaves *h, const void *pos, int pos_type, const float
     // at most one part-filled group a ground cell; up to n leaves
     const int64_t most = std::min<int64_t>(n, n / h->group_size + h->n_cells);
     const int gb = grid_for(most, kBoxes), lb = grid_for(n, kBoxes);
-    k_groups<<<gb + cell_blocks, kThreads, 0, s>>>(gt, gb, sk, boxes, T, xw, n, cell_first, leaf_of, cnt, h->n_cells,
-                                                   cell_leaf_first);
-    count_launch();
-    k_leaves<<<lb, kThreads, 0, s>>>(lt, fr, sk, boxes, T, xw);
-    count_launch();
+    launch_chained(true, k_groups, gb + cell_blocks, kThreads, 0, s, gt, gb, sk, boxes, T, xw, n, cell_first, leaf_of,
+                   cnt, h->n_cells, cell_leaf_first);
+    launch_chained(true, k_leaves, lb, kThreads, 0, s, lt, fr, sk, boxes, T, xw);
     if (h->tree_leaves) {
-        k_leaf_mass<<<grid_for(n), kThreads, 0, s>>>(lfirst, cnt, xw, ms, lref, n, pos_leaf);
-        count_launch();
+        launch_chained(true, k_leaf_mass, grid_for(n), kThreads, 0, s, lfirst, cnt, xw, ms, lref, n, pos_leaf);
     }
     int rc = 0;
     if (h->active) {

@@ -17,9 +17,10 @@
 namespace phpp {
 int build_leaves_device(ph_leaves *h, const void *pos, int pos_type, const float *mass, cudaStream_t s);
 int build_pairs_device(const ph_leaves *lv, ph_pairs *pr, cudaStream_t s, bool sizing_sync);
-int pp_exact_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s);
-int pp_learned_device(const ph_leaves *lv, const ph_pairs *pr, const float *mlp_w, float *d_acc, cudaStream_t s);
-int pp_table_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s);
+int pp_exact_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s, bool chained);
+int pp_learned_device(const ph_leaves *lv, const ph_pairs *pr, const float *mlp_w, float *d_acc, cudaStream_t s,
+                      bool chained);
+int pp_table_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s, bool chained);
 int ensure_table(ph_leaves *lv, cudaStream_t s);
 }  // namespace phpp
 
@@ -118,9 +119,9 @@ int ph_graph_create(ph_leaves *leaves, ph_pairs *pairs, const void *d_pos, int p
         if (!rc2) rc2 = build_leaves_device(leaves, d_pos, pos_type, d_mass, s);
         if (!rc2 && pairs) rc2 = build_pairs_device(leaves, pairs, s, false);
         if (!rc2 && leaves->n > 0)
-            rc2 = g_mode == PH_G_TABLE ? pp_table_device(leaves, pairs, d_acc, s)
-                  : learned ? pp_learned_device(leaves, pairs, static_cast<const float *>(mlp->theta.p), d_acc, s)
-                            : pp_exact_device(leaves, pairs, d_acc, s);
+            rc2 = g_mode == PH_G_TABLE ? pp_table_device(leaves, pairs, d_acc, s, pairs != nullptr)
+                  : learned ? pp_learned_device(leaves, pairs, static_cast<const float *>(mlp->theta.p), d_acc, s, pairs != nullptr)
+                            : pp_exact_device(leaves, pairs, d_acc, s, pairs != nullptr);
         cudaGraph_t gr = nullptr;
         rc = cuda_check(cudaStreamEndCapture(s, &gr), "end capture");
         g->graph = gr;

@@ -24,7 +24,7 @@
 namespace phpp {
 int build_leaves_device(ph_leaves *h, const void *pos, int pos_type, const float *mass, cudaStream_t s);
 int build_pairs_device(const ph_leaves *lv, ph_pairs *pr, cudaStream_t s, bool sizing_sync);
-int pp_exact_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s);
+int pp_exact_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s, bool chained);
 }  // namespace phpp
 
 using namespace phpp;
@@ -226,7 +226,7 @@ extern "C" int ph_accel_noalloc(const float *d_pos, const float *d_mass, int64_t
                         "copy box table");
     if (!rc) rc = build_leaves_device(&lv, d_pos, PH_F32, d_mass, s);
     if (!rc) rc = build_pairs_device(&lv, &pr, s, false);
-    if (!rc) rc = pp_exact_device(&lv, &pr, d_acc, s);
+    if (!rc) rc = pp_exact_device(&lv, &pr, d_acc, s, true);
     // one synchronisation: the box record lives on this stack frame, and the
     // latched device status decides the return code
     uint32_t st[2] = {0, 0};

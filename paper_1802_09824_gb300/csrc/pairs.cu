@@ -103,6 +103,7 @@ __device__ __forceinline__ int cost_bucket(unsigned c)
 template <bool kFill>
 __global__ void __launch_bounds__(kThreads) k_pairs(PairArgs a)
 {
+    chain_begin();
     __shared__ int2 s_run[kThreads / 32][32];   // per warp: (image code, first leaf - excl) of each run
     __shared__ float4 s_sh[kThreads / 32][32];  // per warp: the run's cell offset (dx h, dy h, dz h) in the group's frame
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -288,12 +289,22 @@ __global__ void __launch_bounds__(kThreads) k_pairs(PairArgs a)
     }
 }
 
+__global__ void __launch_bounds__(kThreads) k_clear_counts(uint32_t *p, int64_t n)
+{
+    chain_begin();
+    for (int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads) p[i] = 0u;
+}
+
 // The list's offsets: exclusive prefix of the groups' counts (off[n_groups]:
 // all entries), one block per kOffChunk groups; the chunks before its own it
 // adds up from the count pass's sums.
 __global__ void __launch_bounds__(kThreads) k_offsets(const int64_t *cnt, const int32_t *n_groups,
-                                                      const unsigned long long *chunk_sum, int64_t *off)
+                                                      const unsigned long long *chunk_sum, int64_t *off,
+                                                      unsigned long long *work)
 {
+    chain_begin();
+    // the PP kernel's queue and counters (a captured step has no other reset)
+    if (blockIdx.x == 0 && threadIdx.x < 3) work[threadIdx.x] = 0;
     __shared__ long long s_w[kThreads / 32];
     const int ng = *n_groups, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int g0 = blockIdx.x * kOffChunk;
@@ -425,8 +436,7 @@ static int fill_pairs(ph_pairs *pr, PairArgs &a, const int32_t *n_all, int grid,
     a.ent = static_cast<float4 *>(pr->entries.p);
     a.ecnt = static_cast<uint8_t *>(pr->ecount.p);
     a.cap = pr->capacity;
-    k_pairs<true><<<grid, kThreads, 0, s>>>(a);
-    count_launch();
+    launch_chained(!sizing_sync, k_pairs<true>, grid, kThreads, 0, s, a);
     return PH_OK;
 }
 
@@ -478,17 +488,14 @@ int build_pairs_device(const ph_leaves *lv, ph_pairs *pr, cudaStream_t s, bool s
         const int rz = cuda_check(cudaMemsetAsync(a.cnt, 0, 8 * (size_t)(n > 0 ? n : 1), s), "clear counts");
         if (rz) return rz;
     }
-    {
-        const int rz = cuda_check(cudaMemsetAsync(ot, 0, order_temp_bytes(n), s), "clear the queue's counts");
-        if (rz) return rz;
-    }
-    k_pairs<false><<<grid, kThreads, 0, s>>>(a);
-    count_launch();
+    const int64_t words = (int64_t)(order_temp_bytes(n) / sizeof(uint32_t));
+    launch_chained(false, k_clear_counts, (int)std::min<int64_t>((words + 1023) / 1024, 152), kThreads, 0, s,
+                   reinterpret_cast<uint32_t *>(ot), words);
+    launch_chained(true, k_pairs<false>, grid, kThreads, 0, s, a);
     // at most one part-filled group a ground cell
     const int64_t most = std::min<int64_t>(n, n / lv->group_size + lv->n_cells);
-    k_offsets<<<(int)(most / kOffChunk) + 1, kThreads, 0, s>>>(a.cnt, n_all, a.chunk_sum,
-                                                              static_cast<int64_t *>(pr->group_off.p));
-    count_launch();
+    launch_chained(true, k_offsets, (int)(most / kOffChunk) + 1, kThreads, 0, s, a.cnt, n_all, a.chunk_sum,
+                   static_cast<int64_t *>(pr->group_off.p), static_cast<unsigned long long *>(pr->work.p));
     int rc = fill_pairs(pr, a, n_all, grid, s, sizing_sync, n);
     if (rc) return rc;
     return cuda_check(cudaGetLastError(), "pair kernels");

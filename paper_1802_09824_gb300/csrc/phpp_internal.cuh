@@ -180,6 +180,44 @@ int cuda_check(cudaError_t e, const char *what);
 // Host-side count of kernel launches issued by the library (all threads).
 void count_launch(int n = 1);
 
+// The kernels of a step are launched as a chain: each may be set up (blocks
+// placed, parameters loaded) while its predecessor still runs, and begins by
+// waiting for the predecessor's completion (programmatic dependent launch).
+// chain_begin has to be a chained kernel's first statement in every block,
+// before any memory access; the predecessor's completion implies that of all
+// work before it, since it waited the same way.  Measured without and with:
+// the no-allocation step of 1000 particles 131 and 108 us, the captured step of
+// 4096 78.5 and 69.3 us, 50,021 particles 404 and 382 us; 0.2 % at 128^3, where
+// the gaps are a small part.
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launches a kernel that starts with chain_begin behind the previous kernel of
+// the stream.  chained = false where the previous operation may not be a
+// kernel (a copy or a memset being captured).
+template <typename... KArgs, typename... Args>
+inline void launch_chained(bool chained, void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
+                           Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = chained ? 1 : 0;
+    (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);   // (errors: cudaGetLastError of the caller)
+    count_launch();
+}
+#endif
+
 // Debug bounds checks (checks.cuh): each translation unit of a checked build
 // registers a reader of its device words (hits, first site) at load time.
 void register_bounds_reader(int (*read)(unsigned int *hits, unsigned int *site));
@@ -215,7 +253,7 @@ struct SortCounts {
 };
 size_t sort_temp_bytes(int64_t n);
 SortCounts sort_counts(int64_t n, void *temp);
-int sort_begin(int64_t n, void *temp, cudaStream_t s);
+int sort_begin(int64_t n, void *temp, cudaStream_t s);   // (a kernel: the next one may be chained to it)
 int radix_sort_pairs(uint64_t *keys, int32_t *vals, uint64_t *keys_alt, int32_t *vals_alt, int64_t n, int bits,
                      void *temp, cudaStream_t s, bool *result_in_alt);
 

@@ -548,6 +548,7 @@ __device__ __noinline__ void finish_task(const PPArgs &a, int t, int ni, int i0,
 template <int NPOLY, bool kLearned, int kMinBlocks, int kSplit, bool kUniform, bool kTable = false>
 __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
 {
+    chain_begin();
     __shared__ float4 sA[kPPWarps][kJBuf / 2];
     __shared__ float4 sB[kPPWarps][kJBuf / 2];
     __shared__ float4 sQ[kLearned ? kPPWarps : 1][kLearned ? kLQ + 1 : 1];   // learned: the pair queue
@@ -1083,14 +1084,15 @@ static void pp_args(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, PPArg
 }
 
 template <bool kLearned, int kMinBlocks, int kSplit, bool kUniform>
-static void launch_pp(int npoly, int grid, cudaStream_t s, const PPArgs &a)
+static void launch_pp(bool chained, int npoly, int grid, cudaStream_t s, const PPArgs &a)
 {
+    auto launch = [&](auto kernel) { launch_chained(chained, kernel, grid, kPPThreads, 0, s, a); };
     switch (npoly) {
-    case kInvDeg: k_pp<kInvDeg, kLearned, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
-    case 10: k_pp<10, kLearned, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
-    case 12: k_pp<12, kLearned, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
-    case 14: k_pp<14, kLearned, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
-    default: k_pp<16, kLearned, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
+    case kInvDeg: launch(k_pp<kInvDeg, kLearned, kMinBlocks, kSplit, kUniform>); break;
+    case 10: launch(k_pp<10, kLearned, kMinBlocks, kSplit, kUniform>); break;
+    case 12: launch(k_pp<12, kLearned, kMinBlocks, kSplit, kUniform>); break;
+    case 14: launch(k_pp<14, kLearned, kMinBlocks, kSplit, kUniform>); break;
+    default: launch(k_pp<16, kLearned, kMinBlocks, kSplit, kUniform>); break;
     }
 }
 
@@ -1130,7 +1132,7 @@ static void launch_walk(const ph_leaves *lv, int npoly, bool uni, cudaStream_t s
 constexpr int kTabBytes = (kTabN + 1) * (int)sizeof(float2);
 
 template <int kSplit>
-static void launch_table_one(int grid, cudaStream_t s, const PPArgs &a)
+static void launch_table_one(bool chained, int grid, cudaStream_t s, const PPArgs &a)
 {
     static bool ready = false;
     if (!ready) {
@@ -1138,7 +1140,7 @@ static void launch_table_one(int grid, cudaStream_t s, const PPArgs &a)
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kTabBytes);
         ready = true;
     }
-    k_pp<10, false, kBlocks0, kSplit, true, true><<<grid, kPPThreads, kTabBytes, s>>>(a);
+    launch_chained(chained, k_pp<10, false, kBlocks0, kSplit, true, true>, grid, kPPThreads, kTabBytes, s, a);
 }
 
 constexpr int kL1Bytes = 4 * kL1Nodes * (int)sizeof(float4);   // layer 1's table (dynamic shared memory)
@@ -1160,20 +1162,21 @@ int pp_learned_setup()
     return rc;
 }
 
-int pp_learned_device(const ph_leaves *lv, const ph_pairs *pr, const float *mlp_w, float *d_acc, cudaStream_t s)
+int pp_learned_device(const ph_leaves *lv, const ph_pairs *pr, const float *mlp_w, float *d_acc, cudaStream_t s,
+                      bool chained)
 {
     PPArgs a;
     pp_args(lv, pr, d_acc, a);
     a.mlp_w = mlp_w;
-    int rc = cuda_check(cudaMemsetAsync(pr->work.p, 0, 24, s), "reset work queue");
+    int rc = chained ? PH_OK : cuda_check(cudaMemsetAsync(pr->work.p, 0, 24, s), "reset work queue");
     if (rc) return rc;
     const int grid = sm_count() * kBlocks0;
     rc = pp_learned_setup();
     if (rc) return rc;
-    if (lv->group_size == 8) k_pp<10, true, kBlocks0, 4, false><<<grid, kPPThreads, kL1Bytes, s>>>(a);
-    else if (lv->group_size == 16) k_pp<10, true, kBlocks0, 2, false><<<grid, kPPThreads, kL1Bytes, s>>>(a);
-    else k_pp<10, true, kBlocks0, 1, false><<<grid, kPPThreads, kL1Bytes, s>>>(a);
-    count_launch();
+    auto launch = [&](auto kernel) { launch_chained(chained, kernel, grid, kPPThreads, kL1Bytes, s, a); };
+    if (lv->group_size == 8) launch(k_pp<10, true, kBlocks0, 4, false>);
+    else if (lv->group_size == 16) launch(k_pp<10, true, kBlocks0, 2, false>);
+    else launch(k_pp<10, true, kBlocks0, 1, false>);
     return cuda_check(cudaGetLastError(), "learned pp kernel");
 }
 
@@ -1218,7 +1221,7 @@ static bool uniform_consts(const ph_leaves *lv, PairConsts &uc, bool general)
 
 // PP with the tabulated factor (every box shares one rcut and rs; the table
 // is lv->table, filled by the caller for them).
-int pp_table_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s)
+int pp_table_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s, bool chained)
 {
     PPArgs a;
     pp_args(lv, pr, d_acc, a);
@@ -1226,22 +1229,23 @@ int pp_table_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaS
     if (!uniform_consts(lv, a.uc, true)) return fail(PH_ERR_ARG, "the tabulated factor needs one rcut and rs for all boxes");
     a.table = static_cast<const float2 *>(lv->table.p);
     a.tab_scale2 = (float)((kTabN / lv->table_rcut) * (kTabN / lv->table_rcut));
-    int rc2 = cuda_check(cudaMemsetAsync(pr->work.p, 0, 24, s), "reset work queue");
+    int rc2 = chained ? PH_OK : cuda_check(cudaMemsetAsync(pr->work.p, 0, 24, s), "reset work queue");
     if (rc2) return rc2;
     const int grid = sm_count() * kBlocks0;
-    if (lv->group_size == 8) launch_table_one<4>(grid, s, a);
-    else if (lv->group_size == 16) launch_table_one<2>(grid, s, a);
-    else launch_table_one<1>(grid, s, a);
-    count_launch();
+    if (lv->group_size == 8) launch_table_one<4>(chained, grid, s, a);
+    else if (lv->group_size == 16) launch_table_one<2>(chained, grid, s, a);
+    else launch_table_one<1>(chained, grid, s, a);
     return cuda_check(cudaGetLastError(), "table pp kernel");
 }
 
-int pp_exact_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s)
+// chained (here and for the other factors): launched right behind the passes
+// that made the list, which also reset the queue.
+int pp_exact_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaStream_t s, bool chained)
 {
     PPArgs a;
     pp_args(lv, pr, d_acc, a);
     a.mlp_w = nullptr;
-    int rc = cuda_check(cudaMemsetAsync(pr ? pr->work.p : lv->work.p, 0, 24, s), "reset work queue");
+    int rc = chained ? PH_OK : cuda_check(cudaMemsetAsync(pr ? pr->work.p : lv->work.p, 0, 24, s), "reset work queue");
     if (rc) return rc;
     const int npoly = lv->poly_degree;
     if (npoly != kInvDeg && npoly != 10 && npoly != 12 && npoly != 14 && npoly != 16)
@@ -1257,22 +1261,21 @@ int pp_exact_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaS
     const int gs = lv->group_size;
     if (uni) {
         if (three) {
-            if (gs == 8) launch_pp<false, kBlocks1, 4, true>(npoly, grid, s, a);
-            else if (gs == 16) launch_pp<false, kBlocks1, 2, true>(npoly, grid, s, a);
-            else launch_pp<false, kBlocks1, 1, true>(npoly, grid, s, a);
+            if (gs == 8) launch_pp<false, kBlocks1, 4, true>(chained, npoly, grid, s, a);
+            else if (gs == 16) launch_pp<false, kBlocks1, 2, true>(chained, npoly, grid, s, a);
+            else launch_pp<false, kBlocks1, 1, true>(chained, npoly, grid, s, a);
         } else {
-            if (gs == 8) launch_pp<false, kBlocks0, 4, true>(npoly, grid, s, a);
-            else if (gs == 16) launch_pp<false, kBlocks0, 2, true>(npoly, grid, s, a);
-            else launch_pp<false, kBlocks0, 1, true>(npoly, grid, s, a);
+            if (gs == 8) launch_pp<false, kBlocks0, 4, true>(chained, npoly, grid, s, a);
+            else if (gs == 16) launch_pp<false, kBlocks0, 2, true>(chained, npoly, grid, s, a);
+            else launch_pp<false, kBlocks0, 1, true>(chained, npoly, grid, s, a);
         }
     } else {
         // boxes with different constants: the two-block shape only
         const int g2 = sm_count() * kBlocks0;
-        if (gs == 8) launch_pp<false, kBlocks0, 4, false>(npoly, g2, s, a);
-        else if (gs == 16) launch_pp<false, kBlocks0, 2, false>(npoly, g2, s, a);
-        else launch_pp<false, kBlocks0, 1, false>(npoly, g2, s, a);
+        if (gs == 8) launch_pp<false, kBlocks0, 4, false>(chained, npoly, g2, s, a);
+        else if (gs == 16) launch_pp<false, kBlocks0, 2, false>(chained, npoly, g2, s, a);
+        else launch_pp<false, kBlocks0, 1, false>(chained, npoly, g2, s, a);
     }
-    count_launch();
     return cuda_check(cudaGetLastError(), "pp kernel");
 }
 

@@ -63,6 +63,7 @@ __device__ __forceinline__ int block_excl(int v, int *s_wsum)
 // Exclusive prefix over the tiles of one digit's counts, and its total.
 __global__ void __launch_bounds__(kSortThreads) k_digit_scan(const int32_t *hist, int row, int32_t *offs, int32_t *total)
 {
+    chain_begin();
     __shared__ int s_wsum[kSortWarps];
     __shared__ int s_sum;
     const int32_t *h = hist + (int64_t)blockIdx.x * row;
@@ -83,6 +84,13 @@ __global__ void __launch_bounds__(kSortThreads) k_digit_scan(const int32_t *hist
     if (threadIdx.x == 0) total[blockIdx.x] = run;
 }
 
+__global__ void __launch_bounds__(kSortThreads) k_clear(int4 *p, int n)
+{
+    chain_begin();
+    for (int i = blockIdx.x * kSortThreads + threadIdx.x; i < n; i += gridDim.x * kSortThreads)
+        p[i] = make_int4(0, 0, 0, 0);
+}
+
 struct PassArgs {
     const uint64_t *keys;
     const int32_t *vals;
@@ -101,6 +109,7 @@ struct PassArgs {
 template <int kItems, bool kDirect>
 __global__ void __launch_bounds__(kSortThreads) k_radix_pass(PassArgs a)
 {
+    chain_begin();
     constexpr int kTile = kSortThreads * kItems;
     __shared__ uint16_t cnt[kSortWarps][kBins];   // (a tile has at most 2048 keys)
     __shared__ int32_t s_off[kBins];            // output position of the tile's first key of each digit
@@ -219,8 +228,7 @@ SortLayout layout_for(int64_t n)
 template <int kItems, bool kDirect>
 void launch_pass(const PassArgs &a, cudaStream_t s)
 {
-    k_radix_pass<kItems, kDirect><<<a.ntiles, kSortThreads, 0, s>>>(a);
-    count_launch();
+    launch_chained(true, k_radix_pass<kItems, kDirect>, a.ntiles, kSortThreads, 0, s, a);
 }
 
 }  // namespace
@@ -239,7 +247,10 @@ SortCounts sort_counts(int64_t n, void *temp)
 
 int sort_begin(int64_t n, void *temp, cudaStream_t s)
 {
-    return cuda_check(cudaMemsetAsync(temp, 0, 2 * layout_for(n).counts, s), "clear digit counts");
+    const int words = (int)(2 * layout_for(n).counts / sizeof(int4));
+    k_clear<<<std::min((words + 1023) / 1024, 152 * 4), kSortThreads, 0, s>>>(static_cast<int4 *>(temp), words);
+    count_launch();
+    return cuda_check(cudaGetLastError(), "clear digit counts");
 }
 
 int radix_sort_pairs(uint64_t *keys, int32_t *vals, uint64_t *keys_alt, int32_t *vals_alt, int64_t n, int bits,
@@ -276,8 +287,7 @@ int radix_sort_pairs(uint64_t *keys, int32_t *vals, uint64_t *keys_alt, int32_t 
         a.hist_next = last ? nullptr : hist[(p + 1) % 3];
         a.hist_clear = last ? nullptr : hist[(p + 2) % 3];
         if (!direct) {
-            k_digit_scan<<<kBins, kSortThreads, 0, s>>>(a.hist, l.row, offs, total);
-            count_launch();
+            launch_chained(true, k_digit_scan, kBins, kSortThreads, 0, s, a.hist, l.row, offs, total);
         }
         if (l.tile == 512) launch_pass<2, true>(a, s);
         else if (l.tile == 1024) launch_pass<4, true>(a, s);
