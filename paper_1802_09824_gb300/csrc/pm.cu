@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(kPmThreads) k_pm_prepare(const float *mass, in
                                                            uint4 *mesh, int64_t mesh16, uint32_t *block_max,
                                                            uint32_t *status)
 {
+    chain_begin();
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = t0; i < mesh16; i += step) mesh[i] = make_uint4(0u, 0u, 0u, 0u);
     uint32_t best = mass ? 0u : __float_as_uint(fabsf(mass_default));
@@ -235,6 +236,7 @@ __global__ void k_pm_deposit(const void *pos, const float *mass, int64_t n, floa
                              double inv_dg, CellScale cs, int N, const uint32_t *block_max, int n_max,
                              uint32_t *mmax_bits, unsigned long long *mesh_q, uint32_t *status)
 {
+    chain_begin();
     uint32_t best = 0;
     for (int b = threadIdx.x; b < n_max; b += kPmThreads) best = max(best, block_max[b]);
     __shared__ uint32_t s_max;
@@ -293,6 +295,7 @@ __global__ void k_pm_deposit(const void *pos, const float *mass, int64_t n, floa
 __global__ void k_pm_unfix(const unsigned long long *mesh_q, int64_t cells, int64_t n, const uint32_t *mmax_bits,
                            float *mesh_r)
 {
+    chain_begin();
     const int kS = pm_scale_exp_block(mmax_bits, n);   // S = 2^kS
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < cells; i += (int64_t)gridDim.x * blockDim.x)
         mesh_r[i] = ll2f_scaled((long long)mesh_q[i], kS);
@@ -319,6 +322,7 @@ __global__ void k_pm_green(float2 *mc, int N, const float *s2, const float *ek, 
 // -grad phi by the 2-point central difference; phi kept in w.
 __global__ void k_pm_grad(const float *phi, int N, float c_half, float4 *mesh_a)
 {
+    chain_begin();
     const uint32_t n = N, nn = n * n, cells = nn * n;   // (N^3 <= 2^30)
     for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < cells; idx += gridDim.x * blockDim.x) {
         const uint32_t r = idx / n, k = idx - r * n, i = r / n, j = r - i * n;
@@ -338,6 +342,7 @@ template <int PT>
 __global__ void k_pm_interp(const void *pos, int64_t n, double L, double inv_dg, CellScale cs, int N,
                             const float4 *mesh_a, float *acc, float *pot, int accumulate, const uint8_t *active)
 {
+    chain_begin();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         if (active && !active[i]) continue;
         bool finite;
@@ -577,15 +582,11 @@ int ph_pm_accel(const void *pos, int pos_type, const float *mass, int64_t n, con
     uint32_t *bmax = mmax + 4;
     const int pblocks = std::min(kPmMaxBlocks, grid_of(std::max<int64_t>(cells / 2, dmass ? n : 0)));
     k_pm_prepare<<<pblocks, kPmThreads, 0, s>>>(dmass, n, mdef, reinterpret_cast<uint4 *>(mq), cells / 2, bmax, st);
-    if (pos_type == PH_F64)
-        k_pm_deposit<PH_F64><<<grid_of(n), kPmThreads, 0, s>>>(dpos, dmass, n, mdef, p.L, inv_dg, cs, N, bmax, pblocks,
-                                                               mmax, mq, st);
-    else
-        k_pm_deposit<PH_F32><<<grid_of(n), kPmThreads, 0, s>>>(dpos, dmass, n, mdef, p.L, inv_dg, cs, N, bmax, pblocks,
-                                                               mmax, mq, st);
+    count_launch();
+    launch_chained(true, pos_type == PH_F64 ? k_pm_deposit<PH_F64> : k_pm_deposit<PH_F32>, grid_of(n), kPmThreads, 0, s,
+                   dpos, dmass, n, mdef, p.L, inv_dg, cs, N, bmax, pblocks, mmax, mq, st);
     float *mr = static_cast<float *>(h->mesh_r.p);
-    k_pm_unfix<<<grid_of(cells), kPmThreads, 0, s>>>(mq, cells, n, mmax, mr);
-    count_launch(3);
+    launch_chained(true, k_pm_unfix, grid_of(cells), kPmThreads, 0, s, mq, cells, n, mmax, mr);
     rc = cufft_check(cufftSetStream(h->plan_r2c, s), "cufftSetStream");
     if (!rc) rc = cufft_check(cufftSetStream(h->plan_c2r, s), "cufftSetStream");
     if (!rc) rc = cufft_check(cufftExecR2C(h->plan_r2c, mr, static_cast<cufftComplex *>(h->mesh_c.p)), "R2C");
@@ -599,13 +600,9 @@ int ph_pm_accel(const void *pos, int pos_type, const float *mass, int64_t n, con
     if (rc) return rc;
     float4 *ma = static_cast<float4 *>(h->mesh_a.p);
     k_pm_grad<<<grid_of(cells), kPmThreads, 0, s>>>(mr, N, (float)(-0.5 / dg), ma);
-    if (pos_type == PH_F64)
-        k_pm_interp<PH_F64><<<grid_of(n), kPmThreads, 0, s>>>(dpos, n, p.L, inv_dg, cs, N, ma, dacc, dpot,
-                                                              accumulate, h->active);
-    else
-        k_pm_interp<PH_F32><<<grid_of(n), kPmThreads, 0, s>>>(dpos, n, p.L, inv_dg, cs, N, ma, dacc, dpot,
-                                                              accumulate, h->active);
-    count_launch(2);
+    count_launch();
+    launch_chained(true, pos_type == PH_F64 ? k_pm_interp<PH_F64> : k_pm_interp<PH_F32>, grid_of(n), kPmThreads, 0, s,
+                   dpos, n, p.L, inv_dg, cs, N, ma, dacc, dpot, accumulate, h->active);
     rc = cuda_check(cudaGetLastError(), "PM kernels");
     if (!rc && host_acc)
         rc = cuda_check(cudaMemcpyAsync(acc, dacc, (size_t)n * 12, cudaMemcpyDeviceToHost, s), "copy acc out");
