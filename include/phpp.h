@@ -106,7 +106,8 @@ extern "C" {
  *             class in the order the pair builder meets the groups) -- the
  *             heaviest groups start first, so the launch ends on short
  *             ones; 1 = plain group order (along the curve).  Same results
- *             (each group is summed by one warp on its own).  The direct
+ *             (a group's list is summed in segments that are added in
+ *             order, whichever warps sum them).  The direct
  *             mode (no stored list) and the active-particle mode take group
  *             order.
  *   theta     opening criterion of the tree part (Sec. 3.3), in [0, 1):

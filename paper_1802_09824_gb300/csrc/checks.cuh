@@ -29,7 +29,7 @@ enum BoundsSite : uint32_t {
     BS_PM_NODE = 12,      // PM: mesh node
     BS_DOM_ROW = 13,      // device exchange: row of the send or receive buffer
     BS_ORDER = 14,        // group order: output slot
-    BS_PP_TASK = 15,      // pair builder and k_pp: task slot of a split group
+    BS_PP_TASK = 15,      // k_pp: task slot of a split group
 };
 
 #ifdef PHPP_BOUNDS_CHECK

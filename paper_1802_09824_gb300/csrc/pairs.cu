@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(kThreads) k_clear_counts(uint32_t *p, int64_t 
 // adds up from the count pass's sums.
 __global__ void __launch_bounds__(kThreads) k_offsets(const int64_t *cnt, const int32_t *n_groups,
                                                       const unsigned long long *chunk_sum, int64_t *off,
-                                                      unsigned long long *work)
+                                                      unsigned long long *work, int64_t *total)
 {
     chain_begin();
     // the PP kernel's queue and counters (a captured step has no other reset)
@@ -344,14 +344,15 @@ __global__ void __launch_bounds__(kThreads) k_offsets(const int64_t *cnt, const 
 #pragma unroll
     for (int k = 0; k < 4; k++) {
         if (g + k <= ng) off[g + k] = e;
+        if (g + k == ng) *total = e;
         e += v[k];
     }
 }
 
 }  // namespace
 
-// Scratch of the queue: the per-key counts and cursors, the number of tasks;
-// then the chunk sums of k_offsets.
+// Scratch of the queue: the per-key counts and cursors, the number of tasks
+// written and needed, all entries (int64); then the chunk sums of k_offsets.
 constexpr int kOrdInts = 2 * kOrdKeys + 4;
 size_t order_temp_bytes(int64_t n) { return kOrdInts * sizeof(int32_t) + (n / kOffChunk + 2) * sizeof(int64_t); }
 
@@ -398,25 +399,20 @@ int ensure_tasks(ph_pairs *pr, int64_t slots, int64_t n)
 
 // The sizing (with `sizing_sync`: read the total, grow the entry buffers)
 // and the fill pass, on stream s.
-static int fill_pairs(ph_pairs *pr, PairArgs &a, const int32_t *n_all, int grid, cudaStream_t s, bool sizing_sync,
-                      int64_t n)
+static int fill_pairs(ph_pairs *pr, PairArgs &a, int grid, cudaStream_t s, bool sizing_sync, int64_t n)
 {
     int rc = 0;
     if (sizing_sync) {
-        // total = group_off[n_groups]; read the count then the total
-        int32_t ng = 0, nt = 0;
-        rc = cuda_check(cudaMemcpyAsync(&nt, a.n_tasks + 1, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "copy n_tasks");
-        if (!rc) rc = cuda_check(cudaMemcpyAsync(&ng, n_all, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "copy n_groups");
+        // tasks written so far, tasks needed, all entries: one read
+        struct {
+            int32_t tasks[2];
+            int64_t total;
+        } need = {{0, 0}, 0};
+        rc = cuda_check(cudaMemcpyAsync(&need, a.n_tasks, sizeof need, cudaMemcpyDeviceToHost, s), "copy pair total");
+        if (!rc) rc = cuda_check(cudaStreamSynchronize(s), "sync pair total");
         if (rc) return rc;
-        rc = cuda_check(cudaStreamSynchronize(s), "sync n_groups");
-        if (rc) return rc;
-        int64_t total = 0;
-        rc = cuda_check(cudaMemcpyAsync(&total, static_cast<const int64_t *>(pr->group_off.p) + ng, sizeof(int64_t),
-                                        cudaMemcpyDeviceToHost, s),
-                        "copy pair total");
-        if (rc) return rc;
-        rc = cuda_check(cudaStreamSynchronize(s), "sync pair total");
-        if (rc) return rc;
+        const int64_t total = need.total;
+        const int32_t nt = need.tasks[1];
         pr->n_pairs = total;
         if (total > pr->capacity) {
             int64_t cap = total + total / 8 + 1024;
@@ -495,8 +491,9 @@ int build_pairs_device(const ph_leaves *lv, ph_pairs *pr, cudaStream_t s, bool s
     // at most one part-filled group a ground cell
     const int64_t most = std::min<int64_t>(n, n / lv->group_size + lv->n_cells);
     launch_chained(true, k_offsets, (int)(most / kOffChunk) + 1, kThreads, 0, s, a.cnt, n_all, a.chunk_sum,
-                   static_cast<int64_t *>(pr->group_off.p), static_cast<unsigned long long *>(pr->work.p));
-    int rc = fill_pairs(pr, a, n_all, grid, s, sizing_sync, n);
+                   static_cast<int64_t *>(pr->group_off.p), static_cast<unsigned long long *>(pr->work.p),
+                   reinterpret_cast<int64_t *>(a.n_tasks + 2));
+    int rc = fill_pairs(pr, a, grid, s, sizing_sync, n);
     if (rc) return rc;
     return cuda_check(cudaGetLastError(), "pair kernels");
 }

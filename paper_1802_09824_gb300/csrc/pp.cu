@@ -509,7 +509,7 @@ __device__ __noinline__ void finish_task(const PPArgs &a, int t, int ni, int i0,
     const int first = t - tk.y;
     const int64_t b = a.group_off[tk.x], e = a.group_off[tk.x + 1];
     const int nseg = (int)(((e < a.cap ? e : a.cap) - b + a.segment - 1) / a.segment);
-    if (lane < G) {
+    if (lane < G && in_bounds(t, a.task_cap, BS_PP_TASK)) {
         float *p = a.task_part + (int64_t)t * 96 + lane;
         __stcg(p, tx);
         __stcg(p + 32, ty);
