@@ -52,12 +52,13 @@ UNIT = "interactions/s"
 
 # FP32 operations per evaluated pair in the exact PP kernel (counted from the
 # source, FADD/FMUL = 1 flop, FFMA = 2, SFU rsqrt/sqrt/ex2 = 0, Kahan adds and
-# the cutoff select not counted): d 3 FADD; r^2 1 FMUL + 2 FFMA; scaled
-# r^2 s2 + eps2s 1 FFMA; its cube 2 FMUL (one SFU rsqrt then gives the
-# inverse cube); t = sqrt(r^2) 2/rcut - 1 1 FFMA; degree-10 Horner 10 FFMA;
-# ex2 argument 1 FMUL; f 1 FMUL; w 2 FMUL; accumulation 3 FFMA
-#   ->  3 FADD + 7 FMUL + 17 FFMA = 44 flop.
-# The ncu counters of one 128^3 launch (sm__sass_thread_inst_executed_op_
+# the cutoff select not counted).  Inverse-distance form (every workload
+# here): d 3 FADD; x = r^2 + eps^2 3 FFMA; y^2 1 FMUL; x y^2 - k 1 FFMA; the
+# softening terms 1 FFMA; their sum 1 FFMA; z 1 FADD; degree-9 Horner 9 FFMA;
+# the weight 1 FFMA and 1 FMUL (mass); accumulation 3 FFMA
+#   ->  4 FADD + 2 FMUL + 19 FFMA = 44 flop,
+# the number of the general form too (3 FADD + 7 FMUL + 17 FFMA), for which
+# the ncu counters of one 128^3 launch (sm__sass_thread_inst_executed_op_
 # {fadd2,fmul2,ffma2}_pred_on) give 44.13 flop per evaluated pair for the
 # packed pair arithmetic (the excess is the padded lanes of partial runs).
 FLOPS_PER_INTERACTION = 44
