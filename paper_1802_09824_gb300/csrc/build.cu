@@ -142,7 +142,10 @@ __global__ void k_keys(const void *pos, int64_t n, const int32_t *box_first, int
                        int key_kind, uint64_t *keys, int32_t *vals, SortCounts sc, uint32_t *status)
 {
     chain_begin();
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    // (the loop's bound is the block's, so that its warps stay whole)
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x; i0 < n; i0 += (int64_t)gridDim.x * blockDim.x) {
+        const bool in = i0 + threadIdx.x < n;
+        const int64_t i = in ? i0 + threadIdx.x : n - 1;
         const int bi = nb > 1 ? find_box(box_first, nb, i) : 0;
         const BoxDev &bx = boxes[bi];
         uint32_t qx = 0, qy = 0, qz = 0;
@@ -169,9 +172,11 @@ __global__ void k_keys(const void *pos, int64_t n, const int32_t *box_first, int
                                                     : interleave3(qx & lm, qy & lm, qz & lm);
         uint64_t boxbits = 3 * T < 64 ? ((uint64_t)bi << (3 * T)) : 0ull;
         const uint64_t key = boxbits | (ground << (3 * b)) | local;
-        keys[i] = key;
-        vals[i] = (int32_t)i;
-        atomicAdd(sc.hist + (int64_t)(key & ((1u << kSortBits) - 1u)) * sc.row + (i >> sc.tile_shift), 1);
+        if (in) {
+            keys[i] = key;
+            vals[i] = (int32_t)i;
+        }
+        count_digit(sc.hist, (int)(key & ((1u << kSortBits) - 1u)) * sc.row + (int)(i >> sc.tile_shift), in);
     }
 }
 

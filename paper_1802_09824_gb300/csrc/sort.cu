@@ -194,16 +194,19 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_pass(PassArgs a)
     // ... then written out slot by slot: consecutive threads write consecutive
     // positions of a digit's run
     const int tile_n = a.n - tile0 < kTile ? (int)(a.n - tile0) : kTile;
-    for (int slot = threadIdx.x; slot < tile_n; slot += kSortThreads) {
-        const uint64_t key = s_key[slot];
+    for (int s0 = 0; s0 < tile_n; s0 += kSortThreads) {
+        const int slot = s0 + threadIdx.x;
+        const bool ok = slot < tile_n;
+        const uint64_t key = ok ? s_key[slot] : 0ull;
         const int d = (int)((key >> a.shift) & (kBins - 1));
-        const int pos = s_off[d] + (slot - s_start[d]);
-        if (in_bounds(pos, a.n, BS_SORT_OUT)) {
+        const int pos = ok ? s_off[d] + (slot - s_start[d]) : 0;
+        const bool in = ok && in_bounds(pos, a.n, BS_SORT_OUT);
+        if (in) {
             a.keys_out[pos] = key;
             a.vals_out[pos] = s_val[slot];
-            if (a.hist_next)
-                atomicAdd(a.hist_next + (int64_t)((key >> (a.shift + kSortBits)) & (kBins - 1)) * a.row + pos / kTile, 1);
         }
+        if (a.hist_next)
+            count_digit(a.hist_next, (int)((key >> (a.shift + kSortBits)) & (kBins - 1)) * a.row + pos / kTile, in);
     }
 }
 

@@ -29,3 +29,22 @@ def test_sorted_order_is_stable(gpu_lib, n):
     np.testing.assert_array_equal(perm, np.argsort(by_row, kind="stable"))
     np.testing.assert_array_equal(np.sort(perm), np.arange(n))
     B.ph_free(lv)
+
+
+def test_equal_digits_share_their_counters(gpu_lib):
+    # particles on a coarse grid (low digits all alike) and in a few cells
+    # (high digits alike), with lanes left over in the last warp
+    import torch
+    B = gpu_lib
+    n = 140_003
+    rng = np.random.default_rng(5)
+    grid = (rng.integers(0, 8, (n, 3)) / 8.0 + 1.0 / 16).astype(np.float32)
+    clump = (0.4 + 0.01 * rng.random((n, 3))).astype(np.float32)
+    for pos in (grid, clump):
+        lv = B.ph_build_leaves(torch.from_numpy(pos).cuda(), None, B.make_params(1.0, 1.0, 1e-3, 0.03, 0.1, 64))
+        v = B.ph_leaves_get_view(lv)
+        perm = v["perm"].cpu().numpy()
+        by_row = np.empty(n, np.uint64)
+        by_row[perm] = v["keys"].cpu().numpy().view(np.uint64)
+        np.testing.assert_array_equal(perm, np.argsort(by_row, kind="stable"))
+        B.ph_free(lv)
