@@ -103,6 +103,9 @@ struct ph_pairs {
     uint8_t *split_of = nullptr; // [n] of a group with several segments: whether it has tasks
     int64_t task_cap = 0;
     int64_t n_tasks = 0;         // host copy (valid after sizing sync)
+    // capacity and task slots the list on the device was made with (a graph's
+    // capture makes room for the lists of its replays)
+    int64_t list_cap = 0, list_task_cap = 0;
     bool ordered = false;
 };
 
@@ -114,6 +117,10 @@ int check_built(const ph_leaves *lv, const ph_pairs *pr);
 
 // Room for `slots` tasks of a list over n particles (pairs.cu).
 int ensure_tasks(ph_pairs *pr, int64_t slots, int64_t n);
+
+// Room for `capacity` entries and `slots` tasks, the list over n particles and
+// its tasks kept (on stream s, which it synchronises); unchanged on failure.
+int grow_pairs(ph_pairs *pr, int64_t capacity, int64_t slots, int64_t n, cudaStream_t s);
 
 // A fingerprint of the device buffers of a leaves (and pairs) handle: their
 // addresses and sizes.  A captured graph holds these addresses; it may only

@@ -397,6 +397,60 @@ int ensure_tasks(ph_pairs *pr, int64_t slots, int64_t n)
     return PH_OK;
 }
 
+int grow_pairs(ph_pairs *pr, int64_t capacity, int64_t slots, int64_t n, cudaStream_t s)
+{
+    const bool more = capacity > pr->capacity, tasks = slots > pr->task_cap;
+    const int64_t cap = pr->capacity, task_cap = pr->task_cap;
+    DevBuf ent, ecnt;
+    ph_pairs t;   // the new tasks' arrays
+    int rc = PH_OK;
+    if (more) {
+        rc = ensure(ent, (size_t)capacity * sizeof(float4));
+        if (!rc) rc = ensure(ecnt, (size_t)capacity);
+        if (!rc && cap > 0)
+            rc = cuda_check(cudaMemcpyAsync(ent.p, pr->entries.p, (size_t)cap * sizeof(float4), cudaMemcpyDeviceToDevice, s),
+                            "move entries");
+        if (!rc && cap > 0)
+            rc = cuda_check(cudaMemcpyAsync(ecnt.p, pr->ecount.p, (size_t)cap, cudaMemcpyDeviceToDevice, s), "move counts");
+    }
+    if (!rc && tasks) {
+        rc = ensure_tasks(&t, slots, n);
+        if (!rc && task_cap > 0)
+            rc = cuda_check(cudaMemcpyAsync(t.tasks, pr->tasks, (size_t)task_cap * sizeof(int2), cudaMemcpyDeviceToDevice, s),
+                            "move tasks");
+        if (!rc && task_cap > 0)
+            rc = cuda_check(cudaMemcpyAsync(t.task_done, pr->task_done, (size_t)task_cap * sizeof(int32_t),
+                                            cudaMemcpyDeviceToDevice, s),
+                            "move task counters");
+        if (!rc && n > 0)
+            rc = cuda_check(cudaMemcpyAsync(t.split_of, pr->split_of, (size_t)n, cudaMemcpyDeviceToDevice, s), "move marks");
+    }
+    if (!rc) rc = cuda_check(cudaStreamSynchronize(s), "sync after growing");
+    if (rc) {
+        release(ent);
+        release(ecnt);
+        release(t.task_mem);
+        return rc;
+    }
+    if (more) {
+        release(pr->entries);
+        release(pr->ecount);
+        pr->entries = ent;
+        pr->ecount = ecnt;
+        pr->capacity = capacity;
+    }
+    if (tasks) {
+        release(pr->task_mem);
+        pr->task_mem = t.task_mem;
+        pr->tasks = t.tasks;
+        pr->task_done = t.task_done;
+        pr->task_part = t.task_part;
+        pr->split_of = t.split_of;
+        pr->task_cap = t.task_cap;
+    }
+    return PH_OK;
+}
+
 // The sizing (with `sizing_sync`: read the total, grow the entry buffers)
 // and the fill pass, on stream s.
 static int fill_pairs(ph_pairs *pr, PairArgs &a, int grid, cudaStream_t s, bool sizing_sync, int64_t n)
@@ -432,6 +486,8 @@ static int fill_pairs(ph_pairs *pr, PairArgs &a, int grid, cudaStream_t s, bool 
     a.ent = static_cast<float4 *>(pr->entries.p);
     a.ecnt = static_cast<uint8_t *>(pr->ecount.p);
     a.cap = pr->capacity;
+    pr->list_cap = pr->capacity;
+    pr->list_task_cap = pr->task_cap;
     launch_chained(!sizing_sync, k_pairs<true>, grid, kThreads, 0, s, a);
     return PH_OK;
 }

@@ -1057,7 +1057,7 @@ static void pp_args(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, PPArg
     a.group_off = pr ? static_cast<const int64_t *>(pr->group_off.p) : nullptr;
     a.entries = pr ? static_cast<const float4 *>(pr->entries.p) : nullptr;
     a.ecount = pr ? static_cast<const uint8_t *>(pr->ecount.p) : nullptr;
-    a.cap = pr ? pr->capacity : 0;
+    a.cap = pr ? pr->list_cap : 0;
     a.order = pr && pr->ordered ? static_cast<const int32_t *>(pr->group_order.p) : nullptr;
     a.group_cell = static_cast<const int32_t *>(lv->group_cell.p);
     a.group_c4 = static_cast<const float4 *>(lv->group_c4.p);
@@ -1080,7 +1080,7 @@ static void pp_args(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, PPArg
     a.task_done = pr ? pr->task_done : nullptr;
     a.task_part = pr ? pr->task_part : nullptr;
     a.split_of = pr ? pr->split_of : nullptr;
-    a.task_cap = pr ? pr->task_cap : 0;
+    a.task_cap = pr ? pr->list_task_cap : 0;
 }
 
 template <bool kLearned, int kMinBlocks, int kSplit, bool kUniform>
