@@ -746,9 +746,11 @@ static double one_minus_f_over_u3(double v)
 // polynomial P in x at the zeros of the weighted minimax error curve for
 // U = 2.25 (weight x^(3/2): the error in units of the Newtonian term), scaled
 // to [0, U^2].  kappa = 0.46 instead of the Taylor 0.375 evens the rest out
-// over r ~ eps.  Error in those units: 8e-8 at U = 2.25, 1.2e-7 at U = 2.3,
-// and 1.1e-7 at r < eps for eps = 2R_s / 64 (the form it replaced: 3.5e-7
-// from its degree-10 polynomial and ex2).
+// over r ~ eps.  Error in units of the Newtonian term: 8e-8 at U = 2.25, 1.2e-7
+// at U = 2.3, and 1.1e-7 at r < eps for eps = 2R_s / 64.  The general form's
+// 3.5e-7 (its degree-10 polynomial and ex2) is relative to the weight, which is
+// f = 0.0175 of the Newtonian term at the cutoff for U = 2.25; in FP32 no fit
+// changes that, since the terms subtracted here are rounded (dense_group).
 // The kernel evaluates (1 - k) W = Y (y (x Y - k) + b1' + b2' Y) + P', with
 // y = rsqrt(x), Y = y^2 and k = 5/3: (x Y - k) / (1 - k) = 1 + 1.5 (1 - x Y)
 // corrects the three-fold error of an SFU rsqrt in y^3 to second order.  k is

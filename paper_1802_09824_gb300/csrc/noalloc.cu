@@ -163,7 +163,7 @@ extern "C" int ph_accel_noalloc(const float *d_pos, const float *d_mass, int64_t
     if (p.level_bits != 0 && p.level_bits != 1 && p.level_bits != 3) return fail(PH_ERR_ARG, "level_bits must be 0, 1 or 3");
     if (p.pp_variant != 0 && p.pp_variant != 1) return fail(PH_ERR_ARG, "pp_variant must be 0 or 1");
     if (poly_degree_for(p.rcut / (2.0 * p.rs)) < 0) return fail(PH_ERR_ARG, "rcut/rs = %g above the supported 9.2", p.rcut / p.rs);
-    const int deg = exact_degree_for(&p, 1);
+    const int deg = exact_degree_for(&p, &n, 1);
     const int g = ground_level(p.L, p.rcut);
     const int nside = 1 << g;
     const int cells = nside * nside * nside;

@@ -27,6 +27,7 @@ struct TraceRange {
 // ---------------------------------------------------------------- limits
 constexpr int kMaxPoly = 16;          // highest degree of the factor polynomial
 constexpr int kInvDeg = 9;            // degree of the inverse-distance form's polynomial
+constexpr int kInvGeneral = 10;       // of the general form's where that form holds (poly_degree_for)
 constexpr float kInvK = 5.f / 3.f;    // its constant 5/3 as the FP32 number the kernel subtracts
 constexpr int kMaxLeaf = 256;         // largest leaf_max accepted
 constexpr int kGroundMax = 7;         // N_side <= 2^7 per box
@@ -67,8 +68,8 @@ struct BoxDev {
     float L_up;        // smallest FP32 number >= L: an FP32 x is below L iff x < L_up
     float c_acc;       // 1 / theta of the tree part (infinite: every leaf pair by PP)
     // The exact kernel's inverse-distance form of the factor (fit_inverse_form;
-    // used where inverse_form_ok holds for every box): lengths scaled by the
-    // power of two sc = sqrt(s2), x = sc^2 (r^2 + eps^2), z = x + inv_zc.
+    // for dense groups where inverse_form_ok holds for every box): lengths scaled
+    // by the power of two sc = sqrt(s2), x = sc^2 (r^2 + eps^2), z = x + inv_zc.
     float sc;
     float inv_poly[kInvDeg + 1];
     float inv_b1, inv_b2, inv_zc;
@@ -99,10 +100,11 @@ int poly_degree_for(double U);
 // box (fit_inverse_form); api.cu.
 bool inverse_form_ok(const struct ph_params &p);
 
-// Degree of the exact kernel's polynomial for these boxes: kInvDeg (the
-// inverse-distance form) where every box allows it, else the largest
-// poly_degree_for; api.cu.
-int exact_degree_for(const struct ph_params *p, int n_boxes);
+// Degree of the exact kernel's polynomial for boxes of n[b] particles: kInvDeg
+// where every box allows the inverse-distance form and they are dense on the
+// whole (dense groups take that form, the others the general one of degree
+// kInvGeneral), else the largest poly_degree_for; api.cu.
+int exact_degree_for(const struct ph_params *p, const int64_t *n, int n_boxes);
 
 // The device record of one box (constants of the build, the pair builder and
 // the PP kernel) from its parameters; api.cu.

@@ -14,12 +14,13 @@
 //
 // Per pair (Eq. (split), Plummer factor, hard cutoff):
 //   r2 = |d|^2,  w = m_j f(r) / (r2 + eps^2)^{3/2}  if r2 < rcut^2 else 0
-// in one of two forms: the inverse-distance form, the Newtonian term minus a
-// polynomial in r2 + eps^2 (one SFU rsqrt; see interact2), or, for boxes
-// outside its range, f(r) = 2^(r2 c_e) h(t), t = 2r / rcut - 1, h a
-// degree-NPOLY polynomial, with rsqrt, sqrt and ex2 on the SFU.  Partial sums
-// over runs of 16 sources are added to the total with Kahan compensation.
+// in one of two forms: f(r) = 2^(r2 c_e) h(t), t = 2r / rcut - 1, h a
+// degree-NPOLY polynomial, with rsqrt, sqrt and ex2 on the SFU, or, for dense
+// groups of boxes in its range (dense_group), the inverse-distance form, the
+// Newtonian term minus a polynomial in r2 + eps^2 with one SFU rsqrt.  Partial
+// sums over runs of 16 sources are added to the total with Kahan compensation.
 #include <cstring>
+#include <type_traits>
 
 #include "factor.cuh"
 #include "handles.cuh"
@@ -50,9 +51,15 @@ constexpr int kJBuf = 256;      // staged sources per warp (even)
 struct PairConsts {
     f2_t poly[kMaxPoly + 1];
     f2_t s2, eps2s, c_t, c_e, m1;
-    float rcut2, rfilt2;   // scaled by sc^2 in the inverse-distance form
-    f2_t zc, b1, b2, m53;  // inverse-distance form (poly holds its polynomial)
-    float sc;              // length scale of the staged sources (1 in the general form)
+    float rcut2, rfilt2;
+};
+
+// Those of the inverse-distance form (lengths scaled by the power of two sc).
+struct InvConsts {
+    f2_t poly[kInvDeg + 1];
+    f2_t eps2s, zc, b1, b2, m53;
+    float cut, rfilt2;     // rcut^2 + eps^2 and the filter's radius squared, scaled by sc^2
+    float sc;
 };
 
 struct PPArgs {
@@ -77,6 +84,7 @@ struct PPArgs {
     // constants shared by every box (the uniform kernels read them straight
     // from the parameter bank instead of holding them in registers)
     PairConsts uc;
+    InvConsts ui;
     // the leaf-pair walk of the direct mode (no stored list)
     const int32_t *group_cell;       // global ground cell of each group
     const float4 *group_c4;          // group box centre in its cell frame
@@ -96,33 +104,75 @@ struct PPArgs {
     const uint8_t *split_of;
     int64_t task_cap;
     int segment;                     // entries per segment
-    bool inverse;                    // the exact kernel runs the inverse-distance form (count kernel)
+    bool inverse;                    // the exact kernel's dense groups take the inverse-distance form (count kernel)
     const int32_t *order;            // queue slot -> group (groups by decreasing cost), or NULL
 };
 
 // The constants of a group's box (boxes with different constants).
-template <int NPOLY>
+template <int N>
 __device__ __forceinline__ void box_consts(const BoxDev &bx, PairConsts &c)
 {
-    constexpr bool inv = NPOLY == kInvDeg;
-    const float *p = inv ? bx.inv_poly : bx.poly;
 #pragma unroll
-    for (int q = 0; q <= NPOLY; q++) c.poly[q] = pk(p[q], p[q]);
+    for (int q = 0; q <= N; q++) c.poly[q] = pk(bx.poly[q], bx.poly[q]);
+    c.s2 = pk(bx.s2, bx.s2);
     c.eps2s = pk(bx.eps2s, bx.eps2s);
-    c.rcut2 = inv ? bx.inv_cut : bx.rcut2;
-    c.rfilt2 = inv ? bx.rfilt2 * bx.s2 : bx.rfilt2;
-    c.sc = inv ? bx.sc : 1.f;
-    if (inv) {
-        c.zc = pk(bx.inv_zc, bx.inv_zc);
-        c.b1 = pk(bx.inv_b1, bx.inv_b1);
-        c.b2 = pk(bx.inv_b2, bx.inv_b2);
-        c.m53 = pk(-kInvK, -kInvK);
-    } else {
-        c.s2 = pk(bx.s2, bx.s2);
-        c.c_t = pk(bx.c_t, bx.c_t);
-        c.c_e = pk(bx.c_e, bx.c_e);
-        c.m1 = pk(-1.f, -1.f);
-    }
+    c.c_t = pk(bx.c_t, bx.c_t);
+    c.c_e = pk(bx.c_e, bx.c_e);
+    c.m1 = pk(-1.f, -1.f);
+    c.rcut2 = bx.rcut2;
+    c.rfilt2 = bx.rfilt2;
+}
+
+template <int N>
+__device__ __forceinline__ void box_consts(const BoxDev &bx, InvConsts &c)
+{
+#pragma unroll
+    for (int q = 0; q <= kInvDeg; q++) c.poly[q] = pk(bx.inv_poly[q], bx.inv_poly[q]);
+    c.eps2s = pk(bx.eps2s, bx.eps2s);
+    c.zc = pk(bx.inv_zc, bx.inv_zc);
+    c.b1 = pk(bx.inv_b1, bx.inv_b1);
+    c.b2 = pk(bx.inv_b2, bx.inv_b2);
+    c.m53 = pk(-kInvK, -kInvK);
+    c.cut = bx.inv_cut;
+    c.rfilt2 = bx.rfilt2 * bx.s2;
+    c.sc = bx.sc;
+}
+
+// The constants of a form: of the general form of degree N, or (N = kInvDeg) of
+// the inverse-distance form.
+template <int N>
+struct FormConsts {
+    using T = PairConsts;
+    static __device__ __forceinline__ const T &uniform(const PPArgs &a) { return a.uc; }
+    static __device__ __forceinline__ float scale(const T &) { return 1.f; }
+};
+template <>
+struct FormConsts<kInvDeg> {
+    using T = InvConsts;
+    static __device__ __forceinline__ const T &uniform(const PPArgs &a) { return a.ui; }
+    static __device__ __forceinline__ float scale(const T &c) { return c.sc; }
+};
+
+// Whether a group (half extents h, ni targets) takes the inverse-distance form.
+// That form's error is a fixed part of a pair's Newtonian term, of which the
+// weight leaves 1/57 at the cutoff (rcut = 4.5 R_s): 5e-6 of the weight there,
+// where the general form keeps 2e-7 everywhere.  With many sources the near
+// ones outweigh that, a target with a few distant ones keeps it.  Relative force
+// error, 99th percentile, of sources spread evenly in the sphere (general /
+// inverse-distance): 1 source 6.1e-7 / 8.9e-6, 5 7.4e-7 / 2.9e-6, 20 7.5e-7 /
+// 9.0e-7, 30 7.4e-7 / 6.7e-7, 47 9.0e-7 / 6.2e-7, 93 7.9e-7 / 5.0e-7, 700 8.3e-7 /
+// 4.2e-7 (median and 2-norm: below the general form's from 20 on).  So it is
+// left to groups of 16 targets and more whose own box is dense enough for 60
+// sources within the cutoff, ni (4 pi / 3) rcut^3 >= 60 V, V the cube of the
+// same diagonal: (|h| / rcut)^6 <= 2.05e-3 ni^2.  A clump of just such a group
+// and nothing else: 32 targets 5.9e-7 / 5.0e-7, 16 5.4e-7 / 4.6e-7.  (The box's
+// mean would leave out voids and the edges of haloes.)  Rounded step by step, so
+// that every kernel decides alike.
+constexpr int kDenseMin = 16;
+__device__ __forceinline__ bool dense_group(const float4 h, int ni, float rcut2)
+{
+    const float q = __fdiv_rn(__fmaf_rn(h.z, h.z, __fmaf_rn(h.y, h.y, __fmul_rn(h.x, h.x))), rcut2);
+    return ni >= kDenseMin && __fmul_rn(__fmul_rn(q, q), q) <= __fmul_rn(2.05e-3f, (float)(ni * ni));
 }
 
 struct Kahan3 {
@@ -139,38 +189,40 @@ struct Kahan3 {
 // Two sources (A = x0 x1 y0 y1, B = z0 z1 m0 m1) against one target: add
 // m_j f(r) d / (r^2 + eps^2)^{3/2} into the pair accumulators.
 //
-// NPOLY = kInvDeg is the inverse-distance form (fit_inverse_form; lengths
-// scaled by sc): 25 packed FP32 instructions and one SFU operation per pair,
-// where the general form (NPOLY = 10 and up) takes 27 and three.  Bound by
-// the FMA pipe (ncu: 80 % busy): a loop over staged pairs alone took 66.2
-// cycles per two pairs and warp, 69.3 with the general form.  2-norm of the
-// force error against FP64 sums: 1.1e-7 of the forces' on uniform boxes
-// (general form 1.6e-7), 4.3e-8 on halo mixtures (9.0e-8).
+// The inverse-distance form (fit_inverse_form; lengths scaled by sc): 25 packed
+// FP32 instructions and one SFU operation per pair, where the general form takes
+// 27 and three.  Bound by the FMA pipe (ncu: 80 % busy): a loop over staged
+// pairs alone took 66.2 cycles per two pairs and warp, 69.3 with the general form.
+template <int NPOLY>
+__device__ __forceinline__ void interact2(const float4 a, const float4 b, const f2_t xi, const f2_t yi, const f2_t zi,
+                                          const InvConsts &c, f2_t &px, f2_t &py, f2_t &pz)
+{
+    const f2_t dx = sub2(pk(a.x, a.y), xi), dy = sub2(pk(a.z, a.w), yi), dz = sub2(pk(b.x, b.y), zi);
+    f2_t x = fma2(dx, dx, c.eps2s);
+    x = fma2(dy, dy, x);
+    x = fma2(dz, dz, x);
+    const f2_t y = pk(rsqrt_sfu(lo_of(x)), rsqrt_sfu(hi_of(x)));
+    const f2_t Y = mul2(y, y);
+    const f2_t z = add2(x, c.zc);
+    f2_t h = c.poly[kInvDeg];
+#pragma unroll
+    for (int q = kInvDeg - 1; q >= 0; q--) h = fma2(h, z, c.poly[q]);
+    const f2_t q = fma2(fma2(x, Y, c.m53), y, fma2(c.b2, Y, c.b1));
+    const f2_t w = mul2(pk(b.z, b.w), fma2(q, Y, h));
+    const float w0 = lo_of(x) < c.cut ? lo_of(w) : 0.f;
+    const float w1 = hi_of(x) < c.cut ? hi_of(w) : 0.f;
+    const f2_t wm = pk(w0, w1);
+    px = fma2(wm, dx, px);
+    py = fma2(wm, dy, py);
+    pz = fma2(wm, dz, pz);
+}
+
+// The general form.
 template <int NPOLY>
 __device__ __forceinline__ void interact2(const float4 a, const float4 b, const f2_t xi, const f2_t yi, const f2_t zi,
                                           const PairConsts &c, f2_t &px, f2_t &py, f2_t &pz)
 {
     const f2_t dx = sub2(pk(a.x, a.y), xi), dy = sub2(pk(a.z, a.w), yi), dz = sub2(pk(b.x, b.y), zi);
-    if (NPOLY == kInvDeg) {
-        f2_t x = fma2(dx, dx, c.eps2s);
-        x = fma2(dy, dy, x);
-        x = fma2(dz, dz, x);
-        const f2_t y = pk(rsqrt_sfu(lo_of(x)), rsqrt_sfu(hi_of(x)));
-        const f2_t Y = mul2(y, y);
-        const f2_t z = add2(x, c.zc);
-        f2_t h = c.poly[kInvDeg];
-#pragma unroll
-        for (int q = kInvDeg - 1; q >= 0; q--) h = fma2(h, z, c.poly[q]);
-        const f2_t q = fma2(fma2(x, Y, c.m53), y, fma2(c.b2, Y, c.b1));
-        const f2_t w = mul2(pk(b.z, b.w), fma2(q, Y, h));
-        const float w0 = lo_of(x) < c.rcut2 ? lo_of(w) : 0.f;
-        const float w1 = hi_of(x) < c.rcut2 ? hi_of(w) : 0.f;
-        const f2_t wm = pk(w0, w1);
-        px = fma2(wm, dx, px);
-        py = fma2(wm, dy, py);
-        pz = fma2(wm, dz, pz);
-        return;
-    }
     f2_t r2 = mul2(dx, dx);
     r2 = fma2(dy, dy, r2);
     r2 = fma2(dz, dz, r2);
@@ -210,9 +262,9 @@ __device__ __forceinline__ void interact2(const float4 a, const float4 b, const 
 constexpr int kRun = PHPP_PP_RUN;
 constexpr int kUnroll = PHPP_PP_UNROLL;
 
-template <int NPOLY, int kSplit>
+template <int NPOLY, int kSplit, typename Consts>
 __device__ __forceinline__ void sum_buffer(const float4 *A, const float4 *B, int npair, int h, const f2_t xi,
-                                           const f2_t yi, const f2_t zi, const PairConsts &c, Kahan3 &k)
+                                           const f2_t yi, const f2_t zi, const Consts &c, Kahan3 &k)
 {
     const int nstep = npair / kSplit;
     int s = 0;
@@ -534,6 +586,138 @@ __device__ __noinline__ void finish_task(const PPArgs &a, int t, int ni, int i0,
     }
 }
 
+// The sum over one run of a group's list, entries [e0, e1): what every lane has
+// for its target (all kSplit lanes of a target the same), and the sources summed.
+struct ListSum {
+    float x, y, z;
+    int staged;
+};
+
+// The warp's memory: the staging buffer's two halves, the learned factor's ring
+// and the factor or layer table.
+struct WarpMem {
+    float4 *A, *B, *ring;
+    const float4 *dyn;
+};
+
+template <int N, bool kLearned, int kSplit, bool kUniform, bool kTable, bool kApart = false>
+__device__ __forceinline__ ListSum sum_list(const PPArgs &a, const BoxDev &bx, const WarpMem m, const MlpLane &L, int64_t e0,
+                                            int64_t e1, int i0, int ni, float4 gh)
+{
+    constexpr int G = 32 / kSplit;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int ti = lane & (G - 1), hs = lane / G;   // target slot, source slot
+    float4 *const A = m.A, *const Bq = m.B, *const ring = m.ring;
+    const float4 *const dyn = m.dyn;
+    float *const Af = reinterpret_cast<float *>(A), *const Bf = reinterpret_cast<float *>(Bq);
+    int staged = 0;
+    typename FormConsts<N>::T cl;
+    if (!kUniform) box_consts<N>(bx, cl);
+    else if (kApart) cl = FormConsts<N>::uniform(a);   // (a is no parameter bank there)
+    const auto &c = kUniform && !kApart ? FormConsts<N>::uniform(a) : cl;
+    const float rf2 = c.rfilt2;
+    float4 xi4 = ti < ni ? a.pos_group[i0 + ti] : make_float4(0.f, 0.f, 0.f, 0.f);
+    // the inverse-distance form works in lengths scaled by a power of two
+    const float sc = FormConsts<N>::scale(c);
+    if (N == kInvDeg) {
+        gh.x *= sc; gh.y *= sc; gh.z *= sc;
+        xi4.x *= sc; xi4.y *= sc; xi4.z *= sc;
+    }
+    const f2_t xi = pk(xi4.x, xi4.x), yi = pk(xi4.y, xi4.y), zi = pk(xi4.z, xi4.z);
+    Kahan3 k;
+    int nbuf = 0;
+    LearnedQueue lq;
+    if (kLearned) {
+        lq.q = ring;
+        lq.l1 = dyn;
+        if (lane == 0) lq.q[kLQ] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    // Entries are taken 32 at a time; each round loads 32 concatenated
+    // source particles of the batch, one per lane.
+    for (int64_t eb = e0; eb < e1; eb += 32) {
+        EntryBatch bt;
+        bt.load(a, eb, e1, lane);
+        int before = 0;
+        for (int q0 = 0; q0 < bt.total; q0 += 32) {
+            Round cur;
+            cur.issue(a, bt, q0, lane, before);
+            float4 p = cur.p;
+            bool keep = false;
+            if (cur.valid) {
+                // sc (p + o), rounded once: sc is a power of two
+                p.x = __fmaf_rn(p.x, sc, cur.ox * sc);
+                p.y = __fmaf_rn(p.y, sc, cur.oy * sc);
+                p.z = __fmaf_rn(p.z, sc, cur.oz * sc);
+                const float qx = fmaxf(fabsf(p.x) - gh.x, 0.f);
+                const float qy = fmaxf(fabsf(p.y) - gh.y, 0.f);
+                const float qz = fmaxf(fabsf(p.z) - gh.z, 0.f);
+                keep = qx * qx + qy * qy + qz * qz < rf2;
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, keep);
+            const int nk = __popc(bal);
+            if (nbuf + nk > kJBuf) {
+                const int padded = pad_sources<kSplit>(Af, Bf, nbuf, lane);
+                __syncwarp();
+                if constexpr (kLearned)
+                    sum_buffer_learned<kSplit>(A, Bq, padded, hs, xi4, ti < ni, bx.eps2, bx.rcut2, bx.c_v, L, lq, k);
+                else if constexpr (kTable)
+                    sum_buffer_table<kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, reinterpret_cast<const float2 *>(dyn),
+                                             pk(a.tab_scale2, a.tab_scale2), k);
+                else
+                    sum_buffer<N, kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, k);
+                staged += nbuf;
+                nbuf = 0;
+                __syncwarp();
+            }
+            const int idx = nbuf + __popc(bal & lt);
+            if (keep && in_bounds(idx, kJBuf, BS_PP_STAGE)) {
+                const int mm = idx >> 1, sl = idx & 1;
+                Af[mm * 4 + sl] = p.x;
+                Af[mm * 4 + 2 + sl] = p.y;
+                Bf[mm * 4 + sl] = p.z;
+                Bf[mm * 4 + 2 + sl] = p.w;
+            }
+            nbuf += nk;
+        }
+    }
+    const int padded = pad_sources<kSplit>(Af, Bf, nbuf, lane);
+    __syncwarp();
+    if constexpr (kLearned)
+        sum_buffer_learned<kSplit>(A, Bq, padded, hs, xi4, ti < ni, bx.eps2, bx.rcut2, bx.c_v, L, lq, k);
+    else if constexpr (kTable)
+        sum_buffer_table<kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, reinterpret_cast<const float2 *>(dyn), pk(a.tab_scale2, a.tab_scale2), k);
+    else
+        sum_buffer<N, kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, k);
+    staged += nbuf;
+    if (kLearned && lq.n > 0) {
+        // the queue's last, partial batch
+        float px = 0.f, py = 0.f, pz = 0.f;
+        learned_flush(lq, lq.n, lane, bx.eps2, bx.c_v, L, px, py, pz);
+        k.add(px, py, pz);
+    }
+    __syncwarp();
+    // the kSplit source slots of a target add up their compensated totals
+    float tx = k.sx - k.cx, ty = k.sy - k.cy, tz = k.sz - k.cz;
+#pragma unroll
+    for (int o = G; o < 32; o <<= 1) {
+        tx += __shfl_xor_sync(0xffffffffu, tx, o);
+        ty += __shfl_xor_sync(0xffffffffu, ty, o);
+        tz += __shfl_xor_sync(0xffffffffu, tz, o);
+    }
+    return ListSum{tx, ty, tz, staged};
+}
+
+// The general form's sums in a kernel whose loops are the inverse-distance
+// form's.  Inlined there, the two forms cost each other 1.6 % (128^3 lattice step
+// 4085 us, as a call 4005; everything in the general form 4144).
+template <int N, int kSplit, bool kUniform>
+__device__ __noinline__ ListSum sum_list_apart(const PPArgs &a, const BoxDev &bx, const WarpMem m, int64_t e0, int64_t e1,
+                                               int i0, int ni, float4 gh)
+{
+    return sum_list<N, false, kSplit, kUniform, false, true>(a, bx, m, MlpLane(), e0, e1, i0, ni, gh);
+}
+
 // Source staging and summation for one target group.  Entries are taken 32
 // at a time, one per lane; the lanes' leaf sizes are prefix-summed and the
 // concatenated source particles are loaded 32 per round, each lane finding
@@ -549,15 +733,13 @@ template <int NPOLY, bool kLearned, int kMinBlocks, int kSplit, bool kUniform, b
 __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
 {
     chain_begin();
+    constexpr bool kBoth = NPOLY == kInvDeg;         // both forms, chosen per group
+    constexpr int kDeg = kBoth ? kInvGeneral : NPOLY;   // degree of the general form
     __shared__ float4 sA[kPPWarps][kJBuf / 2];
     __shared__ float4 sB[kPPWarps][kJBuf / 2];
     __shared__ float4 sQ[kLearned ? kPPWarps : 1][kLearned ? kLQ + 1 : 1];   // learned: the pair queue
     extern __shared__ float4 sDyn[];   // dynamic: the factor table (kTable) or layer 1's table (kLearned)
-    float2 *const sTab = reinterpret_cast<float2 *>(sDyn);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const unsigned lt = (1u << lane) - 1u;
-    float4 *A = sA[w], *Bq = sB[w];
-    float *Af = reinterpret_cast<float *>(A), *Bf = reinterpret_cast<float *>(Bq);
     const int ng = *a.n_groups;
     const int nt = *a.n_tasks < a.task_cap ? *a.n_tasks : (int)a.task_cap;
     unsigned long long inter = 0, staged = 0;
@@ -568,7 +750,8 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
         __syncthreads();
     }
     if (kTable) {
-        for (int i = threadIdx.x; i <= kTabN; i += blockDim.x) sTab[i] = a.table[i];
+        float2 *const tab = reinterpret_cast<float2 *>(sDyn);
+        for (int i = threadIdx.x; i <= kTabN; i += blockDim.x) tab[i] = a.table[i];
         __syncthreads();
     }
     // The queue: the tasks of split groups, then the other groups in their
@@ -613,93 +796,122 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
                 continue;   // its tasks came first
             }
         }
-        PairConsts cl;
-        if (!kUniform) box_consts<NPOLY>(bx, cl);
-        const PairConsts &c = kUniform ? a.uc : cl;
-        const float rf2 = c.rfilt2;
         constexpr int G = 32 / kSplit;
         const int ti = lane & (G - 1), hs = lane / G;   // target slot, source slot
-        float4 xi4 = ti < ni ? a.pos_group[i0 + ti] : make_float4(0.f, 0.f, 0.f, 0.f);
-        // the inverse-distance form works in lengths scaled by a power of two
-        const float sc = NPOLY == kInvDeg ? c.sc : 1.f;
-        if (NPOLY == kInvDeg) {
-            gh.x *= sc; gh.y *= sc; gh.z *= sc;
-            xi4.x *= sc; xi4.y *= sc; xi4.z *= sc;
+        const WarpMem mem{sA[w], sB[w], kLearned ? sQ[kLearned ? w : 0] : nullptr, kLearned || kTable ? sDyn : nullptr};
+        const bool inv = kBoth && dense_group(gh, ni, kUniform ? a.uc.rcut2 : bx.rcut2);
+        ListSum s;
+        if constexpr (kBoth)
+            s = inv ? sum_list<kInvDeg, false, kSplit, kUniform, false>(a, bx, mem, L, e0, e1, i0, ni, gh)
+                    : sum_list_apart<kDeg, kSplit, kUniform>(a, bx, mem, e0, e1, i0, ni, gh);
+        else
+            s = sum_list<kDeg, kLearned, kSplit, kUniform, kTable>(a, bx, mem, L, e0, e1, i0, ni, gh);
+        inter += (unsigned long long)s.staged * ni;
+        staged += s.staged;
+        const float Gc = kLearned ? bx.G : kBoth && inv ? bx.inv_g : bx.c_g;
+        if (task) {
+            finish_task<G>(a, t, ni, i0, Gc, s.x, s.y, s.z);
+        } else if (hs == 0 && ti < ni) {
+            const int64_t o = a.perm[i0 + ti];
+            a.acc[3 * o + 0] = Gc * s.x;
+            a.acc[3 * o + 1] = Gc * s.y;
+            a.acc[3 * o + 2] = Gc * s.z;
         }
-        const f2_t xi = pk(xi4.x, xi4.x), yi = pk(xi4.y, xi4.y), zi = pk(xi4.z, xi4.z);
-        Kahan3 k;
-        int nbuf = 0;
-        LearnedQueue lq;
-        if (kLearned) {
-            lq.q = sQ[kLearned ? w : 0];
-            lq.l1 = sDyn;
-            if (lane == 0) lq.q[kLQ] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        // Entries are taken 32 at a time; each round loads 32 concatenated
-        // source particles of the batch, one per lane.
-        for (int64_t eb = e0; eb < e1; eb += 32) {
-            EntryBatch bt;
-            bt.load(a, eb, e1, lane);
-            int before = 0;
-            for (int q0 = 0; q0 < bt.total; q0 += 32) {
-                Round cur;
-                cur.issue(a, bt, q0, lane, before);
-                float4 p = cur.p;
-                bool keep = false;
-                if (cur.valid) {
-                    // sc (p + o), rounded once: sc is a power of two
-                    p.x = __fmaf_rn(p.x, sc, cur.ox * sc);
-                    p.y = __fmaf_rn(p.y, sc, cur.oy * sc);
-                    p.z = __fmaf_rn(p.z, sc, cur.oz * sc);
-                    const float qx = fmaxf(fabsf(p.x) - gh.x, 0.f);
-                    const float qy = fmaxf(fabsf(p.y) - gh.y, 0.f);
-                    const float qz = fmaxf(fabsf(p.z) - gh.z, 0.f);
-                    keep = qx * qx + qy * qy + qz * qz < rf2;
-                }
-                const unsigned bal = __ballot_sync(0xffffffffu, keep);
-                const int nk = __popc(bal);
-                if (nbuf + nk > kJBuf) {
-                    const int padded = pad_sources<kSplit>(Af, Bf, nbuf, lane);
-                    __syncwarp();
-                    if (kLearned)
-                        sum_buffer_learned<kSplit>(A, Bq, padded, hs, xi4, ti < ni, bx.eps2, bx.rcut2, bx.c_v, L, lq, k);
-                    else if (kTable)
-                        sum_buffer_table<kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, sTab,
-                                                 pk(a.tab_scale2, a.tab_scale2), k);
-                    else
-                        sum_buffer<NPOLY, kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, k);
-                    inter += (unsigned long long)nbuf * ni;
-                    staged += nbuf;
-                    nbuf = 0;
-                    __syncwarp();
-                }
-                const int idx = nbuf + __popc(bal & lt);
-                if (keep && in_bounds(idx, kJBuf, BS_PP_STAGE)) {
-                    const int m = idx >> 1, sl = idx & 1;
-                    Af[m * 4 + sl] = p.x;
-                    Af[m * 4 + 2 + sl] = p.y;
-                    Bf[m * 4 + sl] = p.z;
-                    Bf[m * 4 + 2 + sl] = p.w;
-                }
-                nbuf += nk;
+    }
+    if (lane == 0 && inter) {
+        atomicAdd(a.n_inter, inter);
+        atomicAdd(a.n_staged, staged);
+    }
+}
+
+// The warp's memory of the direct mode: the staging buffer's halves, the cell
+// runs, the queue of found entries and the sum over the segments done.
+struct WalkMem {
+    float4 *A, *B;
+    int2 *run;
+    float4 *qent;
+    int *qcnt;
+    Kahan3 *fold;
+};
+
+// The sum of one group: its leaf pairs found, staged and summed segment by segment.
+template <int N, int kSplit, bool kUniform>
+__device__ __forceinline__ ListSum walk_group(const PPArgs &a, const BoxDev &bx, const WalkMem m, int g, int i0, int ni,
+                                              const float4 gh0)
+{
+    constexpr int G = 32 / kSplit;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int ti = lane & (G - 1), hs = lane / G;   // target slot, source slot
+    float4 *const A = m.A, *const Bq = m.B;
+    float *const Af = reinterpret_cast<float *>(A), *const Bf = reinterpret_cast<float *>(Bq);
+    int staged = 0;
+    float4 gh = gh0;
+    typename FormConsts<N>::T cl;
+    if (!kUniform) box_consts<N>(bx, cl);
+    const auto &c = kUniform ? FormConsts<N>::uniform(a) : cl;
+    const float rf2 = c.rfilt2;   // of the staged (scaled) sources
+    float4 xi4 = ti < ni ? a.pos_group[i0 + ti] : make_float4(0.f, 0.f, 0.f, 0.f);
+    // the inverse-distance form works in lengths scaled by a power of two
+    const float sc = FormConsts<N>::scale(c);
+    if (N == kInvDeg) {
+        gh.x *= sc; gh.y *= sc; gh.z *= sc;
+        xi4.x *= sc; xi4.y *= sc; xi4.z *= sc;
+    }
+    const f2_t xi = pk(xi4.x, xi4.x), yi = pk(xi4.y, xi4.y), zi = pk(xi4.z, xi4.z);
+    Kahan3 k;
+    int nbuf = 0;
+    // The source particles of a batch of (up to) 32 entries, one per lane:
+    // each round loads 32 concatenated particles, one per lane.
+    auto stage_batch = [&](const EntryBatch &bt) {
+        int before = 0;
+        for (int q0 = 0; q0 < bt.total; q0 += 32) {
+            Round cur;
+            cur.issue(a, bt, q0, lane, before);
+            float4 p = cur.p;
+            bool keep = false;
+            if (cur.valid) {
+                // sc (p + o), rounded once: sc is a power of two
+                p.x = __fmaf_rn(p.x, sc, cur.ox * sc);
+                p.y = __fmaf_rn(p.y, sc, cur.oy * sc);
+                p.z = __fmaf_rn(p.z, sc, cur.oz * sc);
+                const float qx = fmaxf(fabsf(p.x) - gh.x, 0.f);
+                const float qy = fmaxf(fabsf(p.y) - gh.y, 0.f);
+                const float qz = fmaxf(fabsf(p.z) - gh.z, 0.f);
+                keep = qx * qx + qy * qy + qz * qz < rf2;
             }
+            const unsigned bal = __ballot_sync(0xffffffffu, keep);
+            const int nk = __popc(bal);
+            if (nbuf + nk > kJBuf) {
+                const int padded = pad_sources<kSplit>(Af, Bf, nbuf, lane);
+                __syncwarp();
+                sum_buffer<N, kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, k);
+                staged += nbuf;
+                nbuf = 0;
+                __syncwarp();
+            }
+            const int idx = nbuf + __popc(bal & lt);
+            if (keep && in_bounds(idx, kJBuf, BS_PP_STAGE)) {
+                const int mm = idx >> 1, sl = idx & 1;
+                Af[mm * 4 + sl] = p.x;
+                Af[mm * 4 + 2 + sl] = p.y;
+                Bf[mm * 4 + sl] = p.z;
+                Bf[mm * 4 + 2 + sl] = p.w;
+            }
+            nbuf += nk;
         }
+    };
+    // A segment's end: its sum joins the group's, as the list kernel's
+    // tasks do (finish_task).
+    Kahan3 &fold = m.fold[lane];
+    fold = Kahan3();
+    int left = a.segment;          // entries the segment still takes
+    auto end_segment = [&]() {
         const int padded = pad_sources<kSplit>(Af, Bf, nbuf, lane);
         __syncwarp();
-        if (kLearned)
-            sum_buffer_learned<kSplit>(A, Bq, padded, hs, xi4, ti < ni, bx.eps2, bx.rcut2, bx.c_v, L, lq, k);
-        else if (kTable)
-            sum_buffer_table<kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, sTab, pk(a.tab_scale2, a.tab_scale2), k);
-        else
-            sum_buffer<NPOLY, kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, k);
-        inter += (unsigned long long)nbuf * ni;
+        sum_buffer<N, kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, k);
         staged += nbuf;
-        if (kLearned && lq.n > 0) {
-            // the queue's last, partial batch
-            float px = 0.f, py = 0.f, pz = 0.f;
-            learned_flush(lq, lq.n, lane, bx.eps2, bx.c_v, L, px, py, pz);
-            k.add(px, py, pz);
-        }
+        nbuf = 0;
         __syncwarp();
         // the kSplit source slots of a target add up their compensated totals
         float tx = k.sx - k.cx, ty = k.sy - k.cy, tz = k.sz - k.cz;
@@ -709,20 +921,127 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
             ty += __shfl_xor_sync(0xffffffffu, ty, o);
             tz += __shfl_xor_sync(0xffffffffu, tz, o);
         }
-        const float Gc = kLearned ? bx.G : NPOLY == kInvDeg ? bx.inv_g : bx.c_g;
-        if (task) {
-            finish_task<G>(a, t, ni, i0, Gc, tx, ty, tz);
-        } else if (hs == 0 && ti < ni) {
-            const int64_t o = a.perm[i0 + ti];
-            a.acc[3 * o + 0] = Gc * tx;
-            a.acc[3 * o + 1] = Gc * ty;
-            a.acc[3 * o + 2] = Gc * tz;
+        fold.add(tx, ty, tz);
+        k = Kahan3();
+    };
+    {
+        // Direct mode: the leaf pairs of the group are found here, as the
+        // pair builder finds them (same test, same order), and queued
+        // until 32 make a batch.  Lane t < 27 takes neighbour cell t.
+        const int ns = bx.nside;
+        const int ground = a.group_cell[g] - bx.cell_base;
+        const int gx = ground / (ns * ns), gy = (ground / ns) % ns, gz = ground % ns;
+        const float4 gc = a.group_c4[g];
+        const float hc = (float)bx.h;
+        const float rfb = bx.rfilt2;   // of the boxes (not scaled)
+        int l0 = 0, cnt = 0;
+        if (lane < 27) {
+            const int dx = lane / 9 - 1, dy = (lane / 3) % 3 - 1, dz = lane % 3 - 1;
+            const int ax = gx + dx, ay = gy + dy, az = gz + dz;
+            const int sx = ax < 0 ? -1 : (ax >= ns ? 1 : 0);
+            const int sy = ay < 0 ? -1 : (ay >= ns ? 1 : 0);
+            const int sz = az < 0 ? -1 : (az >= ns ? 1 : 0);
+            const int nc = bx.cell_base + ((ax - sx * ns) * ns + (ay - sy * ns)) * ns + (az - sz * ns);
+            const float qx = fmaxf(fmaxf(dx * hc - (gc.x + gh0.x), (gc.x - gh0.x) - (dx + 1) * hc), 0.f);
+            const float qy = fmaxf(fmaxf(dy * hc - (gc.y + gh0.y), (gc.y - gh0.y) - (dy + 1) * hc), 0.f);
+            const float qz = fmaxf(fmaxf(dz * hc - (gc.z + gh0.z), (gc.z - gh0.z) - (dz + 1) * hc), 0.f);
+            if (qx * qx + qy * qy + qz * qz < rfb * 1.0001f) {
+                l0 = a.cell_leaf_first[nc];
+                cnt = a.cell_leaf_first[nc + 1] - l0;
+            }
         }
+        const int cincl = warp_incl_scan_i(cnt, lane);
+        const int cexcl = cincl - cnt;
+        const int ctotal = __shfl_sync(0xffffffffu, cincl, 31);
+        const unsigned nonempty = __ballot_sync(0xffffffffu, cnt > 0);
+        if (cnt > 0) m.run[__popc(nonempty & lt)] = make_int2(lane, l0 - cexcl);
+        __syncwarp();
+        const float4 gr4 = a.group_r4[g];
+        int qn = 0;        // queued entries
+        int runs = 0;      // cell runs started before c0
+        for (int c0 = 0; c0 < ctotal; c0 += 32) {
+            const int q = c0 + lane;
+            const unsigned sq = (unsigned)(cexcl - c0);
+            const unsigned starts = __reduce_or_sync(0xffffffffu, (cnt > 0 && sq < 32u) ? 1u << sq : 0u);
+            const int r = runs + __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
+            runs += __popc(starts);
+            const int2 ru = m.run[r];
+            const int o = ru.x;
+            const int odx = o / 9 - 1, ody = (o / 3) % 3 - 1, odz = o % 3 - 1;
+            bool acc = false;
+            float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
+            int ec = 0;
+            if (q < ctotal) {
+                const int l = ru.y + q;
+                const float4 lc = a.leaf_c4[l], lh = a.leaf_h4[l];
+                const float px = fmaxf(fabsf((lc.x + odx * hc) - gc.x) - (gh0.x + lh.x), 0.f);
+                const float py = fmaxf(fabsf((lc.y + ody * hc) - gc.y) - (gh0.y + lh.y), 0.f);
+                const float pz = fmaxf(fabsf((lc.z + odz * hc) - gc.z) - (gh0.z + lh.z), 0.f);
+                acc = px * px + py * py + pz * pz < rfb;
+                if (acc) {
+                    const int ax = gx + odx, ay = gy + ody, az = gz + odz;
+                    const int sx = ax < 0 ? -1 : (ax >= ns ? 1 : 0);
+                    const int sy = ay < 0 ? -1 : (ay >= ns ? 1 : 0);
+                    const int sz = az < 0 ? -1 : (az >= ns ? 1 : 0);
+                    if ((sx | sy | sz) == 0) {
+                        const float4 lr4 = a.leaf_r4[l];
+                        ent.x = __fsub_rn(lr4.x, gr4.x);
+                        ent.y = __fsub_rn(lr4.y, gr4.y);
+                        ent.z = __fsub_rn(lr4.z, gr4.z);
+                    } else {
+                        const double *lr = a.leaf_ref + 3 * (int64_t)l;
+                        const double *gr = a.group_ref + 3 * (int64_t)g;
+                        const double L = bx.L;
+                        ent.x = __double2float_rn((lr[0] + sx * L) - gr[0]);
+                        ent.y = __double2float_rn((lr[1] + sy * L) - gr[1]);
+                        ent.z = __double2float_rn((lr[2] + sz * L) - gr[2]);
+                    }
+                    ent.w = lc.w;
+                    ec = __float_as_int(lh.w);
+                }
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, acc);
+            if (acc) {
+                const int slot = qn + __popc(bal & lt);
+                m.qent[slot] = ent;
+                m.qcnt[slot] = ec;
+            }
+            qn += __popc(bal);
+            __syncwarp();
+            for (int nb = left < 32 ? left : 32; qn >= nb; nb = left < 32 ? left : 32) {
+                EntryBatch bt;
+                const bool has = lane < nb;
+                bt.set(has ? m.qent[lane] : make_float4(0.f, 0.f, 0.f, 0.f), has ? m.qcnt[lane] : 0, lane);
+                // the rest moves up (qn - nb may exceed 32: two per lane)
+                const int s0 = nb + lane, s1 = nb + 32 + lane;
+                float4 m0, m1;
+                int c0m = 0, c1m = 0;
+                if (s0 < qn) { m0 = m.qent[s0]; c0m = m.qcnt[s0]; }
+                if (s1 < qn) { m1 = m.qent[s1]; c1m = m.qcnt[s1]; }
+                __syncwarp();
+                if (s0 < qn) { m.qent[lane] = m0; m.qcnt[lane] = c0m; }
+                if (s1 < qn) { m.qent[32 + lane] = m1; m.qcnt[32 + lane] = c1m; }
+                __syncwarp();
+                qn -= nb;
+                stage_batch(bt);
+                left -= nb;
+                if (left == 0) {
+                    end_segment();
+                    left = a.segment;
+                }
+            }
+        }
+        if (qn > 0) {
+            EntryBatch bt;
+            bt.set(lane < qn ? m.qent[lane] : make_float4(0.f, 0.f, 0.f, 0.f), lane < qn ? m.qcnt[lane] : 0,
+                   lane);
+            stage_batch(bt);
+            left -= qn;
+        }
+        __syncwarp();   // sRun and the queue are rewritten for the next group
     }
-    if (lane == 0 && inter) {
-        atomicAdd(a.n_inter, inter);
-        atomicAdd(a.n_staged, staged);
-    }
+    if (left < a.segment) end_segment();   // the last one, unless the entries just filled it
+    return ListSum{fold.sx - fold.cx, fold.sy - fold.cy, fold.sz - fold.cz, staged};
 }
 
 // Direct mode (exact factor): k_pp without a stored pair list.  Each group's
@@ -737,6 +1056,8 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
 template <int NPOLY, int kMinBlocks, int kSplit, bool kUniform>
 __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
 {
+    constexpr bool kBoth = NPOLY == kInvDeg;         // both forms, chosen per group
+    constexpr int kDeg = kBoth ? kInvGeneral : NPOLY;   // degree of the general form
     __shared__ float4 sA[kPPWarps][kJBuf / 2];
     __shared__ float4 sB[kPPWarps][kJBuf / 2];
     // direct mode: cell runs and the queue of found entries
@@ -745,9 +1066,6 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
     __shared__ int sQCnt[kPPWarps][64];
     __shared__ Kahan3 sFold[kPPWarps][32];   // the sum over the segments done
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const unsigned lt = (1u << lane) - 1u;
-    float4 *A = sA[w], *Bq = sB[w];
-    float *Af = reinterpret_cast<float *>(A), *Bf = reinterpret_cast<float *>(Bq);
     const int ng = *a.n_groups;
     unsigned long long inter = 0, staged = 0;
     for (;;) {
@@ -757,213 +1075,25 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
         if (g >= ng) break;
         const int i0 = a.group_first[g], ni = a.group_first[g + 1] - i0;
         const BoxDev &bx = a.boxes[a.group_box[g]];
-        PairConsts cl;
-        if (!kUniform) box_consts<NPOLY>(bx, cl);
-        const PairConsts &c = kUniform ? a.uc : cl;
-        const float rf2 = c.rfilt2;   // of the staged (scaled) sources
         const float4 gh0 = a.group_h4[g];
-        float4 gh = gh0;
+        const bool inv = kBoth && dense_group(gh0, ni, kUniform ? a.uc.rcut2 : bx.rcut2);
         constexpr int G = 32 / kSplit;
         const int ti = lane & (G - 1), hs = lane / G;   // target slot, source slot
-        float4 xi4 = ti < ni ? a.pos_group[i0 + ti] : make_float4(0.f, 0.f, 0.f, 0.f);
-        // the inverse-distance form works in lengths scaled by a power of two
-        const float sc = NPOLY == kInvDeg ? c.sc : 1.f;
-        if (NPOLY == kInvDeg) {
-            gh.x *= sc; gh.y *= sc; gh.z *= sc;
-            xi4.x *= sc; xi4.y *= sc; xi4.z *= sc;
-        }
-        const f2_t xi = pk(xi4.x, xi4.x), yi = pk(xi4.y, xi4.y), zi = pk(xi4.z, xi4.z);
-        Kahan3 k;
-        int nbuf = 0;
-        // The source particles of a batch of (up to) 32 entries, one per lane:
-        // each round loads 32 concatenated particles, one per lane.
-        auto stage_batch = [&](const EntryBatch &bt) {
-            int before = 0;
-            for (int q0 = 0; q0 < bt.total; q0 += 32) {
-                Round cur;
-                cur.issue(a, bt, q0, lane, before);
-                float4 p = cur.p;
-                bool keep = false;
-                if (cur.valid) {
-                    // sc (p + o), rounded once: sc is a power of two
-                    p.x = __fmaf_rn(p.x, sc, cur.ox * sc);
-                    p.y = __fmaf_rn(p.y, sc, cur.oy * sc);
-                    p.z = __fmaf_rn(p.z, sc, cur.oz * sc);
-                    const float qx = fmaxf(fabsf(p.x) - gh.x, 0.f);
-                    const float qy = fmaxf(fabsf(p.y) - gh.y, 0.f);
-                    const float qz = fmaxf(fabsf(p.z) - gh.z, 0.f);
-                    keep = qx * qx + qy * qy + qz * qz < rf2;
-                }
-                const unsigned bal = __ballot_sync(0xffffffffu, keep);
-                const int nk = __popc(bal);
-                if (nbuf + nk > kJBuf) {
-                    const int padded = pad_sources<kSplit>(Af, Bf, nbuf, lane);
-                    __syncwarp();
-                    sum_buffer<NPOLY, kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, k);
-                    inter += (unsigned long long)nbuf * ni;
-                    staged += nbuf;
-                    nbuf = 0;
-                    __syncwarp();
-                }
-                const int idx = nbuf + __popc(bal & lt);
-                if (keep && in_bounds(idx, kJBuf, BS_PP_STAGE)) {
-                    const int m = idx >> 1, sl = idx & 1;
-                    Af[m * 4 + sl] = p.x;
-                    Af[m * 4 + 2 + sl] = p.y;
-                    Bf[m * 4 + sl] = p.z;
-                    Bf[m * 4 + 2 + sl] = p.w;
-                }
-                nbuf += nk;
-            }
-        };
-        // A segment's end: its sum joins the group's, as the list kernel's
-        // tasks do (finish_task).
-        Kahan3 &fold = sFold[w][lane];
-        fold = Kahan3();
-        int left = a.segment;          // entries the segment still takes
-        auto end_segment = [&]() {
-            const int padded = pad_sources<kSplit>(Af, Bf, nbuf, lane);
-            __syncwarp();
-            sum_buffer<NPOLY, kSplit>(A, Bq, padded >> 1, hs, xi, yi, zi, c, k);
-            inter += (unsigned long long)nbuf * ni;
-            staged += nbuf;
-            nbuf = 0;
-            __syncwarp();
-            // the kSplit source slots of a target add up their compensated totals
-            float tx = k.sx - k.cx, ty = k.sy - k.cy, tz = k.sz - k.cz;
-#pragma unroll
-            for (int o = G; o < 32; o <<= 1) {
-                tx += __shfl_xor_sync(0xffffffffu, tx, o);
-                ty += __shfl_xor_sync(0xffffffffu, ty, o);
-                tz += __shfl_xor_sync(0xffffffffu, tz, o);
-            }
-            fold.add(tx, ty, tz);
-            k = Kahan3();
-        };
-        {
-            // Direct mode: the leaf pairs of the group are found here, as the
-            // pair builder finds them (same test, same order), and queued
-            // until 32 make a batch.  Lane t < 27 takes neighbour cell t.
-            const int ns = bx.nside;
-            const int ground = a.group_cell[g] - bx.cell_base;
-            const int gx = ground / (ns * ns), gy = (ground / ns) % ns, gz = ground % ns;
-            const float4 gc = a.group_c4[g];
-            const float hc = (float)bx.h;
-            const float rfb = bx.rfilt2;   // of the boxes (not scaled)
-            int l0 = 0, cnt = 0;
-            if (lane < 27) {
-                const int dx = lane / 9 - 1, dy = (lane / 3) % 3 - 1, dz = lane % 3 - 1;
-                const int ax = gx + dx, ay = gy + dy, az = gz + dz;
-                const int sx = ax < 0 ? -1 : (ax >= ns ? 1 : 0);
-                const int sy = ay < 0 ? -1 : (ay >= ns ? 1 : 0);
-                const int sz = az < 0 ? -1 : (az >= ns ? 1 : 0);
-                const int nc = bx.cell_base + ((ax - sx * ns) * ns + (ay - sy * ns)) * ns + (az - sz * ns);
-                const float qx = fmaxf(fmaxf(dx * hc - (gc.x + gh0.x), (gc.x - gh0.x) - (dx + 1) * hc), 0.f);
-                const float qy = fmaxf(fmaxf(dy * hc - (gc.y + gh0.y), (gc.y - gh0.y) - (dy + 1) * hc), 0.f);
-                const float qz = fmaxf(fmaxf(dz * hc - (gc.z + gh0.z), (gc.z - gh0.z) - (dz + 1) * hc), 0.f);
-                if (qx * qx + qy * qy + qz * qz < rfb * 1.0001f) {
-                    l0 = a.cell_leaf_first[nc];
-                    cnt = a.cell_leaf_first[nc + 1] - l0;
-                }
-            }
-            const int cincl = warp_incl_scan_i(cnt, lane);
-            const int cexcl = cincl - cnt;
-            const int ctotal = __shfl_sync(0xffffffffu, cincl, 31);
-            const unsigned nonempty = __ballot_sync(0xffffffffu, cnt > 0);
-            if (cnt > 0) sRun[w][__popc(nonempty & lt)] = make_int2(lane, l0 - cexcl);
-            __syncwarp();
-            const float4 gr4 = a.group_r4[g];
-            int qn = 0;        // queued entries
-            int runs = 0;      // cell runs started before c0
-            for (int c0 = 0; c0 < ctotal; c0 += 32) {
-                const int q = c0 + lane;
-                const unsigned sq = (unsigned)(cexcl - c0);
-                const unsigned starts = __reduce_or_sync(0xffffffffu, (cnt > 0 && sq < 32u) ? 1u << sq : 0u);
-                const int r = runs + __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
-                runs += __popc(starts);
-                const int2 ru = sRun[w][r];
-                const int o = ru.x;
-                const int odx = o / 9 - 1, ody = (o / 3) % 3 - 1, odz = o % 3 - 1;
-                bool acc = false;
-                float4 ent = make_float4(0.f, 0.f, 0.f, 0.f);
-                int ec = 0;
-                if (q < ctotal) {
-                    const int l = ru.y + q;
-                    const float4 lc = a.leaf_c4[l], lh = a.leaf_h4[l];
-                    const float px = fmaxf(fabsf((lc.x + odx * hc) - gc.x) - (gh0.x + lh.x), 0.f);
-                    const float py = fmaxf(fabsf((lc.y + ody * hc) - gc.y) - (gh0.y + lh.y), 0.f);
-                    const float pz = fmaxf(fabsf((lc.z + odz * hc) - gc.z) - (gh0.z + lh.z), 0.f);
-                    acc = px * px + py * py + pz * pz < rfb;
-                    if (acc) {
-                        const int ax = gx + odx, ay = gy + ody, az = gz + odz;
-                        const int sx = ax < 0 ? -1 : (ax >= ns ? 1 : 0);
-                        const int sy = ay < 0 ? -1 : (ay >= ns ? 1 : 0);
-                        const int sz = az < 0 ? -1 : (az >= ns ? 1 : 0);
-                        if ((sx | sy | sz) == 0) {
-                            const float4 lr4 = a.leaf_r4[l];
-                            ent.x = __fsub_rn(lr4.x, gr4.x);
-                            ent.y = __fsub_rn(lr4.y, gr4.y);
-                            ent.z = __fsub_rn(lr4.z, gr4.z);
-                        } else {
-                            const double *lr = a.leaf_ref + 3 * (int64_t)l;
-                            const double *gr = a.group_ref + 3 * (int64_t)g;
-                            const double L = bx.L;
-                            ent.x = __double2float_rn((lr[0] + sx * L) - gr[0]);
-                            ent.y = __double2float_rn((lr[1] + sy * L) - gr[1]);
-                            ent.z = __double2float_rn((lr[2] + sz * L) - gr[2]);
-                        }
-                        ent.w = lc.w;
-                        ec = __float_as_int(lh.w);
-                    }
-                }
-                const unsigned bal = __ballot_sync(0xffffffffu, acc);
-                if (acc) {
-                    const int slot = qn + __popc(bal & lt);
-                    sQEnt[w][slot] = ent;
-                    sQCnt[w][slot] = ec;
-                }
-                qn += __popc(bal);
-                __syncwarp();
-                for (int nb = left < 32 ? left : 32; qn >= nb; nb = left < 32 ? left : 32) {
-                    EntryBatch bt;
-                    const bool has = lane < nb;
-                    bt.set(has ? sQEnt[w][lane] : make_float4(0.f, 0.f, 0.f, 0.f), has ? sQCnt[w][lane] : 0, lane);
-                    // the rest moves up (qn - nb may exceed 32: two per lane)
-                    const int s0 = nb + lane, s1 = nb + 32 + lane;
-                    float4 m0, m1;
-                    int c0m = 0, c1m = 0;
-                    if (s0 < qn) { m0 = sQEnt[w][s0]; c0m = sQCnt[w][s0]; }
-                    if (s1 < qn) { m1 = sQEnt[w][s1]; c1m = sQCnt[w][s1]; }
-                    __syncwarp();
-                    if (s0 < qn) { sQEnt[w][lane] = m0; sQCnt[w][lane] = c0m; }
-                    if (s1 < qn) { sQEnt[w][32 + lane] = m1; sQCnt[w][32 + lane] = c1m; }
-                    __syncwarp();
-                    qn -= nb;
-                    stage_batch(bt);
-                    left -= nb;
-                    if (left == 0) {
-                        end_segment();
-                        left = a.segment;
-                    }
-                }
-            }
-            if (qn > 0) {
-                EntryBatch bt;
-                bt.set(lane < qn ? sQEnt[w][lane] : make_float4(0.f, 0.f, 0.f, 0.f), lane < qn ? sQCnt[w][lane] : 0,
-                       lane);
-                stage_batch(bt);
-                left -= qn;
-            }
-            __syncwarp();   // sRun and the queue are rewritten for the next group
-        }
-        if (left < a.segment) end_segment();   // the last one, unless the entries just filled it
-        const float tx = fold.sx - fold.cx, ty = fold.sy - fold.cy, tz = fold.sz - fold.cz;
+        const WalkMem mem{sA[w], sB[w], sRun[w], sQEnt[w], sQCnt[w], sFold[w]};
+        ListSum s;
+        if constexpr (kBoth)
+            s = inv ? walk_group<kInvDeg, kSplit, kUniform>(a, bx, mem, g, i0, ni, gh0)
+                    : walk_group<kDeg, kSplit, kUniform>(a, bx, mem, g, i0, ni, gh0);
+        else
+            s = walk_group<kDeg, kSplit, kUniform>(a, bx, mem, g, i0, ni, gh0);
+        inter += (unsigned long long)s.staged * ni;
+        staged += s.staged;
         if (hs == 0 && ti < ni) {
             const int64_t o = a.perm[i0 + ti];
-            const float Gc = NPOLY == kInvDeg ? bx.inv_g : bx.c_g;
-            a.acc[3 * o + 0] = Gc * tx;
-            a.acc[3 * o + 1] = Gc * ty;
-            a.acc[3 * o + 2] = Gc * tz;
+            const float Gc = inv ? bx.inv_g : bx.c_g;
+            a.acc[3 * o + 0] = Gc * s.x;
+            a.acc[3 * o + 1] = Gc * s.y;
+            a.acc[3 * o + 2] = Gc * s.z;
         }
     }
     if (lane == 0 && inter) {
@@ -974,7 +1104,7 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp_walk(PPArgs a)
 
 // Number of (i, j) pairs, j != i, with r^2 < rcut^2 in the lists (the self
 // pair is recognised by its index: sources and targets share the sorted
-// order): the work the cutoff keeps, counted with the PP kernel's own FP32
+// order): the work the cutoff keeps, counted with the exact kernel's own FP32
 // decision.  Groups without a list (active-particle mode) count nothing.
 __global__ void __launch_bounds__(kPPThreads) k_count_within(PPArgs a)
 {
@@ -991,8 +1121,9 @@ __global__ void __launch_bounds__(kPPThreads) k_count_within(PPArgs a)
         if (g >= ng) break;
         const int i0 = a.group_first[g], ni = a.group_first[g + 1] - i0;
         const BoxDev &bx = a.boxes[a.group_box[g]];
-        const float sc = a.inverse ? bx.sc : 1.f, eps2 = a.inverse ? bx.eps2s : 0.f;
-        const float cut = a.inverse ? bx.inv_cut : bx.rcut2;
+        const bool inv = a.inverse && dense_group(a.group_h4[g], ni, bx.rcut2);
+        const float sc = inv ? bx.sc : 1.f, eps2 = inv ? bx.eps2s : 0.f;
+        const float cut = inv ? bx.inv_cut : bx.rcut2;
         float4 xi = lane < ni ? a.pos_group[i0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
         xi.x *= sc; xi.y *= sc; xi.z *= sc;
         const int64_t e1 = a.group_off[g + 1] < a.cap ? a.group_off[g + 1] : a.cap;
@@ -1088,7 +1219,9 @@ static void launch_pp(bool chained, int npoly, int grid, cudaStream_t s, const P
 {
     auto launch = [&](auto kernel) { launch_chained(chained, kernel, grid, kPPThreads, 0, s, a); };
     switch (npoly) {
-    case kInvDeg: launch(k_pp<kInvDeg, kLearned, kMinBlocks, kSplit, kUniform>); break;
+    case kInvDeg:
+        if constexpr (32 / kSplit >= kDenseMin) launch(k_pp<kInvDeg, kLearned, kMinBlocks, kSplit, kUniform>);
+        break;
     case 10: launch(k_pp<10, kLearned, kMinBlocks, kSplit, kUniform>); break;
     case 12: launch(k_pp<12, kLearned, kMinBlocks, kSplit, kUniform>); break;
     case 14: launch(k_pp<14, kLearned, kMinBlocks, kSplit, kUniform>); break;
@@ -1100,7 +1233,9 @@ template <int kMinBlocks, int kSplit, bool kUniform>
 static void launch_walk_one(int npoly, int grid, cudaStream_t s, const PPArgs &a)
 {
     switch (npoly) {
-    case kInvDeg: k_pp_walk<kInvDeg, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
+    case kInvDeg:
+        if constexpr (32 / kSplit >= kDenseMin) k_pp_walk<kInvDeg, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a);
+        break;
     case 10: k_pp_walk<10, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
     case 12: k_pp_walk<12, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
     case 14: k_pp_walk<14, kMinBlocks, kSplit, kUniform><<<grid, kPPThreads, 0, s>>>(a); break;
@@ -1181,9 +1316,8 @@ int pp_learned_device(const ph_leaves *lv, const ph_pairs *pr, const float *mlp_
 }
 
 // true if every box has the same factor constants (then the kernel reads
-// them from its parameter bank); general: those of the general form, which
-// the tabulated factor's kernel uses whatever the exact kernel does
-static bool uniform_consts(const ph_leaves *lv, PairConsts &uc, bool general)
+// them from its parameter bank)
+static bool uniform_consts(const ph_leaves *lv, PairConsts &uc, InvConsts &ui)
 {
     if ((int)lv->boxes_host.size() < lv->n_boxes || lv->n_boxes < 1) return false;   // no host copy of the boxes
     const BoxDev &b0 = lv->boxes_host[0];
@@ -1202,20 +1336,23 @@ static bool uniform_consts(const ph_leaves *lv, PairConsts &uc, bool general)
         u = ((uint64_t)bits << 32) | bits;
         return (f2_t)u;
     };
-    const bool inv = lv->poly_degree == kInvDeg && !general;
-    for (int q = 0; q <= kMaxPoly; q++) uc.poly[q] = dup(!inv ? b0.poly[q] : q <= kInvDeg ? b0.inv_poly[q] : 0.f);
+    for (int q = 0; q <= kMaxPoly; q++) uc.poly[q] = dup(b0.poly[q]);
     uc.s2 = dup(b0.s2);
     uc.eps2s = dup(b0.eps2s);
     uc.c_t = dup(b0.c_t);
     uc.c_e = dup(b0.c_e);
     uc.m1 = dup(-1.f);
-    uc.rcut2 = inv ? b0.inv_cut : b0.rcut2;
-    uc.rfilt2 = inv ? b0.rfilt2 * b0.s2 : b0.rfilt2;
-    uc.zc = dup(b0.inv_zc);
-    uc.b1 = dup(b0.inv_b1);
-    uc.b2 = dup(b0.inv_b2);
-    uc.m53 = dup(-kInvK);
-    uc.sc = inv ? b0.sc : 1.f;
+    uc.rcut2 = b0.rcut2;
+    uc.rfilt2 = b0.rfilt2;
+    for (int q = 0; q <= kInvDeg; q++) ui.poly[q] = dup(b0.inv_poly[q]);
+    ui.eps2s = dup(b0.eps2s);
+    ui.zc = dup(b0.inv_zc);
+    ui.b1 = dup(b0.inv_b1);
+    ui.b2 = dup(b0.inv_b2);
+    ui.m53 = dup(-kInvK);
+    ui.cut = b0.inv_cut;
+    ui.rfilt2 = b0.rfilt2 * b0.s2;
+    ui.sc = b0.sc;
     return true;
 }
 
@@ -1226,7 +1363,7 @@ int pp_table_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaS
     PPArgs a;
     pp_args(lv, pr, d_acc, a);
     a.mlp_w = nullptr;
-    if (!uniform_consts(lv, a.uc, true)) return fail(PH_ERR_ARG, "the tabulated factor needs one rcut and rs for all boxes");
+    if (!uniform_consts(lv, a.uc, a.ui)) return fail(PH_ERR_ARG, "the tabulated factor needs one rcut and rs for all boxes");
     a.table = static_cast<const float2 *>(lv->table.p);
     a.tab_scale2 = (float)((kTabN / lv->table_rcut) * (kTabN / lv->table_rcut));
     int rc2 = chained ? PH_OK : cuda_check(cudaMemsetAsync(pr->work.p, 0, 24, s), "reset work queue");
@@ -1247,10 +1384,11 @@ int pp_exact_device(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, cudaS
     a.mlp_w = nullptr;
     int rc = chained ? PH_OK : cuda_check(cudaMemsetAsync(pr ? pr->work.p : lv->work.p, 0, 24, s), "reset work queue");
     if (rc) return rc;
-    const int npoly = lv->poly_degree;
+    // (groups of 8 are never dense)
+    const int npoly = lv->poly_degree == kInvDeg && lv->group_size < kDenseMin ? kInvGeneral : lv->poly_degree;
     if (npoly != kInvDeg && npoly != 10 && npoly != 12 && npoly != 14 && npoly != 16)
         return fail(PH_ERR_STATE, "unsupported polynomial degree %d", npoly);
-    const bool uni = uniform_consts(lv, a.uc, false);
+    const bool uni = uniform_consts(lv, a.uc, a.ui);
     if (!pr) {
         launch_walk(lv, npoly, uni, s, a);
         count_launch();

@@ -1,6 +1,7 @@
 """The exact PP kernel's two forms of the softened short-range weight: the
-inverse-distance form (rcut / 2R_s <= 2.3 and eps <= 2R_s / 64) and the
-general form, at both sides of the line between them, against the oracle."""
+inverse-distance form (rcut / 2R_s <= 2.3 and eps <= 2R_s / 64, dense groups)
+and the general form, at both sides of the line between them, against the
+oracle.  The boxes are dense: 450 sources a target."""
 import dataclasses
 
 import numpy as np
@@ -12,7 +13,7 @@ from paper_1802_09824_gb300 import synth
 pytestmark = pytest.mark.gpu
 
 
-def _box(U, eps_div, scale=3000, L=1.0):
+def _box(U, eps_div, scale=20_000, L=1.0):
     """A uniform box with rcut / 2R_s = U and eps = 2R_s / eps_div (0: none)."""
     ps = synth.workload("uniform_small", scale=scale)
     bp = ps.boxes[0]
@@ -53,13 +54,14 @@ def test_forms_agree_across_the_line(gpu_lib):
         out.append(got.astype(np.float64))
         for h in (pr, lv):
             gpu_lib.ph_free(h)
+    assert np.mean(out[0] != out[1]) > 0.5          # two forms indeed
     diff = np.linalg.norm(out[0] - out[1], axis=1) / np.linalg.norm(out[0], axis=1)
     assert np.percentile(diff, 90) <= 2e-6
 
 
 def test_one_box_outside_the_range_takes_all_to_the_general_form(gpu_lib):
     # boxes summed in one launch share a form
-    a, b = _box(2.25, 75.0, scale=700), _box(2.25, 8.0, scale=1100)
+    a, b = _box(2.25, 75.0, scale=12_000), _box(2.25, 8.0, scale=15_000)
     ps = synth.ParticleSet(np.concatenate([a.pos, b.pos]), np.concatenate([a.mass, b.mass]), a.boxes + b.boxes,
                            np.array([0, a.n, a.n + b.n]), "two")
     got, lv, pr = gpu_accel(gpu_lib, ps)
