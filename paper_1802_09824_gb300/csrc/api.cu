@@ -599,9 +599,7 @@ int ph_leaf_pairs(ph_leaves *leaves, void *stream, ph_pairs **pairs)
     }
     // (a reserved list is not sized: as many slots as it can need)
     if (!rc && p->fixed_capacity && !p->task_cap)
-        rc = ensure_tasks(p, task_bound(p->capacity, leaves->segment), (int64_t)N);
-    else if (!rc)
-        rc = ensure_tasks(p, p->task_cap, (int64_t)N);
+        rc = ensure_tasks(p, task_bound(p->capacity, leaves->segment, leaves->n));
     if (!rc) rc = build_pairs_device(leaves, p, s, !p->fixed_capacity);
     if (rc) {
         if (fresh) {

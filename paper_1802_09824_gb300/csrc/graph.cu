@@ -9,6 +9,7 @@
 // whose pair list would outgrow the capacity writes no entry beyond it and
 // latches PH_ERR_CAPACITY in the pairs handle's status (ph_status); rebuild
 // with ph_leaf_pairs and create a new graph then.
+#include <algorithm>
 #include <new>
 
 #include "handles.cuh"
@@ -81,13 +82,14 @@ int ph_graph_create(ph_leaves *leaves, ph_pairs *pairs, const void *d_pos, int p
     if (pairs) {
         // fixed pair capacity with headroom over the current list
         const int64_t want = (int64_t)((double)pairs->n_pairs * (1.0 + headroom)) + 1024;
-        const int64_t slots = (int64_t)((double)pairs->n_tasks * (1.0 + headroom)) + 64;
+        const int64_t slots = std::max<int64_t>((int64_t)((double)pairs->n_tasks * (1.0 + headroom)) + 64,
+                                                task_bound(std::max(want, pairs->capacity), leaves->segment, leaves->n));
         if (want > pairs->capacity || slots > pairs->task_cap) {
             // the list stays what it was (ph_pp_accel may sum it before the
             // first replay): its buffers move with their contents
             int rc = cuda_check(cudaStreamSynchronize(caller), "sync before growing");
             if (!rc) rc = cuda_check(cudaStreamSynchronize(pairs->last_stream), "sync before growing");
-            if (!rc) rc = grow_pairs(pairs, want, slots, leaves->n, caller);
+            if (!rc) rc = grow_pairs(pairs, want, slots, caller);
             if (rc) return rc;
         }
         pairs->fixed_capacity = true;
@@ -99,7 +101,7 @@ int ph_graph_create(ph_leaves *leaves, ph_pairs *pairs, const void *d_pos, int p
     ph_graph *g = new (std::nothrow) ph_graph();
     if (!g) return fail(PH_ERR_OOM, "host allocation failed");
     // (the capture makes no list: the one on the device stays current)
-    const int64_t list_cap = pairs ? pairs->list_cap : 0, list_task_cap = pairs ? pairs->list_task_cap : 0;
+    const int64_t list_cap = pairs ? pairs->list_cap : 0;
     cudaStream_t s = nullptr;
     int rc = cuda_check(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking), "create capture stream");
     if (!rc) rc = cuda_check(cudaStreamSynchronize(caller), "sync before capture");
@@ -122,10 +124,7 @@ int ph_graph_create(ph_leaves *leaves, ph_pairs *pairs, const void *d_pos, int p
     g->kernels = ph_launch_counter() - k0;
     if (!rc) rc = cuda_check(cudaGraphInstantiate(&g->exec, g->graph, 0), "instantiate");
     if (s) cudaStreamDestroy(s);
-    if (pairs) {
-        pairs->list_cap = list_cap;
-        pairs->list_task_cap = list_task_cap;
-    }
+    if (pairs) pairs->list_cap = list_cap;
     if (rc) {
         graph_free(g);
         return rc;
@@ -160,10 +159,7 @@ int ph_graph_launch(ph_graph *g, void *stream)
         return fail(PH_ERR_STATE, "the handles' buffers changed since the capture: create a new graph");
     int rc = cuda_check(cudaGraphLaunch(g->exec, static_cast<cudaStream_t>(stream)), "graph launch");
     if (!rc) count_launch((int)g->kernels);
-    if (!rc && g->pairs) {
-        g->pairs->list_cap = g->pairs->capacity;
-        g->pairs->list_task_cap = g->pairs->task_cap;
-    }
+    if (!rc && g->pairs) g->pairs->list_cap = g->pairs->capacity;
     return rc;
 }
 

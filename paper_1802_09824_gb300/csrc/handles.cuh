@@ -94,18 +94,17 @@ struct ph_pairs {
     // pass when these buffers exist; `ordered` says the last list has it
     phpp::DevBuf group_key;      // uint8[n]: 255 - cost bucket
     phpp::DevBuf group_order;    // int32[n]: groups in queue order
-    phpp::DevBuf order_temp;     // groups per key, cursors, the number of tasks written and needed, entries per run of groups
+    phpp::DevBuf order_temp;     // groups per key, cursors, the tasks' record (TaskCtl), entries per run of groups
     // groups with more than one segment are queued as one task per segment
-    phpp::DevBuf task_mem;       // the four arrays below
-    int2 *tasks = nullptr;       // [task_cap] (group, segment), a group's in a row; group -1: none
+    phpp::DevBuf task_mem;       // the three arrays below
+    int2 *tasks = nullptr;       // [task_cap] (group, segment), a group's in a row
     int32_t *task_done = nullptr;// [task_cap] segments summed, at the group's first task
     float *task_part = nullptr;  // [task_cap][3][32] the segments' sums
-    uint8_t *split_of = nullptr; // [n] of a group with several segments: whether it has tasks
     int64_t task_cap = 0;
     int64_t n_tasks = 0;         // host copy (valid after sizing sync)
-    // capacity and task slots the list on the device was made with (a graph's
-    // capture makes room for the lists of its replays)
-    int64_t list_cap = 0, list_task_cap = 0;
+    // capacity the list on the device was made with (a graph's capture makes
+    // room for the lists of its replays)
+    int64_t list_cap = 0;
     bool ordered = false;
 };
 
@@ -115,12 +114,13 @@ namespace phpp {
 // reads buffers that a failed or newer build left behind.
 int check_built(const ph_leaves *lv, const ph_pairs *pr);
 
-// Room for `slots` tasks of a list over n particles (pairs.cu).
-int ensure_tasks(ph_pairs *pr, int64_t slots, int64_t n);
+// The tasks' record of a list (device memory), and room for `slots` tasks (pairs.cu).
+TaskCtl *task_ctl(const ph_pairs *pr);
+int ensure_tasks(ph_pairs *pr, int64_t slots);
 
-// Room for `capacity` entries and `slots` tasks, the list over n particles and
-// its tasks kept (on stream s, which it synchronises); unchanged on failure.
-int grow_pairs(ph_pairs *pr, int64_t capacity, int64_t slots, int64_t n, cudaStream_t s);
+// Room for `capacity` entries and `slots` tasks, the list and its tasks kept
+// (on stream s, which it synchronises); unchanged on failure.
+int grow_pairs(ph_pairs *pr, int64_t capacity, int64_t slots, cudaStream_t s);
 
 // A fingerprint of the device buffers of a leaves (and pairs) handle: their
 // addresses and sizes.  A captured graph holds these addresses; it may only

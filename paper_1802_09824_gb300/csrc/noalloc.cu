@@ -131,12 +131,10 @@ void carve(Carver &c, ph_leaves &lv, ph_pairs &pr, int64_t n, int cells)
     pr.tasks = static_cast<int2 *>(lv.keys.p);
     pr.task_done = static_cast<int32_t *>(lv.keys_alt.p);
     pr.task_part = static_cast<float *>(lv.leaf_ref.p);
-    pr.split_of = static_cast<uint8_t *>(lv.starts.p);
 }
 
-// Segment length of the step: twice segment_entries' (there are fewer task
-// slots than a list at its capacity could ask for: N / 2, with a group whose
-// tasks find no room summed by one warp).
+// Segment length of the step: segment_entries' of twice as many particles
+// (there are fewer task slots than a list at its capacity could ask for: N / 2).
 int noalloc_segment(int64_t n, int leaf_max)
 {
     return segment_entries(2 * n, leaf_max, kDefaultGroup);

@@ -25,8 +25,8 @@
 // pass counts the groups of each key, and the fill pass, which has the
 // counts, places each group after the keys below its own with an atomic
 // cursor per key.  Groups of one key land in the order the fill pass meets
-// them; the forces do not depend on the order (each group is summed by one
-// warp on its own).
+// them; the forces do not depend on the order (a group's list is summed in
+// segments that are added in order, whichever warps sum them).
 #include <algorithm>
 
 #include "checks.cuh"
@@ -58,13 +58,12 @@ struct PairArgs {
     int64_t n_particles;     // mass-centre particle of leaf l: pos_leaf[n_particles + l]
     int64_t cap;
     uint32_t *status;
-    int32_t *n_tasks;        // tasks of split groups: [0] written by the fill pass, [1] needed (count pass)
+    TaskCtl *ctl;
     unsigned long long *chunk_sum;   // entries of every kOffChunk groups (count pass)
     int2 *tasks;
-    uint8_t *split_of;       // [n_groups]: whether a group of several segments has tasks
     int32_t *task_done;
     int64_t task_cap;
-    int segment;             // entries per segment
+    int segment;             // entries per segment where the tasks fit
     int64_t n_leaf_rows;     // rows of the leaf arrays (bounds checks)
 };
 
@@ -123,6 +122,17 @@ __global__ void __launch_bounds__(kThreads) k_pairs(PairArgs a)
         s_start[threadIdx.x] = incl - c;
         __syncthreads();
     }
+    int segment = 0;   // entries per segment of this list
+    if (kFill) {
+        segment = a.segment;
+        if (a.ctl->needed > a.task_cap) {
+            // longer, so that the tasks fit: a list of v > S entries is cut into
+            // fewer than 2 v / S (2^30: none is cut)
+            const int64_t longer = a.task_cap > 0 ? 2 * a.ctl->total / a.task_cap + 1 : 1 << 30;
+            segment = (int)(longer < 1 << 30 ? (longer > segment ? longer : segment) : 1 << 30);
+        }
+        if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->segment = segment;
+    }
     for (int gi = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; gi < ng; gi += warps) {
         const int g = a.group_list ? a.group_list[gi] : gi;
         if (kFill && a.order && lane == 0) {
@@ -134,19 +144,16 @@ __global__ void __launch_bounds__(kThreads) k_pairs(PairArgs a)
         if (kFill) {
             // a group of more than one segment: one task per segment
             const int64_t e0 = a.off[g] < a.cap ? a.off[g] : a.cap, e1 = a.off[g + 1] < a.cap ? a.off[g + 1] : a.cap;
-            if (e1 - e0 > a.segment) {
-                const int nseg = (int)((e1 - e0 + a.segment - 1) / a.segment);
+            if (e1 - e0 > segment) {
+                const int nseg = (int)((e1 - e0 + segment - 1) / segment);
                 int first = 0;
-                if (lane == 0) first = atomicAdd(a.n_tasks, nseg);
+                if (lane == 0) first = atomicAdd(&a.ctl->written, nseg);
                 first = __shfl_sync(0xffffffffu, first, 0);
-                // (a list that outgrew its task slots: the group is summed by
-                // one warp, and the slots left over are empty)
-                const bool fits = first + nseg <= a.task_cap;
-                for (int k = lane; k < nseg && first + k < a.task_cap; k += 32) {
-                    a.tasks[first + k] = make_int2(fits ? g : -1, k);
+                for (int k = lane; k < nseg; k += 32) {
+                    if (!in_bounds(first + k, a.task_cap, BS_PP_TASK)) continue;
+                    a.tasks[first + k] = make_int2(g, k);
                     a.task_done[first + k] = 0;
                 }
-                if (lane == 0) a.split_of[g] = fits ? 1 : 0;
             }
         }
         const BoxDev &bx = a.boxes[a.group_box[g]];
@@ -277,7 +284,7 @@ __global__ void __launch_bounds__(kThreads) k_pairs(PairArgs a)
             if (lane == 0) {
                 a.cnt[g] = count;
                 atomicAdd(a.chunk_sum + g / kOffChunk, (unsigned long long)count);
-                if (count > a.segment) atomicAdd(a.n_tasks + 1, (int)((count + a.segment - 1) / a.segment));
+                if (count > a.segment) atomicAdd(&a.ctl->needed, (int)((count + a.segment - 1) / a.segment));
                 if (a.gkey) {
                     const int k = 255 - cost_bucket(cost);
                     a.gkey[g] = (uint8_t)k;
@@ -300,7 +307,7 @@ __global__ void __launch_bounds__(kThreads) k_clear_counts(uint32_t *p, int64_t 
 // adds up from the count pass's sums.
 __global__ void __launch_bounds__(kThreads) k_offsets(const int64_t *cnt, const int32_t *n_groups,
                                                       const unsigned long long *chunk_sum, int64_t *off,
-                                                      unsigned long long *work, int64_t *total)
+                                                      unsigned long long *work, TaskCtl *ctl)
 {
     chain_begin();
     // the PP kernel's queue and counters (a captured step has no other reset)
@@ -344,16 +351,17 @@ __global__ void __launch_bounds__(kThreads) k_offsets(const int64_t *cnt, const 
 #pragma unroll
     for (int k = 0; k < 4; k++) {
         if (g + k <= ng) off[g + k] = e;
-        if (g + k == ng) *total = e;
+        if (g + k == ng) ctl->total = e;
         e += v[k];
     }
 }
 
 }  // namespace
 
-// Scratch of the queue: the per-key counts and cursors, the number of tasks
-// written and needed, all entries (int64); then the chunk sums of k_offsets.
-constexpr int kOrdInts = 2 * kOrdKeys + 4;
+// Scratch of the queue: the per-key counts and cursors, the tasks' record; then
+// the chunk sums of k_offsets.
+constexpr int kOrdInts = 2 * kOrdKeys + (int)(sizeof(TaskCtl) / sizeof(int32_t));
+static_assert(kOrdInts % 2 == 0 && sizeof(TaskCtl) % sizeof(int64_t) == 0, "the chunk sums are 8-byte aligned");
 size_t order_temp_bytes(int64_t n) { return kOrdInts * sizeof(int32_t) + (n / kOffChunk + 2) * sizeof(int64_t); }
 
 // A warp sums a group's list segment by segment, and a group of several
@@ -381,23 +389,25 @@ int segment_entries(int64_t n, int leaf_max, int group_size)
     return (int)std::max<int64_t>(sources / leaf_max, 8);
 }
 
-int ensure_tasks(ph_pairs *pr, int64_t slots, int64_t n)
+// The tasks' record of a list's scratch.
+TaskCtl *task_ctl(const ph_pairs *pr) { return reinterpret_cast<TaskCtl *>(static_cast<int32_t *>(pr->order_temp.p) + 2 * kOrdKeys); }
+
+int ensure_tasks(ph_pairs *pr, int64_t slots)
 {
     const size_t c = ((size_t)slots + 31) & ~(size_t)31;
-    if (pr->task_cap >= (int64_t)c && pr->task_mem.bytes >= (size_t)pr->task_cap * 396 + (size_t)n) return PH_OK;
+    if (pr->task_cap >= (int64_t)c) return PH_OK;
     pr->task_cap = 0;
-    const int rc = ensure(pr->task_mem, c * 396 + (size_t)n);
+    const int rc = ensure(pr->task_mem, c * 396);
     if (rc) return rc;
     char *p = static_cast<char *>(pr->task_mem.p);
     pr->task_cap = (int64_t)c;
     pr->task_part = reinterpret_cast<float *>(p);
     pr->tasks = reinterpret_cast<int2 *>(p + c * 384);
     pr->task_done = reinterpret_cast<int32_t *>(p + c * 392);
-    pr->split_of = reinterpret_cast<uint8_t *>(p + c * 396);
     return PH_OK;
 }
 
-int grow_pairs(ph_pairs *pr, int64_t capacity, int64_t slots, int64_t n, cudaStream_t s)
+int grow_pairs(ph_pairs *pr, int64_t capacity, int64_t slots, cudaStream_t s)
 {
     const bool more = capacity > pr->capacity, tasks = slots > pr->task_cap;
     const int64_t cap = pr->capacity, task_cap = pr->task_cap;
@@ -414,7 +424,7 @@ int grow_pairs(ph_pairs *pr, int64_t capacity, int64_t slots, int64_t n, cudaStr
             rc = cuda_check(cudaMemcpyAsync(ecnt.p, pr->ecount.p, (size_t)cap, cudaMemcpyDeviceToDevice, s), "move counts");
     }
     if (!rc && tasks) {
-        rc = ensure_tasks(&t, slots, n);
+        rc = ensure_tasks(&t, slots);
         if (!rc && task_cap > 0)
             rc = cuda_check(cudaMemcpyAsync(t.tasks, pr->tasks, (size_t)task_cap * sizeof(int2), cudaMemcpyDeviceToDevice, s),
                             "move tasks");
@@ -422,8 +432,6 @@ int grow_pairs(ph_pairs *pr, int64_t capacity, int64_t slots, int64_t n, cudaStr
             rc = cuda_check(cudaMemcpyAsync(t.task_done, pr->task_done, (size_t)task_cap * sizeof(int32_t),
                                             cudaMemcpyDeviceToDevice, s),
                             "move task counters");
-        if (!rc && n > 0)
-            rc = cuda_check(cudaMemcpyAsync(t.split_of, pr->split_of, (size_t)n, cudaMemcpyDeviceToDevice, s), "move marks");
     }
     if (!rc) rc = cuda_check(cudaStreamSynchronize(s), "sync after growing");
     if (rc) {
@@ -445,7 +453,6 @@ int grow_pairs(ph_pairs *pr, int64_t capacity, int64_t slots, int64_t n, cudaStr
         pr->tasks = t.tasks;
         pr->task_done = t.task_done;
         pr->task_part = t.task_part;
-        pr->split_of = t.split_of;
         pr->task_cap = t.task_cap;
     }
     return PH_OK;
@@ -453,20 +460,17 @@ int grow_pairs(ph_pairs *pr, int64_t capacity, int64_t slots, int64_t n, cudaStr
 
 // The sizing (with `sizing_sync`: read the total, grow the entry buffers)
 // and the fill pass, on stream s.
-static int fill_pairs(ph_pairs *pr, PairArgs &a, int grid, cudaStream_t s, bool sizing_sync, int64_t n)
+static int fill_pairs(ph_pairs *pr, PairArgs &a, int grid, cudaStream_t s, bool sizing_sync)
 {
     int rc = 0;
     if (sizing_sync) {
-        // tasks written so far, tasks needed, all entries: one read
-        struct {
-            int32_t tasks[2];
-            int64_t total;
-        } need = {{0, 0}, 0};
-        rc = cuda_check(cudaMemcpyAsync(&need, a.n_tasks, sizeof need, cudaMemcpyDeviceToHost, s), "copy pair total");
+        // all entries and the tasks needed: one read
+        TaskCtl need = {};
+        rc = cuda_check(cudaMemcpyAsync(&need, a.ctl, sizeof need, cudaMemcpyDeviceToHost, s), "copy pair total");
         if (!rc) rc = cuda_check(cudaStreamSynchronize(s), "sync pair total");
         if (rc) return rc;
         const int64_t total = need.total;
-        const int32_t nt = need.tasks[1];
+        const int32_t nt = need.needed;
         pr->n_pairs = total;
         if (total > pr->capacity) {
             int64_t cap = total + total / 8 + 1024;
@@ -476,18 +480,16 @@ static int fill_pairs(ph_pairs *pr, PairArgs &a, int grid, cudaStream_t s, bool 
             pr->capacity = cap;
         }
         pr->n_tasks = nt;
-        rc = ensure_tasks(pr, nt > pr->task_cap ? nt + nt / 8 : nt, n);
+        rc = ensure_tasks(pr, nt > pr->task_cap ? nt + nt / 8 : nt);
         if (rc) return rc;
     }
     a.tasks = pr->tasks;
     a.task_done = pr->task_done;
     a.task_cap = pr->task_cap;
-    a.split_of = pr->split_of;
     a.ent = static_cast<float4 *>(pr->entries.p);
     a.ecnt = static_cast<uint8_t *>(pr->ecount.p);
     a.cap = pr->capacity;
     pr->list_cap = pr->capacity;
-    pr->list_task_cap = pr->task_cap;
     launch_chained(!sizing_sync, k_pairs<true>, grid, kThreads, 0, s, a);
     return PH_OK;
 }
@@ -524,7 +526,7 @@ int build_pairs_device(const ph_leaves *lv, ph_pairs *pr, cudaStream_t s, bool s
     const bool ordered =
         lv->queue_order == 0 && !lv->active && pr->group_key.p && pr->group_order.p;
     int32_t *const ot = static_cast<int32_t *>(pr->order_temp.p);
-    a.n_tasks = ot + 2 * kOrdKeys;
+    a.ctl = task_ctl(pr);
     a.chunk_sum = reinterpret_cast<unsigned long long *>(ot + kOrdInts);
     a.segment = lv->segment;
     a.gkey = ordered ? static_cast<uint8_t *>(pr->group_key.p) : nullptr;
@@ -547,9 +549,8 @@ int build_pairs_device(const ph_leaves *lv, ph_pairs *pr, cudaStream_t s, bool s
     // at most one part-filled group a ground cell
     const int64_t most = std::min<int64_t>(n, n / lv->group_size + lv->n_cells);
     launch_chained(true, k_offsets, (int)(most / kOffChunk) + 1, kThreads, 0, s, a.cnt, n_all, a.chunk_sum,
-                   static_cast<int64_t *>(pr->group_off.p), static_cast<unsigned long long *>(pr->work.p),
-                   reinterpret_cast<int64_t *>(a.n_tasks + 2));
-    int rc = fill_pairs(pr, a, grid, s, sizing_sync, n);
+                   static_cast<int64_t *>(pr->group_off.p), static_cast<unsigned long long *>(pr->work.p), a.ctl);
+    int rc = fill_pairs(pr, a, grid, s, sizing_sync);
     if (rc) return rc;
     return cuda_check(cudaGetLastError(), "pair kernels");
 }

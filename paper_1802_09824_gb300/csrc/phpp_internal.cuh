@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include <string>
@@ -241,8 +242,24 @@ size_t order_temp_bytes(int64_t n);
 // segments' sums in order, whichever warps computed them.
 int segment_entries(int64_t n, int leaf_max, int group_size);
 
-// pairs.cu: task slots that a list of `capacity` entries can need at most.
-inline int64_t task_bound(int64_t capacity, int segment) { return 2 * (capacity / segment) + 2; }
+// pairs.cu: task slots for a list of up to `capacity` entries over n particles:
+// what it can need at most, but no more than two a particle (792 B; an entry is
+// 17 B, and lists that need more are cut into longer segments).
+inline int64_t task_bound(int64_t capacity, int segment, int64_t n)
+{
+    return std::min<int64_t>(2 * (capacity / segment) + 2, 2 * n + 1024);
+}
+
+// The tasks of one list (in the pair passes' scratch, order_temp).  A list whose
+// tasks would outnumber its slots is cut into longer segments: what the tasks
+// are, and so the sums, depends on the list and its slots alone.
+struct TaskCtl {
+    int32_t written;   // tasks (fill pass)
+    int32_t segment;   // entries per segment (fill pass)
+    int64_t total;     // entries of all groups (k_offsets)
+    int32_t needed;    // tasks with segments of the length given (count pass)
+    int32_t pad;
+};
 
 // build.cu: scratch of the leaf and group numbering.
 size_t build_temp_bytes();

@@ -97,13 +97,12 @@ struct PPArgs {
     float tab_scale2;                // (kTabN / rcut)^2
     int64_t n_pos;                   // rows of pos_leaf (bounds checks)
     // groups of several segments, one task each (pairs.cu)
-    const int32_t *n_tasks;
-    const int2 *tasks;               // (group, segment); group -1: no task
+    const TaskCtl *ctl;
+    const int2 *tasks;               // (group, segment)
     int32_t *task_done;
     float *task_part;                // [task][3][32]
-    const uint8_t *split_of;
     int64_t task_cap;
-    int segment;                     // entries per segment
+    int segment;                     // entries per segment (direct mode)
     bool inverse;                    // the exact kernel's dense groups take the inverse-distance form (count kernel)
     const int32_t *order;            // queue slot -> group (groups by decreasing cost), or NULL
 };
@@ -556,11 +555,11 @@ struct Round {
 template <int G>
 __device__ __noinline__ void finish_task(const PPArgs &a, int t, int ni, int i0, float Gc, float tx, float ty, float tz)
 {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, segment = a.ctl->segment;
     const int2 tk = a.tasks[t];
     const int first = t - tk.y;
     const int64_t b = a.group_off[tk.x], e = a.group_off[tk.x + 1];
-    const int nseg = (int)(((e < a.cap ? e : a.cap) - b + a.segment - 1) / a.segment);
+    const int nseg = (int)(((e < a.cap ? e : a.cap) - b + segment - 1) / segment);
     if (lane < G && in_bounds(t, a.task_cap, BS_PP_TASK)) {
         float *p = a.task_part + (int64_t)t * 96 + lane;
         __stcg(p, tx);
@@ -741,7 +740,7 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
     extern __shared__ float4 sDyn[];   // dynamic: the factor table (kTable) or layer 1's table (kLearned)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int ng = *a.n_groups;
-    const int nt = *a.n_tasks < a.task_cap ? *a.n_tasks : (int)a.task_cap;
+    const int nt = a.ctl->written, segment = a.ctl->segment;
     unsigned long long inter = 0, staged = 0;
     MlpLane L;
     if (kLearned) {
@@ -779,7 +778,6 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
             const int2 tk = a.tasks[t];
             g = tk.x;
             seg = tk.y;
-            if (g < 0) continue;
         } else {
             g = a.order ? a.order[t - nt] : t - nt;
         }
@@ -788,13 +786,10 @@ __global__ void __launch_bounds__(kPPThreads, kMinBlocks) k_pp(PPArgs a)
         const BoxDev &bx = a.boxes[a.group_box[g]];
         float4 gh = a.group_h4[g];
         if (e1 > a.cap) e1 = a.cap;
-        if (e1 - e0 > a.segment) {
-            if (task) {
-                e0 += (int64_t)seg * a.segment;
-                e1 = e0 + a.segment < e1 ? e0 + a.segment : e1;
-            } else if (a.split_of[g]) {
-                continue;   // its tasks came first
-            }
+        if (e1 - e0 > segment) {
+            if (!task) continue;   // its tasks came first
+            e0 += (int64_t)seg * segment;
+            e1 = e0 + segment < e1 ? e0 + segment : e1;
         }
         constexpr int G = 32 / kSplit;
         const int ti = lane & (G - 1), hs = lane / G;   // target slot, source slot
@@ -1206,12 +1201,11 @@ static void pp_args(const ph_leaves *lv, const ph_pairs *pr, float *d_acc, PPArg
     a.acc = d_acc;
     a.inverse = lv->poly_degree == kInvDeg;
     a.segment = lv->segment;
-    a.n_tasks = pr ? static_cast<const int32_t *>(pr->order_temp.p) + 512 : nullptr;
+    a.ctl = pr ? task_ctl(pr) : nullptr;
     a.tasks = pr ? pr->tasks : nullptr;
     a.task_done = pr ? pr->task_done : nullptr;
     a.task_part = pr ? pr->task_part : nullptr;
-    a.split_of = pr ? pr->split_of : nullptr;
-    a.task_cap = pr ? pr->list_task_cap : 0;
+    a.task_cap = pr ? pr->task_cap : 0;
 }
 
 template <bool kLearned, int kMinBlocks, int kSplit, bool kUniform>

@@ -1,6 +1,8 @@
 """Groups whose source lists span several segments: each segment is a task of
 its own, and the group's sum (segments in order, compensated) does not depend
 on which warps made it."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -78,21 +80,75 @@ def test_split_groups_in_active_mode(gpu_lib):
         B.ph_free(h)
 
 
-def test_noalloc_runs_out_of_task_slots(gpu_lib):
-    # a clustered box whose groups ask for more tasks than the fixed array
-    # holds: the groups left over are summed whole
+def _needed(cnt, segment):
+    """Tasks of lists of cnt entries cut into segments."""
+    cnt = cnt[cnt > segment]
+    return int(np.sum(-(-cnt // segment)))
+
+
+def _entries(n, leaf, gs=32):
+    """Entries per segment (of a box with fewer than 14,592 groups)."""
+    return max(min(max(n // 50, 256), 2000) // leaf, 8)
+
+
+# lists that need more tasks than the no-allocation call has slots for (n / 2),
+# though they fit its entries: cut into longer segments, the same in every call
+# (which groups found slots was left to the order of arrival before)
+@pytest.mark.parametrize("n,rcut,runs_out", [(4096, 0.3, True), (16000, 0.3, True)])
+def test_noalloc_and_its_task_slots(gpu_lib, n, rcut, runs_out):
     import torch
     B = gpu_lib
-    ps = synth.workload("uniform_small", scale=3000)
-    pos = ps.pos.copy()
-    pos[:1500] *= np.float32(0.3)
-    ps = synth.ParticleSet(pos, ps.mass, ps.boxes, ps.offsets, "clump")
+    ps = synth.workload("uniform_small", scale=n)
     bp = ps.boxes[0]
-    prm = B.make_params(bp.L, bp.G, bp.eps, bp.rs, bp.rcut, 4)
-    acc = torch.zeros((ps.n, 3), device="cuda")
-    try:
-        B.ph_accel_noalloc(torch.from_numpy(ps.pos).cuda(), torch.from_numpy(ps.mass).cuda(), prm, acc)
-    except B.PhError as e:
-        assert e.code == B.PH_ERR_CAPACITY      # the documented limit of its list
-        pytest.skip("the list itself does not fit")
-    check_parity(acc.cpu().numpy(), oracle_accel(ps))
+    bp = dataclasses.replace(bp, rcut=rcut, rs=rcut / 4.5)
+    ps = synth.ParticleSet(ps.pos, ps.mass, [bp], ps.offsets, "wide")
+    prm = B.make_params(bp.L, bp.G, bp.eps, bp.rs, bp.rcut, 32)
+    pos, mass = torch.from_numpy(ps.pos).cuda(), torch.from_numpy(ps.mass).cuda()
+    acc = torch.zeros((n, 3), device="cuda")
+    lv, pr = B.ph_accel(pos, mass, prm, B.PH_G_EXACT, None, acc)
+    want, cnt = acc.cpu().numpy().copy(), _lists(B, pr)
+    assert cnt.sum() <= 32 * n
+    assert (_needed(cnt, _entries(n, 32)) > n // 2) == runs_out
+    got = []
+    for _ in range(8):
+        acc.fill_(5.0)
+        B.ph_accel_noalloc(pos, mass, prm, acc)
+        got.append(acc.cpu().numpy())
+    for g in got[1:]:
+        np.testing.assert_array_equal(g, got[0])
+    if runs_out:
+        check_parity(got[0], oracle_accel(ps))
+    else:
+        np.testing.assert_array_equal(got[0], want)
+    for h in (pr, lv):
+        B.ph_free(h)
+
+
+# a captured step whose particles gather: many tasks where the capture saw none
+def test_captured_lists_that_grow_into_segments(gpu_lib):
+    import torch
+    B = gpu_lib
+    n = 4096
+    ps = synth.workload("uniform_small", scale=n)
+    bp = ps.boxes[0]
+    prm = B.make_params(bp.L, bp.G, bp.eps, 0.12 / 4.5, 0.12, 1)
+    pos, mass = torch.from_numpy(ps.pos).cuda(), torch.from_numpy(ps.mass).cuda()
+    lv = B.ph_build_leaves(pos, mass, prm)
+    pr = B.ph_leaf_pairs(lv)
+    assert _needed(_lists(B, pr), 256) == 0
+    acc = torch.zeros((n, 3), device="cuda")
+    g = B.ph_graph_create(lv, pr, pos, mass, B.PH_G_EXACT, None, acc, headroom=6.0)
+    pos[: n // 2] = 0.5 + 0.05 * (pos[: n // 2] - 0.5)
+    got = []
+    for _ in range(8):
+        B.ph_graph_launch(g)
+        got.append(acc.cpu().numpy().copy())
+        acc.fill_(5.0)
+    B.ph_status(pr)
+    for a in got[1:]:
+        np.testing.assert_array_equal(a, got[0])
+    lv1, pr1 = B.ph_accel(pos, mass, prm, B.PH_G_EXACT, None, acc)
+    assert _needed(_lists(B, pr1), 256) > 400          # the capture saw none
+    np.testing.assert_array_equal(acc.cpu().numpy(), got[0])
+    for h in (g, pr, lv, pr1, lv1):
+        B.ph_free(h)
