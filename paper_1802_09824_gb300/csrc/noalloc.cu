@@ -133,13 +133,6 @@ void carve(Carver &c, ph_leaves &lv, ph_pairs &pr, int64_t n, int cells)
     pr.task_part = static_cast<float *>(lv.leaf_ref.p);
 }
 
-// Segment length of the step: segment_entries' of twice as many particles
-// (there are fewer task slots than a list at its capacity could ask for: N / 2).
-int noalloc_segment(int64_t n, int leaf_max)
-{
-    return segment_entries(2 * n, leaf_max, kDefaultGroup);
-}
-
 }  // namespace
 
 extern "C" int ph_accel_noalloc(const float *d_pos, const float *d_mass, int64_t n, const ph_params *params,
@@ -204,7 +197,7 @@ extern "C" int ph_accel_noalloc(const float *d_pos, const float *d_mass, int64_t
     lv.group_size = kDefaultGroup;
     lv.poly_degree = deg;
     lv.max_leaf = p.leaf_max;
-    lv.segment = noalloc_segment(n, p.leaf_max);
+    lv.segment = segment_entries(n, p.leaf_max, kDefaultGroup);
     lv.key_kind = p.key_kind;
     lv.level_bits = p.level_bits ? p.level_bits : 1;
     lv.pp_variant = p.pp_variant == 1 ? 1 : 0;

@@ -93,8 +93,10 @@ def _entries(n, leaf, gs=32):
 
 # lists that need more tasks than the no-allocation call has slots for (n / 2),
 # though they fit its entries: cut into longer segments, the same in every call
-# (which groups found slots was left to the order of arrival before)
-@pytest.mark.parametrize("n,rcut,runs_out", [(4096, 0.3, True), (16000, 0.3, True)])
+# (which groups found slots was left to the order of arrival before); and lists
+# with room, summed as ph_accel sums them
+@pytest.mark.parametrize("n,rcut,runs_out", [(4096, 0.3, True), (16000, 0.3, True), (1000, 0.17, False),
+                                             (12000, 0.17, False)])
 def test_noalloc_and_its_task_slots(gpu_lib, n, rcut, runs_out):
     import torch
     B = gpu_lib
