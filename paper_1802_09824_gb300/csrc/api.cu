@@ -558,6 +558,7 @@ int ph_pairs_reserve(ph_pairs **pairs, int64_t capacity)
     }
     p->capacity = capacity;
     p->fixed_capacity = true;
+    p->slots_due = true;
     *pairs = p;
     return PH_OK;
 }
@@ -597,9 +598,20 @@ int ph_leaf_pairs(ph_leaves *leaves, void *stream, ph_pairs **pairs)
         if (!rc) rc = ensure(p->ecount, 1024);
         if (!rc) p->capacity = 1024;
     }
-    // (a reserved list is not sized: as many slots as it can need)
-    if (!rc && p->fixed_capacity && !p->task_cap)
-        rc = ensure_tasks(p, task_bound(p->capacity, leaves->segment, leaves->n));
+    // a reserved list is not sized: as many slots as it can need, at the first
+    // build after each ph_pairs_reserve (later ones leave the buffers where a
+    // captured step may hold them), unless the caller is capturing
+    if (!rc && p->slots_due) {
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess) {
+            cudaGetLastError();
+            capturing = cudaStreamCaptureStatusActive;
+        }
+        if (capturing == cudaStreamCaptureStatusNone) {
+            rc = ensure_tasks(p, task_bound(p->capacity, leaves->segment, leaves->n));
+            if (!rc) p->slots_due = false;
+        }
+    }
     if (!rc) rc = build_pairs_device(leaves, p, s, !p->fixed_capacity);
     if (rc) {
         if (fresh) {

@@ -80,6 +80,7 @@ struct ph_pairs {
     uint64_t leaves_generation = 0;
     int64_t capacity = 0;        // entries
     bool fixed_capacity = false;
+    bool slots_due = false;      // reserved since the last build: the task slots are still to be made
     int64_t n_pairs = 0;         // host copy (valid after sizing sync)
     int32_t n_groups_cap = 0;
     const ph_leaves *built_from = nullptr;

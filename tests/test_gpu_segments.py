@@ -154,3 +154,25 @@ def test_captured_lists_that_grow_into_segments(gpu_lib):
     np.testing.assert_array_equal(acc.cpu().numpy(), got[0])
     for h in (g, pr, lv, pr1, lv1):
         B.ph_free(h)
+
+
+# a handle reserved for few entries, then for many, and made for other leaves:
+# the list has its tasks' slots each time, so that the sums are the direct mode's
+def test_reserved_lists_get_their_slots_at_every_build(gpu_lib):
+    import torch
+    B = gpu_lib
+    pr = None
+    for n, leaf, capacity in ((300, 32, 2000), (9000, 32, 400_000), (9000, 4, 2_000_000)):
+        ps = synth.workload("uniform_small", scale=n)
+        bp = ps.boxes[0]
+        prm = B.make_params(bp.L, bp.G, bp.eps, bp.rs, bp.rcut, leaf)
+        lv = B.ph_build_leaves(torch.from_numpy(ps.pos).cuda(), torch.from_numpy(ps.mass).cuda(), prm)
+        pr = B.ph_pairs_reserve(capacity, pairs=pr)
+        pr = B.ph_leaf_pairs(lv, pairs=pr)
+        acc, direct = (torch.full((n, 3), 5.0, device="cuda") for _ in range(2))
+        B.ph_pp_accel(lv, pr, B.PH_G_EXACT, None, acc)
+        B.ph_pp_accel(lv, None, B.PH_G_EXACT, None, direct)
+        B.ph_status(pr)
+        assert torch.equal(acc, direct)
+        B.ph_free(lv)
+    B.ph_free(pr)
