@@ -87,8 +87,8 @@ int ph_graph_create(ph_leaves *leaves, ph_pairs *pairs, const void *d_pos, int p
         if (want > pairs->capacity || slots > pairs->task_cap) {
             // the list stays what it was (ph_pp_accel may sum it before the
             // first replay): its buffers move with their contents
-            int rc = cuda_check(cudaStreamSynchronize(caller), "sync before growing");
-            if (!rc) rc = cuda_check(cudaStreamSynchronize(pairs->last_stream), "sync before growing");
+            // (the list may have been made on another stream, gone by now)
+            int rc = cuda_check(cudaDeviceSynchronize(), "sync before growing");
             if (!rc) rc = grow_pairs(pairs, want, slots, caller);
             if (rc) return rc;
         }

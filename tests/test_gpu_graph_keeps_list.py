@@ -90,3 +90,31 @@ def test_a_capture_on_a_reserved_list_that_overflowed(gpu_lib):
     assert B.ph_count_within(lv, pr) == want[4]
     for h in (g, pr, full, lv):
         B.ph_free(h)
+
+
+def test_a_capture_of_a_list_made_on_another_stream(gpu_lib):
+    # the growth waits for a list that another stream is still making, and that
+    # stream need not live on
+    import torch
+    B = gpu_lib
+    ps = synth.workload("uniform_small", scale=50_021)
+    bp = ps.boxes[0]
+    prm = B.make_params(bp.L, bp.G, bp.eps, bp.rs, bp.rcut, 32)
+    pos, mass = torch.from_numpy(ps.pos).cuda(), torch.from_numpy(ps.mass).cuda()
+    torch.cuda.synchronize()
+    lv0, pr0 = B.ph_build_leaves(pos, mass, prm), None
+    pr0 = B.ph_leaf_pairs(lv0)
+    ref = _state(B, lv0, pr0, ps.n)
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    lv = B.ph_build_leaves(pos, mass, prm, stream=a.cuda_stream)
+    pr = B.ph_leaf_pairs(lv, stream=a.cuda_stream)
+    out = torch.full((ps.n, 3), 5.0, device="cuda")
+    torch.cuda.current_stream().synchronize()
+    g = B.ph_graph_create(lv, pr, pos, mass, B.PH_G_EXACT, None, out, headroom=1.0, stream=b.cuda_stream)
+    for x, y in zip(_state(B, lv, pr, ps.n), ref):
+        np.testing.assert_array_equal(x, y)
+    B.ph_graph_launch(g, stream=b.cuda_stream)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(out.cpu().numpy(), ref[0])
+    for h in (g, pr, lv, pr0, lv0):
+        B.ph_free(h)
