@@ -192,7 +192,10 @@ int ph_build_leaves_batched(const void *pos, int pos_type, const float *mass,
  */
 int ph_leaf_pairs(ph_leaves *leaves, void *stream, ph_pairs **pairs);
 
-/* Give a pairs handle a fixed capacity (entries) and stop the sizing sync. */
+/* Give a pairs handle a fixed capacity (entries) and stop the sizing sync.
+ * Memory: 17 bytes an entry, and from the next ph_leaf_pairs on 396 bytes for
+ * each task that a list of that capacity can need (the sums of long lists' segments:
+ * 99 bytes an entry for small boxes, 1 for large ones, at most 792 a particle). */
 int ph_pairs_reserve(ph_pairs **pairs, int64_t capacity);
 
 /*
@@ -203,7 +206,9 @@ int ph_pairs_reserve(ph_pairs **pairs, int64_t capacity);
  *           mode (exact factor only): the PP kernel finds each group's leaf
  *           pairs itself, with the same test and in the same order as
  *           ph_leaf_pairs, so no list is stored and the result is the same
- *           bit for bit.
+ *           bit for bit (but for a list that needs more than two tasks a
+ *           particle in a captured step or a reserved handle: its segments
+ *           are longer, and its sums rounded elsewhere).
  *   g_mode  PH_G_EXACT, PH_G_LEARNED (then mlp and pairs must be non-NULL)
  *           or PH_G_TABLE (pairs must be non-NULL; the table is made on the
  *           host and uploaded at the first call for an rcut / rs).
@@ -234,7 +239,8 @@ int ph_accel(const void *pos, int pos_type, const float *mass, int64_t n,
  *                  for the same particle count and boxes.
  *   d_pos, d_mass, d_acc  device buffers read / written at every replay.
  *   headroom       the pair list gets a fixed capacity of
- *                  (1 + headroom) x its current length (e.g. 0.25).
+ *                  (1 + headroom) x its current length (e.g. 0.25); the list
+ *                  at hand is kept, so ph_pp_accel may sum it before a replay.
  * Replays that would overflow it latch PH_ERR_CAPACITY in ph_status(pairs)
  * (no entry beyond the capacity is written); rebuild the pairs and recreate
  * the graph.  Learned mode with a network that fails its tolerance captures
@@ -559,7 +565,8 @@ int ph_pp_counters(const void *handle, int64_t *interactions, int64_t *staged);
 int ph_leaves_set_active(ph_leaves *leaves, const uint8_t *d_active, int64_t n);
 
 /* Number of ordered pairs (i, j), j != i, with r_ij < rcut in the lists,
- * decided in FP32 exactly as ph_pp_accel decides its cutoff: the work the
+ * decided in FP32 exactly as ph_pp_accel with the exact factor decides its
+ * cutoff (the other factors may differ by pairs within rounding of it): the work the
  * cutoff keeps (the oracle's count up to pairs within rounding of rcut and
  * coincident particles).  Synchronises. */
 int ph_count_within(const ph_leaves *leaves, const ph_pairs *pairs, int64_t *n_within, void *stream);
@@ -673,8 +680,10 @@ int ph_mlp_load(const char *path, float tol, void *stream, ph_mlp **mlp);
  *   params  as for ph_build_leaves, with three limits (else PH_ERR_ARG):
  *           theta must be 0 (every leaf pair by PP), group_size 0 or 32,
  *           and L/rcut must give at most PH_NOALLOC_MAX_CELLS ground cells.
- *           The key depth, factor polynomial and box constants are those
- *           ph_build_leaves derives for the same box.
+ *           The key depth, factor polynomial, box constants and list
+ *           segments are those of ph_accel for the same box, and so is the
+ *           result bit for bit; a list that needs more than n / 2 tasks is
+ *           cut into longer segments (the same result in every call).
  *   d_acc   [n*3] device float32 output, caller order.
  * The call synchronises `stream` once before returning.  PH_ERR_CAPACITY
  * means the leaf-pair list needed more than PH_NOALLOC_PAIRS_PER_PARTICLE

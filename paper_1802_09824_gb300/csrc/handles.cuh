@@ -45,7 +45,7 @@ struct ph_leaves {
     phpp::DevBuf leaf_c4, leaf_h4;        // float4[n] (centre in cell frame, half extents)
     phpp::DevBuf group_ref;      // double[3 n]
     phpp::DevBuf group_c4, group_h4;      // float4[n]
-    phpp::DevBuf leaf_r4, group_r4;       // float4[n]: the reference points in FP32 (exact; see k_boxes)
+    phpp::DevBuf leaf_r4, group_r4;       // float4[n]: the reference points in FP32 (exact; see box_block)
     phpp::DevBuf work;                    // direct-mode PP: group queue and counters (32 B)
     phpp::DevBuf acc_tmp;                 // direct-mode PP into a host buffer: device copy of acc
     phpp::DevBuf table;                   // PH_G_TABLE: float2[4097] factor nodes (value, slope x spacing)

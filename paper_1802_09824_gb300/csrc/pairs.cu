@@ -383,7 +383,8 @@ size_t order_temp_bytes(int64_t n) { return kOrdInts * sizeof(int32_t) + (n / kO
 // most every 32,768 sources.
 int segment_entries(int64_t n, int leaf_max, int group_size)
 {
-    const int64_t warps = 152 * 16;   // resident in the two-block shape
+    const int64_t warps = 152 * 16;   // resident in the two-block shape (one number for all: the segments,
+                                      // and so the sums, depend on neither shape nor device)
     const int64_t most = n / group_size >= 6 * warps ? 32768 : 2000;
     const int64_t sources = std::min<int64_t>(std::max<int64_t>(n / 50, 256), most);
     return (int)std::max<int64_t>(sources / leaf_max, 8);

@@ -10,7 +10,9 @@ from oracle import force
 # tau = 1e-3 median |a_ref|).  The exact path is FP32 with SFU rsqrt/sqrt/ex2
 # (relative error ~2^-22 each), a degree-10 polynomial for the factor
 # (~3e-7) and leaf-relative coordinates (d_ij exact to ~1e-7 of the leaf
-# size); per pair that is a few 1e-7, so 1e-5 at the 99th percentile leaves
+# size); per pair that is a few 1e-7.  Dense groups take the inverse-distance
+# form, whose error is ~1e-7 of a pair's Newtonian term (up to 5e-6 of its weight
+# at the cutoff) and with their many sources below the other form's.  So 1e-5 at the 99th percentile leaves
 # room for the cancellation of many terms, and 1e-3 bounds any single
 # particle (one cutoff-boundary pair classified the other way excepted, which
 # the oracle's near-cutoff sum accounts for).
